@@ -1,5 +1,6 @@
 // lp_api.cu -- the C ABI of liblp.so (include/lp.h): context management,
 // argument checks, and the order of the phases of one LP step (Sec. 2.2).
+#include <math.h>
 #include <stdio.h>
 #include <stdlib.h>
 #include <string.h>
@@ -419,6 +420,9 @@ lp_status lp_create(const lp_config* cfg, lp_ctx** out)
         d.Lper[k] = cfg->box_hi[k] - cfg->box_lo[k];
         d.Lper_h[k] = (float)d.Lper[k];
         d.Lper_l[k] = (float)(d.Lper[k] - (double)d.Lper_h[k]);
+        // (see side_of_split: offsets are told apart in floats while the box is near the origin)
+        const bool near = fabs(d.box_lo[k]) <= 0x1p20 * d.Lper[k] && fabs(d.box_hi[k]) <= 0x1p20 * d.Lper[k];
+        d.side_near[k] = near ? 0.25f * d.Lper_h[k] : -1.0f;
     }
     d.n_fluid = cfg->n_fluid;
     c->cap = cfg->capacity;

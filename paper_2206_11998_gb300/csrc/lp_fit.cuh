@@ -428,12 +428,8 @@ struct Src<float, DIM, F> {
     // record of j already loaded
     __device__ int side_rec(const float (&r)[4 * REC_F4], uint32_t j, int k) const
     {
-        if (!a.c.periodic[k]) {
-            float hj = r[REC_XH + k], hi = ri[REC_XH + k];
-            if (hj != hi) return hj > hi ? 1 : -1;
-            float lj = r[REC_XL + k], li = ri[REC_XL + k];
-            if (lj != li) return lj > li ? 1 : -1;
-        }
+        const int sg = side_split(a.c, k, ri[REC_XH + k], ri[REC_XL + k], r[REC_XH + k], r[REC_XL + k]);
+        if (sg != SIDE_FP64) return sg;
         double d = offset64(a.c, k, a.sx[k][i], a.sx[k][j]);
         return d > 0.0 ? 1 : (d < 0.0 ? -1 : 0);
     }

@@ -12,7 +12,8 @@
 // ones the plain form gives; the host test (tests/test_split_host.py) checks
 // that bit for bit against the compiler's conversions.
 //
-// Also the floor of an FP64 value as an integer, from its bits (floor_clamped).
+// Also the floor of an FP64 value as an integer, from its bits (floor_clamped),
+// and which side of another a split value lies on (side_of_split).
 //
 // Plain C++ so that the host test compiles it as well.
 #pragma once
@@ -135,6 +136,33 @@ LP_SPLIT_FN bool round_exact(double x, float& h)
 {
     float l;
     return split_exact(x, h, l);
+}
+
+// Sign (-1 or 1) of x_j - x_i, on a periodic axis of its minimum image, from
+// the split parts of both values (h = RN(x), l = RN(x - h)); SIDE_FP64 where
+// the FP64 values have to decide.  Both roundings are monotonic, so the first
+// part that differs orders the two values exactly.  On a periodic axis of
+// length L (near = L / 4) the minimum image leaves an offset below L / 4 as it
+// is, and turns one between 3 L / 4 and 0.9999 L to the other side; d, the
+// offset in floats, is within 2^-20 L of it while the box lies within 2^20 L
+// of the origin (near < 0 otherwise: FP64 decides), far inside those margins.
+// Around L / 2, where the image changes, and around L, FP64 decides.
+constexpr int SIDE_FP64 = 2;
+LP_SPLIT_FN int side_of_split(bool periodic, float near, float hi, float li, float hj, float lj)
+{
+    bool flip = false;
+    if (periodic) {
+        const float o = (hj - hi) + (lj - li), d = o < 0.0f ? -o : o;
+        if (!(d < near)) {
+            if (!(near > 0.0f && d > 3.0f * near && d < 3.9996f * near)) return SIDE_FP64;
+            flip = true;
+        }
+    }
+    bool gt;
+    if (hj != hi) gt = hj > hi;
+    else if (lj != li) gt = lj > li;
+    else return SIDE_FP64;
+    return gt != flip ? 1 : -1;
 }
 
 }  // namespace lp
