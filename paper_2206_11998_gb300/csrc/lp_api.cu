@@ -339,7 +339,7 @@ lp_status run_fit(lp_ctx* c, FitArgs a, const StepOut& o, int sched, cudaStream_
         }
         a.list = c->redo_list;
         Phase ph(c, LP_PH_FIT64, 1, s);
-        LP_CUDA(launch_step_f64(dim, a, o, s));
+        LP_CUDA(launch_step_redo(dim, a, o, s));
     } else {
         Phase ph(c, LP_PH_FIT64, split ? 2 : 1, s);
         LP_CUDA(split ? launch_step_split_f64(dim, a, o, s) : launch_step_f64(dim, a, o, s));
@@ -631,7 +631,7 @@ lp_status lp_gfd_derivs(lp_ctx* c, const lp_particles* p, const double* const* f
             }
             a.list = c->redo_list;
             Phase ph(c, LP_PH_FIT64, 1, s);
-            LP_CUDA(launch_derivs_f64(dim, F, a, o, s));
+            LP_CUDA(launch_derivs_redo(dim, F, a, o, s));
         } else {
             Phase ph(c, LP_PH_FIT64, 1, s);
             LP_CUDA(launch_derivs_f64(dim, F, a, o, s));
@@ -670,7 +670,7 @@ lp_status lp_onesided_derivs(lp_ctx* c, const lp_particles* p, const double* con
         }
         a.list = c->redo_list;
         Phase ph(c, LP_PH_FIT64, 1, s);
-        LP_CUDA(launch_onesided_f64(dim, a, derivs, nfields, s));
+        LP_CUDA(launch_onesided_redo(dim, a, derivs, nfields, s));
     } else {
         Phase ph(c, LP_PH_FIT64, 1, s);
         LP_CUDA(launch_onesided_f64(dim, a, derivs, nfields, s));

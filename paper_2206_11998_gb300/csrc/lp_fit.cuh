@@ -345,7 +345,7 @@ struct FitArgs {
     const double* sm;
     unsigned long long* counters;
     uint32_t* redo_list;      // FP32 pass: particles to redo in FP64
-    const uint32_t* list;     // FP64 pass over a list (null: all particles)
+    const uint32_t* list;     // FP64 redo: the particles of the list
     const unsigned long long* list_len;
     const __nv_bfloat16* mlp_w;   // learned-estimator weights (BF16)
     const uint64_t* keys;         // key-sorted keys (simulation above bit key_shift)

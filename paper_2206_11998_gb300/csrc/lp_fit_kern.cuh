@@ -149,6 +149,47 @@ __device__ __forceinline__ bool step_load(const FitArgs& a, const StepOut& o, in
     return true;
 }
 
+// learned estimator: true where the particle is unflagged and its one-sided
+// fits are skipped, its probability below mlp_tau_lo (unless auditing against
+// the plain estimator)
+template <typename T, int DIM, bool GATE>
+__device__ __forceinline__ bool central_gate(const FitArgs& a, const StepOut& o, int64_t i, const Loaded<DIM>& L,
+                                             const T (&cd)[NU<DIM>::v][DIM + 2], const FitStats<T>& fst)
+{
+    constexpr int F = DIM + 2;
+    const DevCfg& c = a.c;
+    bool mlp_skip = false;
+    if (GATE && (o.features || c.estimator == LP_EST_MLP)) {
+        float xf[MLP_IN];
+        mlp_features<T, DIM>(cd, fst, (T)sqrt(a.d2min[i]), (T)L.s0[0], (T)L.s0[F - 1], (T)c.gamma, xf);
+        if (o.features)
+#pragma unroll
+            for (int k = 0; k < MLP_IN; ++k) o.features[i * MLP_IN + k] = xf[k];
+        if (c.estimator == LP_EST_MLP) {
+            const float pg = mlp_prob(xf, a.mlp_w);
+            if (o.gate_p) o.gate_p[i] = pg;
+            mlp_skip = pg < c.mlp_tau_lo;
+            warp_count(a.counters, C_MLP_SKIP, mlp_skip);
+            warp_count(a.counters, C_MLP_UNCERTAIN, !mlp_skip);
+        }
+    }
+    return mlp_skip;
+}
+
+// Lax-Wendroff rates, and the first derivatives the later stages need
+template <typename T, int DIM>
+__device__ __forceinline__ void central_rates(const FitArgs& a, const Loaded<DIM>& L,
+                                              const T (&cd)[NU<DIM>::v][DIM + 2], T (&cdf)[DIM][DIM + 2],
+                                              T (&lw)[DIM + 2])
+{
+    constexpr int F = DIM + 2;
+    lw_rates<T, DIM>((T)a.c.gamma, (T)L.dt, (T)L.s0[0], (T)L.s0[F - 1], cd, lw);
+#pragma unroll
+    for (int k = 0; k < DIM; ++k)
+#pragma unroll
+        for (int f = 0; f < F; ++f) cdf[k][f] = cd[k][f];
+}
+
 // central stage; false when i went to the FP64 redo list (or, DEFER, to the
 // correction kernel's list).  GATE: the learned estimator or the feature
 // output is in use (its inputs and code are compiled out otherwise)
@@ -188,28 +229,8 @@ __device__ inline bool step_central(const FitArgs& a, const StepOut& o, int64_t 
             atomicAdd(a.counters + C_NOFIT, 1ull);
         }
     }
-    // learned estimator: below mlp_tau_lo the particle is unflagged and its
-    // one-sided fits are skipped (unless auditing against the plain estimator)
-    mlp_skip = false;
-    if (GATE && (o.features || c.estimator == LP_EST_MLP)) {
-        float xf[MLP_IN];
-        mlp_features<T, DIM>(cd, fst, (T)sqrt(a.d2min[i]), (T)L.s0[0], (T)L.s0[F - 1], (T)c.gamma, xf);
-        if (o.features)
-#pragma unroll
-            for (int k = 0; k < MLP_IN; ++k) o.features[i * MLP_IN + k] = xf[k];
-        if (c.estimator == LP_EST_MLP) {
-            const float pg = mlp_prob(xf, a.mlp_w);
-            if (o.gate_p) o.gate_p[i] = pg;
-            mlp_skip = pg < c.mlp_tau_lo;
-            warp_count(a.counters, C_MLP_SKIP, mlp_skip);
-            warp_count(a.counters, C_MLP_UNCERTAIN, !mlp_skip);
-        }
-    }
-    lw_rates<T, DIM>((T)c.gamma, (T)L.dt, (T)L.s0[0], (T)L.s0[F - 1], cd, lw);
-#pragma unroll
-    for (int k = 0; k < DIM; ++k)
-#pragma unroll
-        for (int f = 0; f < F; ++f) cdf[k][f] = cd[k][f];
+    mlp_skip = central_gate<T, DIM, GATE>(a, o, i, L, cd, fst);
+    central_rates<T, DIM>(a, L, cd, cdf, lw);
     return true;
 }
 
@@ -235,72 +256,55 @@ __device__ __forceinline__ bool step_plain(const FitArgs& a, int64_t i, const Sr
     return true;
 }
 
+// upwind rates, the 1D operator along each axis (the axis-sum reading)
 template <typename T, int DIM>
-__device__ __forceinline__ void step_finish(const FitArgs& a, const StepOut& o, int64_t i, const Loaded<DIM>& L,
-                                   const T (&os)[DIM][2][DIM + 2], const T (&lw)[DIM + 2], bool plain, bool mlp_skip)
+__device__ __forceinline__ void upwind_rates(T g, T V, T P, const T (&os)[DIM][2][DIM + 2], T (&uw)[DIM + 2])
+{
+    constexpr int F = DIM + 2;
+    using O = RN<T>;
+    const T K = O::div(O::mul(g, P), V);
+    const T sK = sqrt(K);
+    const T hV = O::mul(T(0.5), V);
+    const T hVsK = O::mul(hV, sK);
+    const T hVK = O::mul(hV, K);
+    const T VsK2 = O::div(V, O::mul(T(2), sK));
+    T Vt = T(0), Pt = T(0);
+#pragma unroll
+    for (int k = 0; k < DIM; ++k) {
+        T ul = os[k][0][1 + k], ur = os[k][1][1 + k];
+        T Pl = os[k][0][F - 1], Pr = os[k][1][F - 1];
+        T su = O::add(ur, ul), du = O::sub(ur, ul), sP = O::add(Pr, Pl), dP = O::sub(Pr, Pl);
+        Vt = O::add(Vt, O::sub(O::mul(hV, su), O::mul(VsK2, dP)));
+        uw[1 + k] = O::sub(O::mul(hVsK, du), O::mul(hV, sP));
+        Pt = O::add(Pt, O::sub(O::mul(hVsK, dP), O::mul(hVK, su)));
+    }
+    uw[0] = Vt;
+    uw[F - 1] = Pt;
+}
+
+// limiter value p and new value of one field from its rates
+template <typename T>
+__device__ __forceinline__ double blend_field(const DevCfg& c, double dt, double s0, T uw, T lw, T rs, bool any, T& p)
+{
+    using O = RN<T>;
+    switch (c.limiter) {
+    case LP_LIM_PAPER: p = phi_limiter<T>(rs); break;
+    case LP_LIM_LW: p = T(1); break;
+    case LP_LIM_UW: p = T(0); break;
+    default: p = any ? phi_limiter<T>(rs) : T(1); break;
+    }
+    const T rate = O::sub(uw, O::mul(p, O::sub(uw, lw)));
+    return __dadd_rn(s0, __dmul_rn(dt, (double)rate));   // no contraction: the oracle's rounding
+}
+
+// the safeguard, the mover and the outputs of particle i
+template <int DIM>
+__device__ __forceinline__ void store_state(const FitArgs& a, const StepOut& o, int64_t i, const Loaded<DIM>& L,
+                                            double (&s1)[DIM + 2], bool any)
 {
     constexpr int F = DIM + 2;
     const DevCfg& c = a.c;
     const double dt = L.dt;
-    using O = RN<T>;
-    const T g = (T)c.gamma;
-    const T V = (T)L.s0[0], P = (T)L.s0[F - 1];
-    T uw[F];
-    {
-        // upwind rates, the 1D operator along each axis (the axis-sum reading)
-        const T K = O::div(O::mul(g, P), V);
-        const T sK = sqrt(K);
-        const T hV = O::mul(T(0.5), V);
-        const T hVsK = O::mul(hV, sK);
-        const T hVK = O::mul(hV, K);
-        const T VsK2 = O::div(V, O::mul(T(2), sK));
-        T Vt = T(0), Pt = T(0);
-#pragma unroll
-        for (int k = 0; k < DIM; ++k) {
-            T ul = os[k][0][1 + k], ur = os[k][1][1 + k];
-            T Pl = os[k][0][F - 1], Pr = os[k][1][F - 1];
-            T su = O::add(ur, ul), du = O::sub(ur, ul), sP = O::add(Pr, Pl), dP = O::sub(Pr, Pl);
-            Vt = O::add(Vt, O::sub(O::mul(hV, su), O::mul(VsK2, dP)));
-            uw[1 + k] = O::sub(O::mul(hVsK, du), O::mul(hV, sP));
-            Pt = O::add(Pt, O::sub(O::mul(hVsK, dP), O::mul(hVK, su)));
-        }
-        uw[0] = Vt;
-        uw[F - 1] = Pt;
-    }
-    // estimator
-    const T ell = (T)sqrt(a.d2min[i]);
-    T rs[F];
-    bool any = false;
-#pragma unroll
-    for (int f = 0; f < F; ++f) {
-        T sl[DIM], sr[DIM];
-#pragma unroll
-        for (int k = 0; k < DIM; ++k) { sl[k] = os[k][0][f]; sr[k] = os[k][1][f]; }
-        rs[f] = plain ? estimator_r<T, DIM>(sl, sr, ell, (T)L.s0[f], (T)c.s_ref[f], (T)c.flat_eps, (T)c.active_frac)
-                      : T(1);
-        any = any || rs[f] > T(1.5);
-    }
-    warp_count(a.counters, C_MLP_MISS, mlp_skip && any);
-    if (mlp_skip) {               // the learned call stands; the audit counts misses
-        any = false;
-#pragma unroll
-        for (int f = 0; f < F; ++f) rs[f] = T(1);
-    }
-    double s1[F];
-#pragma unroll
-    for (int f = 0; f < F; ++f) {
-        T p;
-        switch (c.limiter) {
-        case LP_LIM_PAPER: p = phi_limiter<T>(rs[f]); break;
-        case LP_LIM_LW: p = T(1); break;
-        case LP_LIM_UW: p = T(0); break;
-        default: p = any ? phi_limiter<T>(rs[f]) : T(1); break;
-        }
-        T rate = O::sub(uw[f], O::mul(p, O::sub(uw[f], lw[f])));
-        s1[f] = __dadd_rn(L.s0[f], __dmul_rn(dt, (double)rate));   // no contraction: the oracle's rounding
-        if (o.phi) o.phi[i * F + f] = (float)p;
-        if (o.r) o.r[i * F + f] = (float)rs[f];
-    }
     // safeguard: an update that leaves V or P non-positive or any field non-finite
     // is not applied; the particle keeps its state and is counted
     bool admissible = s1[0] > 0.0 && s1[F - 1] > 0.0;
@@ -328,6 +332,44 @@ __device__ __forceinline__ void step_finish(const FitArgs& a, const StepOut& o, 
     o.m[i] = a.sm[i];
     o.id[i] = L.id;
     if (o.flag) o.flag[i] = any ? 1 : 0;
+}
+
+template <typename T, int DIM>
+__device__ __forceinline__ void step_finish(const FitArgs& a, const StepOut& o, int64_t i, const Loaded<DIM>& L,
+                                   const T (&os)[DIM][2][DIM + 2], const T (&lw)[DIM + 2], bool plain, bool mlp_skip)
+{
+    constexpr int F = DIM + 2;
+    const DevCfg& c = a.c;
+    T uw[F];
+    upwind_rates<T, DIM>((T)c.gamma, (T)L.s0[0], (T)L.s0[F - 1], os, uw);
+    // estimator
+    const T ell = (T)sqrt(a.d2min[i]);
+    T rs[F];
+    bool any = false;
+#pragma unroll
+    for (int f = 0; f < F; ++f) {
+        T sl[DIM], sr[DIM];
+#pragma unroll
+        for (int k = 0; k < DIM; ++k) { sl[k] = os[k][0][f]; sr[k] = os[k][1][f]; }
+        rs[f] = plain ? estimator_r<T, DIM>(sl, sr, ell, (T)L.s0[f], (T)c.s_ref[f], (T)c.flat_eps, (T)c.active_frac)
+                      : T(1);
+        any = any || rs[f] > T(1.5);
+    }
+    warp_count(a.counters, C_MLP_MISS, mlp_skip && any);
+    if (mlp_skip) {               // the learned call stands; the audit counts misses
+        any = false;
+#pragma unroll
+        for (int f = 0; f < F; ++f) rs[f] = T(1);
+    }
+    double s1[F];
+#pragma unroll
+    for (int f = 0; f < F; ++f) {
+        T p;
+        s1[f] = blend_field<T>(c, L.dt, L.s0[f], uw[f], lw[f], rs[f], any, p);
+        if (o.phi) o.phi[i * F + f] = (float)p;
+        if (o.r) o.r[i * F + f] = (float)rs[f];
+    }
+    store_state<DIM>(a, o, i, L, s1, any);
     warp_count(a.counters, C_FLAGGED, any);
 }
 
@@ -369,15 +411,8 @@ __device__ void step_one(const FitArgs& a, const StepOut& o, int64_t i)
 template <typename T, int DIM, bool GATE>
 __global__ void __launch_bounds__(FIT_THREADS, FitOcc<T>::fused) k_step(FitArgs a, StepOut o)
 {
-    if (a.list) {
-        unsigned long long len = *a.list_len;
-        for (unsigned long long t = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; t < len;
-             t += (unsigned long long)gridDim.x * blockDim.x)
-            step_one<T, DIM, GATE>(a, o, a.list[t]);
-    } else {
-        int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-        if (i < a.n) step_one<T, DIM, GATE>(a, o, i);
-    }
+    int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (i < a.n) step_one<T, DIM, GATE>(a, o, i);
 }
 
 // intermediate record of the split schedule, component-major over list slots:
@@ -640,15 +675,8 @@ __device__ void derivs_one(const FitArgs& a, const DerivOut& o, int64_t i)
 template <typename T, int DIM, int F>
 __global__ void __launch_bounds__(FIT_THREADS) k_derivs(FitArgs a, DerivOut o)
 {
-    if (a.list) {
-        unsigned long long len = *a.list_len;
-        for (unsigned long long t = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; t < len;
-             t += (unsigned long long)gridDim.x * blockDim.x)
-            derivs_one<T, DIM, F>(a, o, a.list[t]);
-    } else {
-        int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-        if (i < a.n) derivs_one<T, DIM, F>(a, o, i);
-    }
+    int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (i < a.n) derivs_one<T, DIM, F>(a, o, i);
 }
 
 // ---------------------------------------------------------------------------
@@ -705,15 +733,8 @@ __device__ void onesided_one(const FitArgs& a, double* out, int f_real, int64_t 
 template <typename T, int DIM, int F>
 __global__ void __launch_bounds__(FIT_THREADS) k_onesided(FitArgs a, double* out, int f_real)
 {
-    if (a.list) {
-        unsigned long long len = *a.list_len;
-        for (unsigned long long t = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; t < len;
-             t += (unsigned long long)gridDim.x * blockDim.x)
-            onesided_one<T, DIM, F>(a, out, f_real, a.list[t]);
-    } else {
-        int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-        if (i < a.n) onesided_one<T, DIM, F>(a, out, f_real, i);
-    }
+    int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (i < a.n) onesided_one<T, DIM, F>(a, out, f_real, i);
 }
 
 // launchers, defined once per precision in lp_fit_f32.cu / lp_fit_f64.cu
@@ -725,6 +746,11 @@ cudaError_t launch_derivs_f32(int dim, int F, const FitArgs& a, const DerivOut& 
 cudaError_t launch_derivs_f64(int dim, int F, const FitArgs& a, const DerivOut& o, cudaStream_t s);
 cudaError_t launch_onesided_f32(int dim, const FitArgs& a, double* out, int f_real, cudaStream_t s);
 cudaError_t launch_onesided_f64(int dim, const FitArgs& a, double* out, int f_real, cudaStream_t s);
+// the FP64 redo of the particles a.list (a.list_len of them, on the device) that
+// an FP32 pass listed (lp_fit_f64_redo.cu)
+cudaError_t launch_step_redo(int dim, const FitArgs& a, const StepOut& o, cudaStream_t s);
+cudaError_t launch_derivs_redo(int dim, int F, const FitArgs& a, const DerivOut& o, cudaStream_t s);
+cudaError_t launch_onesided_redo(int dim, const FitArgs& a, double* out, int f_real, cudaStream_t s);
 
 // k_step_central_refine over the deferred list (FP32; its own translation
 // unit, lp_fit_f32_refine.cu, so that its instantiation does not change how the
@@ -755,7 +781,7 @@ inline bool split_defers_t(const FitArgs& a)
 
 inline unsigned fit_blocks(const FitArgs& a)
 {
-    return a.list ? 152u * 4u : (unsigned)((a.n + FIT_THREADS - 1) / FIT_THREADS);
+    return (unsigned)((a.n + FIT_THREADS - 1) / FIT_THREADS);
 }
 
 #define LP_DEFINE_FIT_LAUNCHERS(T, SUF)                                                         \
