@@ -458,7 +458,6 @@ lp_status lp_create(const lp_config* cfg, lp_ctx** out)
         A(cudaMemset(c->dt_dev, 0, 8 * ns));
         A(cudaMemcpy(c->level_off_dev, c->level_off, sizeof(int64_t) * (MAX_LEVELS + 1), cudaMemcpyHostToDevice));
         for (int q = 0; q < 2 * EV_PAIRS && ok; ++q) A(cudaEventCreate(&c->ev[q]));
-        A(query_init());
         A(cudaDeviceSynchronize());
     }
     if (!ok) {

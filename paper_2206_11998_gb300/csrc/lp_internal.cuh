@@ -40,8 +40,8 @@ constexpr uint32_t FIT_LINEAR = 1u, FIT_NONE = 2u, FIT_FP64 = 8u;
 // device counters (unsigned long long each)
 enum Counter {
     C_FLAGGED = 0, C_FP64, C_LINEAR, C_NOFIT, C_OVERFLOW, C_NONFINITE, C_MLP_UNCERTAIN,
-    C_MAXCOUNT, C_STATUS, C_REDO_LEN, C_STEPS, C_MLP_SKIP, C_MLP_MISS, C_PLAIN_LEN, C_QFB_LEN, C_REFINED,
-    C_REFINE_LEN, C_QUEUE_TILE, C_QUEUE_CENTRAL, C_QUEUE_PLAIN, C_OCT_GAP, C_COUNT
+    C_MAXCOUNT, C_STATUS, C_REDO_LEN, C_STEPS, C_MLP_SKIP, C_MLP_MISS, C_PLAIN_LEN, C_QFB_LEN, C_GROUP_LEN,
+    C_REFINED, C_REFINE_LEN, C_QUEUE_TILE, C_QUEUE_CENTRAL, C_QUEUE_PLAIN, C_OCT_GAP, C_COUNT
 };
 
 // method constants as the kernels see them
@@ -356,7 +356,6 @@ cudaError_t gather_geometry(lp_ctx* c, const lp_particles* p, cudaStream_t s);
 cudaError_t gather_fields(lp_ctx* c, const lp_particles* p, cudaStream_t s);
 cudaError_t fill_tables(lp_ctx* c, int64_t n, bool clear, cudaStream_t s);
 cudaError_t query_neighbors(lp_ctx* c, int64_t n, cudaStream_t s);
-cudaError_t query_init();   // once per context: kernel attributes
 int query_launches(const lp_ctx* c);   // kernels one query launches
 cudaError_t scatter_back(lp_ctx* c, lp_particles* p, cudaStream_t s);
 cudaError_t split_fields(lp_ctx* c, int64_t n, const double* const* f, int nf, cudaStream_t s);

@@ -40,9 +40,12 @@ struct QueryArgs {
     // the per-particle kernel runs over this list (null: every particle)
     const uint32_t* list;
     const unsigned long long* list_len;
-    // the tile kernel appends the particles it leaves here
+    // the tile kernels append the particles they leave here
     uint32_t* fb_list;
     unsigned long long* fb_len;
+    // and the first of them the parts of the groups it found too large: tile << 32 | lanes
+    unsigned long long* gr_list;
+    unsigned long long* gr_len;
     // the persistent tile kernel's work counter (zero at launch)
     unsigned long long* queue;
 };
@@ -96,6 +99,11 @@ __device__ inline void unpack_cell(unsigned long long e, int& l, int (&w)[3], in
     }
 }
 
+// Entries of buf[0..m), sorted by their float d2, re-ordered by (exact d2, id)
+// where neighbouring float distances are within rounding.
+template <int DIM>
+__device__ void order_ties(const QueryArgs& a, WarpBuf& b, int m, int64_t i);
+
 // Sort buf[0..m) by (d2, id) exactly; returns nothing, buffer sorted in place.
 template <int DIM>
 __device__ void sort_exact(const QueryArgs& a, WarpBuf& b, int m, int64_t i)
@@ -121,10 +129,17 @@ __device__ void sort_exact(const QueryArgs& a, WarpBuf& b, int m, int64_t i)
             __syncwarp();
         }
     }
+    order_ties<DIM>(a, b, m, i);
+}
+
+template <int DIM>
+__device__ void order_ties(const QueryArgs& a, WarpBuf& b, int m, int64_t i)
+{
+    unsigned lane = lane_id();
     // entries whose float distances are within rounding of a neighbour's; the
     // runs are fixed here, before any entry moves
     bool any = false;
-    for (int e0 = 0; e0 < P; e0 += 32) {
+    for (int e0 = 0; e0 < m; e0 += 32) {
         int e = e0 + (int)lane;
         bool tp = false, tn = false;
         if (e < m) {
@@ -188,10 +203,11 @@ struct QueryStart {
     uint64_t sim;
 };
 
-template <int DIM>
+template <int DIM, int THREADS = 32>
 __device__ __forceinline__ void query_start(const QueryArgs& a, WarpBuf& b, int64_t i, QueryStart& st)
 {
-    unsigned lane = lane_id();
+    // (THREADS: a warp, or a block whose threads share the cells; b is per warp or per block)
+    unsigned lane = THREADS == 32 ? lane_id() : threadIdx.x;
     const DevCfg& c = a.c;
     const int mb = c.mbits;
     const uint64_t sim = c.nsim_max > 1 ? (a.keys[i] >> (DIM * mb)) : 0ull;
@@ -249,16 +265,17 @@ __device__ __forceinline__ void query_start(const QueryArgs& a, WarpBuf& b, int6
         if (lane == 0) atomicOr(reinterpret_cast<unsigned int*>(a.counters + C_STATUS), ST_ILLCOND);
         ncells = FCAP;
     }
-    for (int t = lane; t < ncells; t += 32) {
-        int u = t;
+    for (int t = lane; t < ncells; t += THREADS) {
+        unsigned u = (unsigned)t;
         int wv[3] = {0, 0, 0}, shv[3] = {0, 0, 0};
 #pragma unroll
         for (int k = 0; k < DIM; ++k) {
-            long long v = clo[k] + (u % nc[k]);     // unwrapped (periodic axes: within one period)
-            u /= nc[k];
-            long long wr = ((v % ncell_axis) + ncell_axis) % ncell_axis;
+            const unsigned nk = (unsigned)nc[k], d = u / nk;
+            const long long v = clo[k] + (long long)(u - d * nk);   // unwrapped (periodic axes: within one period)
+            u = d;
+            const long long wr = v & (ncell_axis - 1);              // ncell_axis = 2^l0
             wv[k] = (int)wr;
-            shv[k] = (int)((v - wr) / ncell_axis);
+            shv[k] = (int)((v - wr) >> l0);
         }
         b.front[0][t] = pack_cell(l0, wv, shv);
     }
@@ -826,21 +843,270 @@ __device__ void query_one_octant(const QueryArgs& a, WarpBuf& b, int64_t i)
     __syncwarp();
 }
 
-// warp per particle: every particle, or the particles of a list
+// every particle, a warp each
 template <int DIM>
 __global__ void __launch_bounds__(NB_WARPS * 32) k_query(QueryArgs a)
 {
     __shared__ WarpBuf bufs[NB_WARPS];
     const int w = threadIdx.x >> 5;
-    WarpBuf& b = bufs[w];
-    if (a.list) {
-        const unsigned long long len = *a.list_len;
-        for (unsigned long long t = (unsigned long long)blockIdx.x * NB_WARPS + w; t < len;
-             t += (unsigned long long)gridDim.x * NB_WARPS)
-            query_one<DIM>(a, b, (int64_t)a.list[t]);
-    } else {
-        const int64_t i = (int64_t)blockIdx.x * NB_WARPS + w;
-        if (i < a.n) query_one<DIM>(a, b, i);
+    const int64_t i = (int64_t)blockIdx.x * NB_WARPS + w;
+    if (i < a.n) query_one<DIM>(a, bufs[w], i);
+}
+
+// The particles the tiles left, a block each.  They are few (0.3 % of the 2M
+// cloud, 5 % of a cloud of 20k), most with some ten neighbours more than a
+// tile's column holds, some with hundreds among thousands of candidates, so the
+// chain of one particle's work sets the time: by a warp (query_one) it took 100
+// us, two thirds of it in the sort of 64-bit keys in shared memory.  Here the
+// 128 threads of a block test the candidates of all start cells, four each in
+// flight, keep every hit in shared memory, leave out the hits beyond the
+// histogram bin of d2 that holds the NB_CAP-th, and give each of the others its
+// place by counting those that sort before it; the NB_CAP nearest are kept.
+// Particles with more candidates or hits than QL_CAND, QL_HITS, and lists whose
+// last entries tie past the buffer, go through query_one (which prunes by the
+// k_max-th distance) on the first warp.
+constexpr int QL_THREADS = 128;
+constexpr int QL_HITS = 1024;
+constexpr uint32_t QL_CAND = 32768;
+constexpr int QL_LOADS = 4;           // candidates a thread has in flight
+constexpr int QL_BINS = 256;
+static_assert(QL_BINS == 2 * QL_THREADS, "two bins a thread");
+static_assert(FCAP == 2 * QL_THREADS && NB_CAP == QL_THREADS, "two start cells and one kept hit a thread");
+struct LeftBuf {
+    WarpBuf w;
+    alignas(16) unsigned long long key[QL_HITS + 2];  // float bits of d2 << 32 | id
+    uint32_t j[QL_HITS];
+    uint32_t cstart[FCAP], cexcl[FCAP];
+    uint32_t wsum[QL_THREADS / 32];
+    uint32_t hits, near, last_bin;
+    uint32_t hist[QL_BINS];           // hits by d2 / R2
+};
+
+template <int DIM>
+__device__ void query_left(const QueryArgs& a, LeftBuf& b, int64_t i)
+{
+    const unsigned lane = lane_id();
+    const int tid = (int)threadIdx.x, wid = tid >> 5;
+    const DevCfg& c = a.c;
+    const int mb = c.mbits;
+    QueryStart st;
+    query_start<DIM, QL_THREADS>(a, b.w, i, st);
+    if (tid == 0) { b.hits = 0; b.near = 0; }
+    b.hist[tid] = 0;
+    b.hist[tid + QL_THREADS] = 0;
+    __syncthreads();
+    const float bin_scale = st.R2f > 0.0f ? (float)QL_BINS / st.R2f : 0.0f;
+    auto bin_of = [&](float d2f) { return min(QL_BINS - 1, (int)(d2f * bin_scale)); };   // (monotonic in d2f)
+    // the particles of the start cells within reach, two cells a thread
+    uint32_t cs[2] = {0, 0}, cn[2] = {0, 0};
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int e = 2 * tid + h;
+        if (e >= st.ncells) continue;
+        int l, wv[3], shv[3];
+        unpack_cell(b.w.front[0][e], l, wv, shv);
+        uint32_t q[3] = {0, 0, 0};
+        const float size = ldexpf(1.0f, mb - l), period = ldexpf(1.0f, mb);
+        float dmin2 = 0.0f;
+#pragma unroll
+        for (int k = 0; k < DIM; ++k) {
+            q[k] = (uint32_t)wv[k];
+            const float lo = (float)wv[k] * size + (float)shv[k] * period;
+            const float dn = fmaxf(0.0f, fmaxf(lo - st.tq[k], st.tq[k] - (lo + size)));
+            dmin2 += dn * dn;
+        }
+        if (sqrtf(dmin2) >= st.Rout) continue;
+        const uint64_t code = (st.sim << (DIM * l)) | morton<DIM>(q);
+        const unsigned long long ent = a.cells[a.level_off[l] + (int64_t)code];
+        cs[h] = (uint32_t)ent;
+        const uint32_t ce = (uint32_t)(ent >> 32);
+        cn[h] = ce > cs[h] ? ce - cs[h] : 0;
+    }
+    uint32_t incl = cn[0] + cn[1];
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t v = __shfl_up_sync(0xffffffffu, incl, o);
+        if ((int)lane >= o) incl += v;
+    }
+    if (lane == 31) b.wsum[wid] = incl;
+    __syncthreads();
+    uint32_t before = incl - cn[0] - cn[1], T = 0;
+#pragma unroll
+    for (int w = 0; w < QL_THREADS / 32; ++w) {
+        if (w < wid) before += b.wsum[w];
+        T += b.wsum[w];
+    }
+    b.cstart[2 * tid] = cs[0];
+    b.cexcl[2 * tid] = before;
+    b.cstart[2 * tid + 1] = cs[1];
+    b.cexcl[2 * tid + 1] = before + cn[0];
+    __syncthreads();
+    // pass 0: every hit counted, and kept while there is room; with more than
+    // NB_CAP of them, the bin that holds the NB_CAP-th.  Pass 1, where they did
+    // not all fit: the hits up to that bin.  (T, total and the bins are uniform
+    // over the block.)
+    bool small = T <= QL_CAND;
+    uint32_t total = 0;
+    int last = QL_BINS;
+    for (int pass = 0; small && pass < 2; ++pass) {
+        uint32_t* const kept = pass == 0 ? &b.hits : &b.near;
+        for (uint32_t base = 0; base < T; base += QL_THREADS * QL_LOADS) {
+            uint32_t j[QL_LOADS];
+            float4 ph[QL_LOADS], pl[QL_LOADS];
+#pragma unroll
+            for (int u = 0; u < QL_LOADS; ++u) {
+                const uint32_t t = base + (uint32_t)(u * QL_THREADS + tid);
+                j[u] = 0xffffffffu;
+                ph[u] = pl[u] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                if (t >= T) continue;
+                int lo = 0;                                 // the last cell with cexcl <= t
+#pragma unroll
+                for (int s = FCAP / 2; s > 0; s >>= 1)
+                    if (b.cexcl[lo + s] <= t) lo += s;
+                j[u] = b.cstart[lo] + (t - b.cexcl[lo]);
+                ldg256(a.pos4 + 2 * (int64_t)j[u], ph[u], pl[u]);
+            }
+#pragma unroll
+            for (int u = 0; u < QL_LOADS; ++u) {
+                const bool test = j[u] != 0xffffffffu && (int64_t)j[u] != i;
+                const float hj[3] = {ph[u].x, ph[u].y, ph[u].z}, lj[3] = {pl[u].x, pl[u].y, pl[u].z};
+                float d2f = 0.0f;
+#pragma unroll
+                for (int k = 0; k < DIM; ++k) {
+                    float dh = hj[k] - st.hxi[k];
+                    float dl = lj[k] - st.lxi[k];
+                    if (c.periodic[k]) {
+                        if (dh > 0.5f * c.Lper_h[k]) { dh -= c.Lper_h[k]; dl -= c.Lper_l[k]; }
+                        else if (dh < -0.5f * c.Lper_h[k]) { dh += c.Lper_h[k]; dl += c.Lper_l[k]; }
+                    }
+                    const float d = dh + dl;
+                    d2f = fmaf(d, d, d2f);
+                }
+                bool in = test && d2f <= st.R2f * (1.0f - TOL_R);
+                if (test && !in && d2f <= st.R2f * (1.0f + TOL_R))
+                    in = inside64(c, DIM, exact_d2<DIM>(a, i, j[u]), __dmul_rn(a.sm[i], a.sV[i]));
+                const int bin = bin_of(d2f);
+                if (pass == 0) { if (in) atomicAdd(&b.hist[bin], 1u); }
+                else in = in && bin <= last;
+                // (one atomic a warp)
+                const unsigned im = __ballot_sync(0xffffffffu, in);
+                if (!im) continue;
+                uint32_t pos = 0;
+                if (lane == 0) pos = atomicAdd(kept, (uint32_t)__popc(im));
+                pos = __shfl_sync(0xffffffffu, pos, 0) + (uint32_t)__popc(im & ((1u << lane) - 1u));
+                if (in && pos < (uint32_t)QL_HITS) {
+                    b.key[pos] = (unsigned long long)__float_as_uint(d2f) << 32;
+                    b.j[pos] = j[u];
+                }
+            }
+        }
+        __syncthreads();
+        if (pass == 1) break;
+        total = b.hits;
+        if (total <= (uint32_t)NB_CAP) break;
+        const uint32_t h0 = b.hist[2 * tid], h1 = b.hist[2 * tid + 1];
+        uint32_t inc = h0 + h1;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t v = __shfl_up_sync(0xffffffffu, inc, o);
+            if ((int)lane >= o) inc += v;
+        }
+        if (lane == 31) b.wsum[wid] = inc;
+        __syncthreads();
+        for (int w = 0; w < wid; ++w) inc += b.wsum[w];
+        const uint32_t exc = inc - h0 - h1, want = (uint32_t)NB_CAP;
+        if (exc < want && want <= exc + h0) b.last_bin = 2 * tid;
+        else if (exc + h0 < want && want <= inc) b.last_bin = 2 * tid + 1;
+        __syncthreads();
+        last = (int)b.last_bin;
+        if (total <= (uint32_t)QL_HITS) break;
+    }
+    uint32_t near = small && total > (uint32_t)QL_HITS ? b.near : total;      // hits in b.key
+    small = small && near <= (uint32_t)QL_HITS;
+    const int m = (int)min(total, (uint32_t)NB_CAP), kmax = c.k_max;
+    if (small && last == QL_BINS) {
+        if (tid < near) b.key[tid] |= a.sid[b.j[tid]];      // (at most NB_CAP hits: their ids)
+    } else if (small) {
+        // their ids, and only those up to the bin: read by all before any is written
+        unsigned long long k[QL_HITS / QL_THREADS];
+        uint32_t jk[QL_HITS / QL_THREADS];
+        unsigned mine = 0;
+#pragma unroll
+        for (int u = 0; u < QL_HITS / QL_THREADS; ++u) {
+            const uint32_t e = (uint32_t)(u * QL_THREADS + tid);
+            k[u] = 0;
+            jk[u] = 0;
+            if (e >= near) continue;
+            const unsigned long long kk = b.key[e];
+            if (bin_of(key_d2(kk)) > last) continue;
+            jk[u] = b.j[e];
+            k[u] = kk | a.sid[jk[u]];
+            mine |= 1u << u;
+        }
+        __syncthreads();
+        if (tid == 0) b.near = 0;
+        __syncthreads();
+#pragma unroll
+        for (int u = 0; u < QL_HITS / QL_THREADS; ++u)
+            if ((mine >> u) & 1u) {
+                const uint32_t pos = atomicAdd(&b.near, 1u);
+                b.key[pos] = k[u];
+                b.j[pos] = jk[u];
+            }
+        __syncthreads();
+        near = b.near;
+    }
+    if (small) {
+        if (tid < 2) b.key[near + tid] = ~0ull;             // pads the last pair
+        __syncthreads();
+        // each hit's place: the keys before it (equal keys, from equal ids,
+        // keep their order, so the places are distinct)
+        for (uint32_t e = tid; e < near; e += QL_THREADS) {
+            const unsigned long long ke = b.key[e];
+            uint32_t r = 0;
+#pragma unroll 4
+            for (uint32_t q = 0; q < near; q += 2) {
+                const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(&b.key[q]);
+                r += (v.x < ke || (v.x == ke && q < e)) ? 1u : 0u;
+                r += (v.y < ke || (v.y == ke && q + 1 < e)) ? 1u : 0u;
+            }
+            if (r < (uint32_t)NB_CAP) { b.w.key[r] = ke; b.w.j[r] = b.j[e]; }
+        }
+    }
+    __syncthreads();
+    if (wid != 0) return;
+    if (small && total > (uint32_t)NB_CAP) {
+        // hits past the buffer may only be missed by a run of ties that spans
+        // from the last entry kept to the buffer's end
+        int open = 1;
+        for (int e = kmax + (int)lane; e < NB_CAP; e += 32)
+            if (!(key_d2(b.w.key[e]) <= key_d2(b.w.key[e - 1]) * (1.0f + TOL_T))) open = 0;
+        small = !__all_sync(0xffffffffu, open);
+    }
+    if (!small) {
+        query_one<DIM>(a, b.w, i);
+        return;
+    }
+    order_ties<DIM>(a, b.w, m, i);
+    const int cnt = min(m, kmax);
+    for (int e = lane; e < cnt; e += 32) a.idx[i * (int64_t)kmax + e] = b.w.j[e];
+    if (lane == 0) {
+        a.count[i] = (uint32_t)cnt;
+        a.total[i] = min(total, 4u * (uint32_t)kmax);
+        a.d2min[i] = cnt > 0 ? exact_d2<DIM>(a, i, b.w.j[0]) : INFINITY;
+        if (total > (uint32_t)kmax) atomicAdd(a.counters + C_OVERFLOW, 1ull);
+        atomicMax(a.counters + C_MAXCOUNT, (unsigned long long)total);
+    }
+}
+
+template <int DIM>
+__global__ void __launch_bounds__(QL_THREADS) k_query_left(QueryArgs a)
+{
+    __shared__ LeftBuf b;
+    const unsigned long long len = *a.list_len;
+    for (unsigned long long t = blockIdx.x; t < len; t += gridDim.x) {
+        query_left<DIM>(a, b, (int64_t)a.list[t]);
+        __syncthreads();                    // the buffers are reused by the next particle
     }
 }
 
@@ -865,55 +1131,69 @@ __global__ void __launch_bounds__(NB_WARPS * 32) k_query_octant(QueryArgs a)
 }
 
 // ---------------------------------------------------------------------------
-// Tile kernel: one warp per 32 consecutive particles in key order.  The tile
-// is cut into groups where consecutive particles lie more than TQ_GAP radii
-// apart (jumps of the Morton curve) or belong to different simulations; each
-// group is a compact region of space.  For a group:
+// Tile kernel: one block of W warps per 32 consecutive particles in key
+// order.  The tile is cut into groups where consecutive particles lie more than
+// TQ_GAP radii apart (jumps of the Morton curve) or belong to different
+// simulations; each group is a compact region of space.  For a group:
 //   1. the cells of one level (edge >= half the group's largest radius) within
-//      reach of the group's bounding box are classified lane-parallel and the
-//      non-empty ones compacted;
-//   2. their particles are staged 32 at a time in shared memory as positions
-//      relative to the group's first particle, and every lane tests each staged
-//      candidate against its own particle with a margin that covers the
-//      rounding of the relative coordinates (a prefilter: no neighbour is
-//      lost), keeping the index of each hit in its own column of a shared list;
-//   3. per particle, the warp recomputes the hits' distances exactly as the
-//      per-particle kernel does (float hi/lo offsets; FP64 inside the rounding
-//      band of the radius), sorts (float d2, index) with a register bitonic
-//      network, re-orders near-tie runs by (FP64 d2, id) and writes the row.
+//      reach of the group's bounding box are classified a lane per cell, the
+//      warps taking turns, and the non-empty ones compacted;
+//   2. each warp stages the particles of every W-th cell 32 at a time in
+//      shared memory as positions relative to the group's first particle, and
+//      every lane tests each staged candidate against its own particle (lane q
+//      of every warp: particle q) with a margin that covers the rounding of the
+//      relative coordinates (a prefilter: no neighbour is lost), keeping the
+//      index of each hit in its particle's column of a shared list;
+//   3. each warp takes every W-th particle: it recomputes the hits'
+//      distances exactly as the per-particle kernel does (float hi/lo offsets;
+//      FP64 inside the rounding band of the radius), sorts (float d2, index) with
+//      a register bitonic network, re-orders near-tie runs by (FP64 d2, id) and
+//      writes the row.
 // Particles with more than TQ_CAP hits, and groups whose region spans too many
 // cells or candidates, are left to the per-particle kernel.
 // ---------------------------------------------------------------------------
-constexpr int TQ_WARPS = 4;
-constexpr int TQ_CAP = 64;            // prefilter hits a lane keeps (two sort keys per lane)
+constexpr int TQ_CAP = 64;            // prefilter hits a particle keeps (two sort keys per lane)
 constexpr int TQ_PAD = 33;            // column stride: a row read across lanes is conflict-free
-constexpr int TQ_CELLS_MAX = 4096;    // cells a group's region may span
+constexpr int TQ_CELLS_MIN = 512;     // cells the region of a group may span: this many, and
+constexpr int TQ_CELLS_PER = 64;      // so many a particle (a compact group of 32 spans 100 to 1000)
 constexpr uint32_t TQ_CAND_MAX = 2048;   // candidates a group may test (fastest of 2048, 4096, 8192 on the gas cloud)
-constexpr int TQ_KC = 256;            // non-empty cells a group may keep
+constexpr int TQ_KC = 512;            // non-empty cells a group may keep
 constexpr float TQ_GAP = 2.0f;        // in radii
-constexpr int TQ_SPLIT_MIN = 4;       // smallest half a too-large group is split into
+// Warps of a tile's block.  Two, 16 blocks of 64 registers a thread to an SM
+// (32 warps, where a warp per tile with its own column buffer allowed 20), for
+// the throughput of large sets: 1.94 ms at 2M particles, against 2.08 with four
+// warps, 2.65 with eight, 2.34 with a warp per tile.  Four while the tiles are
+// few and a tile's own time counts: 50 us at 20k against 78 with two and 194 with
+// a warp per tile; 158 and 162 us at 131k.
+constexpr int TQ_SMALL_N = 200000;
+constexpr int tile_blocks(int W) { return 32 / W; }      // resident blocks per SM
+constexpr int TQ_DENSE_MAX = 4;       // largest group that is not halved when GROUP_DENSE
 
+template <int W>
 struct TileBuf {
-    uint32_t kj[TQ_CAP][TQ_PAD];      // prefilter hits, one column per lane
+    uint32_t kj[TQ_CAP][TQ_PAD];      // prefilter hits, one column per particle
     unsigned long long kc[TQ_KC];     // kept cells: start | count << 32
-    alignas(16) float cx[32];         // staged candidates: position relative to the group's origin,
-    alignas(16) float cy[32];         // read four at a time by the prefilter
-    alignas(16) float cz[32];
-    uint32_t cj[32];                  // and index
+    alignas(16) float cx[W][32];   // staged candidates: position relative to the group's origin,
+    alignas(16) float cy[W][32];   // read four at a time by the prefilter
+    alignas(16) float cz[W][32];
+    uint32_t cj[W][32];        // and index
+    uint32_t cnt[32];                 // prefilter hits of each particle
+    uint32_t near_j[32];              // each particle's nearest entry (none, or handed over: all ones)
+    uint32_t ncand[2], nk[2];         // candidates and kept cells, by group parity
+    unsigned long long tile;          // persistent form: the tile taken from the queue
 };
-static_assert(sizeof(TileBuf) % 16 == 0, "per-warp buffers keep the 16-byte alignment of cx, cy, cz");
 
 __device__ inline float warp_minf(float v)
 {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = fminf(v, __shfl_xor_sync(0xffffffffu, v, o));
-    return v;
+    float r;
+    asm("redux.sync.min.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
+    return r;
 }
 __device__ inline float warp_maxf(float v)
 {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
-    return v;
+    float r;
+    asm("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
+    return r;
 }
 
 __device__ inline void list_append(const QueryArgs& a, bool pred, uint32_t v)
@@ -1010,18 +1290,24 @@ __device__ inline void bitonic_keys(uint32_t (&key)[2])
     }
 }
 
-// one group of lanes of the tile (act); all 32 lanes take part.  false: the
-// group's region spans too many cells or candidates, nothing was written (the
-// caller splits the group or hands its particles to the per-particle kernel)
-template <int DIM, bool PER>
-__device__ bool tile_group(const QueryArgs& a, TileBuf& b, int64_t i, bool act, uint64_t sim,
-                           const TileLane<DIM>& me)
+// one group of particles of the tile (act, lane q of every warp: particle q);
+// the whole block takes part.  parity: which of the two sets of counters the
+// group uses (zero on entry; the other set is zeroed for the next group).
+// Returns 0 when done; otherwise the group's region spans too many cells or
+// candidates, nothing was written, and the caller splits the group into
+// 2^result parts or, GROUP_DENSE and few, hands it to the per-particle kernel
+enum { GROUP_DONE = 0, GROUP_DENSE = 3 };
+constexpr uint32_t NO_ENTRY = 0xffffffffu, HANDED = 0xfffffffeu;   // TileBuf::near_j
+template <int DIM, bool PER, int W>
+__device__ int tile_group(const QueryArgs& a, TileBuf<W>& b, int64_t i, bool act, uint64_t sim,
+                          const TileLane<DIM>& me, int& parity)
 {
     const unsigned lane = lane_id();
+    const int wid = (int)(threadIdx.x >> 5);
     const DevCfg& c = a.c;
     const int mb = c.mbits;
     const Grid& g = a.g[sim];
-    if (PER && act) {
+    if (PER && act && wid == 0) {
 #pragma unroll
         for (int k = 0; k < DIM; ++k)
             if (c.periodic[k] && 2.0f * me.Rq >= ldexpf(1.0f, mb))
@@ -1067,7 +1353,9 @@ __device__ bool tile_group(const QueryArgs& a, TileBuf& b, int64_t i, bool act, 
         nc[k] = a1 - a0 + 1;
         ncells = nc[k] < 1 ? 0 : ncells * nc[k];
     }
-    if (ncells > TQ_CELLS_MAX) return false;     // a scattered group
+    // a scattered group: its parts have far fewer cells a particle
+    const int np = __popc(__ballot_sync(0xffffffffu, act));
+    if (ncells > TQ_CELLS_MIN + TQ_CELLS_PER * np) return 1;
     const int nct = (int)ncells;
     float rnc[3];
 #pragma unroll
@@ -1105,24 +1393,32 @@ __device__ bool tile_group(const QueryArgs& a, TileBuf& b, int64_t i, bool act, 
     // ---- 1. the group's candidate count (a dense region under a wide group is
     // cheaper per particle) and, while they fit, its non-empty cells compacted
     const unsigned lt = (1u << lane) - 1u;
-    int nk = 0;                       // compacted cells in b.kc
-    bool spill = false;               // more non-empty cells than b.kc holds
-    {
-        uint32_t ncand = 0;
-        for (int base0 = 0; base0 < nct && ncand <= TQ_CAND_MAX; base0 += 32) {
-            uint32_t cs, cn;
-            cell_range(base0 + (int)lane, cs, cn);
-            ncand += __reduce_add_sync(0xffffffffu, cn);
-            const unsigned km = __ballot_sync(0xffffffffu, cn > 0);
-            if (!spill && nk + __popc(km) > TQ_KC) spill = true;
-            if (!spill) {
-                if (cn > 0) b.kc[nk + __popc(km & lt)] = (unsigned long long)cs | ((unsigned long long)cn << 32);
-                nk += __popc(km);
-            }
+    const int par = parity;
+    for (int base0 = 32 * wid; base0 < nct; base0 += 32 * W) {
+        uint32_t cs, cn;
+        cell_range(base0 + (int)lane, cs, cn);
+        const uint32_t add = __reduce_add_sync(0xffffffffu, cn);
+        const unsigned km = __ballot_sync(0xffffffffu, cn > 0);
+        if (!km) continue;
+        uint32_t at = 0, seen = 0;
+        if (lane == 0) {
+            at = atomicAdd(&b.nk[par], (uint32_t)__popc(km));
+            seen = atomicAdd(&b.ncand[par], add) + add;
         }
-        if (ncand > TQ_CAND_MAX) return false;
+        at = __shfl_sync(0xffffffffu, at, 0) + (uint32_t)__popc(km & lt);
+        if (cn > 0 && at < (uint32_t)TQ_KC) b.kc[at] = (unsigned long long)cs | ((unsigned long long)cn << 32);
+        if (__shfl_sync(0xffffffffu, seen, 0) > 4u * TQ_CAND_MAX) break;
     }
-    __syncwarp();
+    if (threadIdx.x < 32) b.cnt[threadIdx.x] = 0;
+    __syncthreads();
+    const uint32_t ncand = b.ncand[par];
+    const int nk = (int)b.nk[par];
+    parity = par ^ 1;
+    if (ncand > TQ_CAND_MAX || nk > TQ_KC) {
+        if (threadIdx.x == 0) { b.ncand[par ^ 1] = 0; b.nk[par ^ 1] = 0; }
+        __syncthreads();
+        return ncand > 4u * TQ_CAND_MAX ? GROUP_DENSE : (ncand > 2u * TQ_CAND_MAX ? 2 : 1);
+    }
 
     // ---- 2. prefilter: candidates relative to the group's first particle
     const int lead = __ffs(__ballot_sync(0xffffffffu, act)) - 1;
@@ -1145,14 +1441,18 @@ __device__ bool tile_group(const QueryArgs& a, TileBuf& b, int64_t i, bool act, 
     float halfL[3], Lh[3];
 #pragma unroll
     for (int k = 0; k < 3; ++k) { Lh[k] = c.Lper_h[k]; halfL[k] = 0.5f * c.Lper_h[k]; }
+    // no minimum image between the group's particles and its candidates: an open
+    // domain, or a periodic one in which the region, with the group on either
+    // side of the origin, stays within half a period
+    const bool flat = !PER || (2.0f * ext + Rqm + size + 8.0f) * 1.001f < 0.5f * period;
     // the group's box in the relative coordinates, and a bound on a candidate's
     // squared distance to it above every lane's threshold (the distance to the
     // box is at most the distance to any lane's particle; the margin covers the
-    // rounding of both): candidates beyond it are not staged (open domains;
-    // the minimum image of a periodic axis has no such box)
+    // rounding of both): candidates beyond it are not staged (where no minimum
+    // image is needed: otherwise there is no such box)
     float rlo[3] = {0.0f, 0.0f, 0.0f}, rhi[3] = {0.0f, 0.0f, 0.0f};
     float thr_box = INFINITY;
-    if (!PER) {
+    if (flat) {
 #pragma unroll
         for (int k = 0; k < DIM; ++k) {
             rlo[k] = warp_minf(act ? ri[k] : INFINITY);
@@ -1162,13 +1462,17 @@ __device__ bool tile_group(const QueryArgs& a, TileBuf& b, int64_t i, bool act, 
         const float Rm = warp_maxf(act ? me.Rf : 0.0f);
         thr_box = thm + ldexpf(thm + 4.0f * E * Rm, -18);
     }
-    uint32_t cnt = 0;                 // prefilter hits of this lane
-    // candidates of the compacted cells b.kc[0..nk), 32 cells at a time
-    auto scan_kept = [&](int nk) {
-        for (int c0 = 0; c0 < nk; c0 += 32) {
+    float* const cx = b.cx[wid];
+    float* const cy = b.cy[wid];
+    float* const cz = b.cz[wid];
+    uint32_t* const cjs = b.cj[wid];
+    // candidates of this warp's share of the kept cells, 32 cells at a time
+    {
+        for (int c0 = wid; c0 < nk; c0 += 32 * W) {
             uint32_t cs = 0, cn = 0;
-            if (c0 + (int)lane < nk) {
-                const unsigned long long ent = b.kc[c0 + lane];
+            const int ce = c0 + (int)lane * W;
+            if (ce < nk) {
+                const unsigned long long ent = b.kc[ce];
                 cs = (uint32_t)ent;
                 cn = (uint32_t)(ent >> 32);
             }
@@ -1207,26 +1511,26 @@ __device__ bool tile_group(const QueryArgs& a, TileBuf& b, int64_t i, bool act, 
                         const float dk = fmaxf(0.0f, fmaxf(rlo[k] - p[k], p[k] - rhi[k]));
                         d2b = fmaf(dk, dk, d2b);
                     }
-                    keep = PER || d2b <= thr_box;
+                    keep = d2b <= thr_box;      // (always, with no box: thr_box is infinite)
                 }
                 // the kept candidates, compacted
                 const unsigned km = __ballot_sync(0xffffffffu, keep);
                 if (keep) {
                     const int sl = __popc(km & lt);
-                    b.cx[sl] = p[0];
-                    b.cy[sl] = p[1];
-                    b.cz[sl] = p[2];
-                    b.cj[sl] = j;
+                    cx[sl] = p[0];
+                    cy[sl] = p[1];
+                    cz[sl] = p[2];
+                    cjs[sl] = j;
                 }
                 __syncwarp();
                 const int nb = __popc(km);
                 if (act && nb > 0) {
                     // bit q: staged candidate q passes the prefilter
                     uint32_t hits = 0;
-                    if (PER) {
+                    if (!flat) {
 #pragma unroll 4
                         for (int qq = 0; qq < nb; ++qq) {
-                            float d[3] = {b.cx[qq] - ri[0], b.cy[qq] - ri[1], b.cz[qq] - ri[2]};
+                            float d[3] = {cx[qq] - ri[0], cy[qq] - ri[1], cz[qq] - ri[2]};
 #pragma unroll
                             for (int k = 0; k < DIM; ++k)
                                 if (c.periodic[k]) {
@@ -1253,20 +1557,20 @@ __device__ bool tile_group(const QueryArgs& a, TileBuf& b, int64_t i, bool act, 
                         uint32_t miss = 0;
 #pragma unroll 1
                         for (int qq = 0; qq < nb; qq += 4) {
-                            const float4 X = *reinterpret_cast<const float4*>(&b.cx[qq]);
+                            const float4 X = *reinterpret_cast<const float4*>(&cx[qq]);
                             const float2 dxa = __fadd2_rn(make_float2(X.x, X.y), nx);
                             const float2 dxb = __fadd2_rn(make_float2(X.z, X.w), nx);
                             float2 d2a = __fmul2_rn(dxa, dxa);
                             float2 d2b = __fmul2_rn(dxb, dxb);
                             if (DIM > 1) {
-                                const float4 Y = *reinterpret_cast<const float4*>(&b.cy[qq]);
+                                const float4 Y = *reinterpret_cast<const float4*>(&cy[qq]);
                                 const float2 dya = __fadd2_rn(make_float2(Y.x, Y.y), ny);
                                 const float2 dyb = __fadd2_rn(make_float2(Y.z, Y.w), ny);
                                 d2a = __ffma2_rn(dya, dya, d2a);
                                 d2b = __ffma2_rn(dyb, dyb, d2b);
                             }
                             if (DIM > 2) {
-                                const float4 Z = *reinterpret_cast<const float4*>(&b.cz[qq]);
+                                const float4 Z = *reinterpret_cast<const float4*>(&cz[qq]);
                                 const float2 dza = __fadd2_rn(make_float2(Z.x, Z.y), nz);
                                 const float2 dzb = __fadd2_rn(make_float2(Z.z, Z.w), nz);
                                 d2a = __ffma2_rn(dza, dza, d2a);
@@ -1285,57 +1589,39 @@ __device__ bool tile_group(const QueryArgs& a, TileBuf& b, int64_t i, bool act, 
                         hits = ~(__brev(miss) >> (32 - nq));
                         if (nb < 32) hits &= (1u << nb) - 1u;   // slots past nb hold no candidate
                     }
-                    // append the hits to this lane's column, highest slot first (the
+                    // append the hits to this particle's column, highest slot first (the
                     // particle itself is one of them: the exact pass below drops it,
-                    // and sorts by (d2, id), so the column's order is free).  A lane
+                    // and sorts by (d2, id), so the column's order is free).  A particle
                     // whose hits overflow the column goes to the per-particle kernel,
                     // so then only the count matters
                     const uint32_t nh = (uint32_t)__popc(hits);
-                    if (cnt + nh <= (uint32_t)TQ_CAP) {
-                        uint32_t* col = &b.kj[cnt][lane];
+                    const uint32_t pos = nh ? atomicAdd(&b.cnt[lane], nh) : 0u;
+                    if (nh && pos + nh <= (uint32_t)TQ_CAP) {
+                        uint32_t* col = &b.kj[pos][lane];
                         while (hits) {
                             const int q = 31 - __clz(hits);
                             hits ^= 1u << q;
-                            *col = b.cj[q];
+                            *col = cjs[q];
                             col += TQ_PAD;
                         }
                     }
-                    cnt += nh;
                 }
                 __syncwarp();
             }
         }
-    };
-    if (!spill) {
-        scan_kept(nk);                // every kept cell is already in b.kc
-    } else {
-        // classify again, compacting the non-empty cells; scan whenever the
-        // buffer of kept cells would overflow, and at the end
-        nk = 0;
-        for (int base0 = 0; base0 < nct; base0 += 32) {
-            uint32_t cs, cn;
-            cell_range(base0 + (int)lane, cs, cn);
-            const unsigned km = __ballot_sync(0xffffffffu, cn > 0);
-            if (nk + __popc(km) > TQ_KC) {
-                __syncwarp();
-                scan_kept(nk);
-                nk = 0;
-            }
-            if (cn > 0) b.kc[nk + __popc(km & lt)] = (unsigned long long)cs | ((unsigned long long)cn << 32);
-            nk += __popc(km);
-        }
-        __syncwarp();
-        scan_kept(nk);
     }
+    if (threadIdx.x == 0) { b.ncand[par ^ 1] = 0; b.nk[par ^ 1] = 0; }
+    __syncthreads();
 
     // ---- 3. per particle: exact membership, order, row
+    const uint32_t cnt = b.cnt[lane];
     const bool mine = act && cnt <= (uint32_t)TQ_CAP;
-    list_append(a, act && !mine, (uint32_t)i);
+    if (wid == 0) list_append(a, act && !mine, (uint32_t)i);
     const uint32_t kmax = (uint32_t)c.k_max;
     uint32_t mx = 0, novf = 0;
-    uint32_t near_j = 0xffffffffu;       // this lane's particle: its nearest entry (none: all ones)
-    bool handed = false;                 // this lane's particle went to the per-particle kernel
-    unsigned todo = __ballot_sync(0xffffffffu, mine);
+    // this warp's share: every W-th of the particles
+    const unsigned all = __ballot_sync(0xffffffffu, mine);
+    unsigned todo = __ballot_sync(0xffffffffu, mine && (__popc(all & lt) & (W - 1)) == wid);
     // the hits of the next particle are loaded while the current one is sorted
     uint32_t fj[2] = {0u, 0u};
     float4 fh[2], fl[2];
@@ -1401,8 +1687,10 @@ __device__ bool tile_group(const QueryArgs& a, TileBuf& b, int64_t i, bool act, 
                                         __popc(__ballot_sync(0xffffffffu, key[1] < 0xffffffc0u)));
         if (c.select == LP_SELECT_OCTANT && nin > kmax) {
             // the octant-balanced selection of more than k_max: the per-particle kernel
-            if (lane == 0) a.fb_list[atomicAdd(a.fb_len, 1ull)] = (uint32_t)ip;
-            if ((int)lane == p) handed = true;
+            if (lane == 0) {
+                a.fb_list[atomicAdd(a.fb_len, 1ull)] = (uint32_t)ip;
+                b.near_j[p] = HANDED;
+            }
             continue;
         }
         if (m <= 32) bitonic_keys<1>(key);
@@ -1476,9 +1764,8 @@ __device__ bool tile_group(const QueryArgs& a, TileBuf& b, int64_t i, bool act, 
 #pragma unroll
         for (int s = 0; s < 2; ++s)
             if (lane + 32u * s < keep) a.idx[ip * (int64_t)kmax + lane + 32 * s] = jv[s];
-        const uint32_t j0 = __shfl_sync(0xffffffffu, jv[0], 0);
-        if ((int)lane == p) near_j = keep > 0 ? j0 : 0xffffffffu;
         if (lane == 0) {
+            b.near_j[p] = keep > 0 ? jv[0] : NO_ENTRY;
             a.count[ip] = keep;
             a.total[ip] = min(nin, 4u * kmax);
         }
@@ -1487,18 +1774,46 @@ __device__ bool tile_group(const QueryArgs& a, TileBuf& b, int64_t i, bool act, 
     }
     if (lane == 0) {
         if (novf) atomicAdd(a.counters + C_OVERFLOW, (unsigned long long)novf);
-        if (mx) atomicMax(a.counters + C_MAXCOUNT, (unsigned long long)mx);
+        // (a stale read can only be too small: the maximum never falls)
+        if ((unsigned long long)mx > __ldcg(a.counters + C_MAXCOUNT))
+            atomicMax(a.counters + C_MAXCOUNT, (unsigned long long)mx);
     }
+    __syncthreads();
     // the exact squared distance to each particle's nearest entry (the CFL
-    // step's ell^2), every lane its own particle
-    if (mine && !handed) a.d2min[i] = near_j != 0xffffffffu ? exact_d2<DIM>(a, i, near_j) : INFINITY;
-    __syncwarp();
-    return true;
+    // step's ell^2), by one warp: FP64 instructions cost the same for any number
+    // of lanes
+    if (wid == 0 && mine) {
+        const uint32_t nj = b.near_j[lane];
+        if (nj != HANDED) a.d2min[i] = nj != NO_ENTRY ? exact_d2<DIM>(a, i, nj) : INFINITY;
+    }
+    return GROUP_DONE;
 }
 
-// the tile of 32 key-ordered particles starting at i0 (< n), one warp
-template <int DIM, bool PER>
-__device__ __forceinline__ void tile_tile(const QueryArgs& a, TileBuf& b, int64_t i0)
+// the lanes g of the tile at i0 as parts of at most `size` particles, in key
+// order, to the list of k_query_groups (one warp)
+__device__ inline void groups_append(const QueryArgs& a, int64_t i0, unsigned g, int size)
+{
+    const unsigned lane = lane_id();
+    const int parts = (__popc(g) + size - 1) / size;
+    unsigned long long base = 0;
+    if (lane == 0) base = atomicAdd(a.gr_len, (unsigned long long)parts);
+    base = __shfl_sync(0xffffffffu, base, 0);
+    const int rank = __popc(g & ((1u << lane) - 1u));
+    if (((g >> lane) & 1u) && rank % size == 0) {
+        unsigned part = 0, rest = g & (0xffffffffu << lane);
+        for (int q = 0; q < size; ++q) { part |= rest & (0u - rest); rest &= rest - 1; }
+        a.gr_list[base + rank / size] = ((unsigned long long)(i0 >> 5) << 32) | part;
+    }
+}
+
+// the tile of 32 key-ordered particles starting at i0 (< n), one block; par: the
+// parity of the counters of its first group, updated for the next tile.  only:
+// the lanes to take (LISTED: a part of a group that was too large; it is halved
+// here down to single particles, where the whole tile's too-large groups are
+// listed, so that no block works through a long series of halves while the
+// others are done: on the 131k cloud such tiles ran for 300 us)
+template <int DIM, bool PER, int W, bool LISTED>
+__device__ __forceinline__ void tile_tile(const QueryArgs& a, TileBuf<W>& b, int64_t i0, int& par, unsigned only)
 {
     const unsigned lane = lane_id();
     const int64_t i = i0 + lane;
@@ -1526,62 +1841,91 @@ __device__ __forceinline__ void tile_tile(const QueryArgs& a, TileBuf& b, int64_
     }
     const float lim = TQ_GAP * fmaxf(Rq, pRq);
     const unsigned starts = __ballot_sync(0xffffffffu, valid && (lane == 0 || psim != mysim || !(gap2 <= lim * lim)));
-    const unsigned vmask = __ballot_sync(0xffffffffu, valid);
-    unsigned rest = starts;
+    const unsigned vmask = __ballot_sync(0xffffffffu, valid) & only;
+    unsigned rest = LISTED ? only & (0u - only) : starts;      // (a part lies within one group)
     while (rest) {                              // the groups, in turn
         const int s0 = __ffs(rest) - 1;
         rest &= rest - 1;
         const int s1 = rest ? __ffs(rest) - 1 : 32;
         const unsigned grp = vmask & ((s1 == 32 ? 0xffffffffu : ((1u << s1) - 1u)) & ~((1u << s0) - 1u));
         const uint64_t sim = __shfl_sync(0xffffffffu, mysim, s0);
-        // a group whose region is too large is halved (by key order: the
-        // halves are smaller regions) down to TQ_SPLIT_MIN particles; what is
-        // still too large goes to the per-particle kernel
-        unsigned stk[6];
+        if (!LISTED) {
+            const int r = tile_group<DIM, PER, W>(a, b, i, ((grp >> lane) & 1u) != 0u, sim, t, par);
+            const int pc = __popc(grp);
+            if (r == GROUP_DONE || threadIdx.x >= 32) continue;
+            if (pc > TQ_DENSE_MAX || (r != GROUP_DENSE && pc >= 2)) groups_append(a, i0, grp, max(1, pc >> (r + 1)));
+            else list_append(a, ((grp >> lane) & 1u) != 0u, (uint32_t)i);
+            continue;
+        }
+        // the part, halved (by key order: the halves are smaller regions) while
+        // its region is too large; single particles, and few particles among
+        // several times too many candidates, go to the per-particle kernel
+        unsigned stk[8];
         int sp = 0;
         stk[sp++] = grp;
         while (sp > 0) {
             const unsigned g = stk[--sp];
-            if (tile_group<DIM, PER>(a, b, i, ((g >> lane) & 1u) != 0u, sim, t)) continue;
+            const int r = tile_group<DIM, PER, W>(a, b, i, ((g >> lane) & 1u) != 0u, sim, t, par);
+            if (r == GROUP_DONE) continue;
             const int pc = __popc(g);
-            if (pc >= 2 * TQ_SPLIT_MIN && sp + 2 <= 6) {
+            if (pc > TQ_DENSE_MAX || (r != GROUP_DENSE && pc >= 2)) {
                 unsigned lo = 0, gg = g;                // the first pc / 2 members
                 for (int q = 0; q < pc / 2; ++q) { lo |= gg & (0u - gg); gg &= gg - 1; }
                 stk[sp++] = g & ~lo;
                 stk[sp++] = lo;
-            } else {
+            } else if (threadIdx.x < 32) {
                 list_append(a, ((g >> lane) & 1u) != 0u, (uint32_t)i);
             }
         }
     }
 }
 
-template <int DIM, bool PER>
-__global__ void __launch_bounds__(TQ_WARPS * 32, 5) k_query_tile(QueryArgs a)
+template <int W>
+__device__ __forceinline__ void tile_init(TileBuf<W>& b)
 {
-    extern __shared__ __align__(16) unsigned char tq_smem[];
-    TileBuf& b = reinterpret_cast<TileBuf*>(tq_smem)[threadIdx.x >> 5];
-    const int64_t i0 = ((int64_t)blockIdx.x * TQ_WARPS + (threadIdx.x >> 5)) * 32;
-    if (i0 >= a.n) return;                      // whole warp
-    tile_tile<DIM, PER>(a, b, i0);
+    if (threadIdx.x < 2) { b.ncand[threadIdx.x] = 0; b.nk[threadIdx.x] = 0; }
+    __syncthreads();
 }
 
-// Persistent form (LP_SCHED_QUEUE_QUERY): a grid of resident blocks whose
-// warps take their next tile from a.queue until none is left, so a warp whose
-// tile was cheap takes another at once instead of holding its slot (and its
-// shared-memory buffer) until the slowest warp of its block ends.
-template <int DIM, bool PER>
-__global__ void __launch_bounds__(TQ_WARPS * 32, 5) k_query_tile_q(QueryArgs a)
+template <int DIM, bool PER, int W>
+__global__ void __launch_bounds__(W * 32, tile_blocks(W)) k_query_tile(QueryArgs a)
 {
-    extern __shared__ __align__(16) unsigned char tq_smem[];
-    TileBuf& b = reinterpret_cast<TileBuf*>(tq_smem)[threadIdx.x >> 5];
+    __shared__ TileBuf<W> b;
+    tile_init(b);
+    int par = 0;
+    tile_tile<DIM, PER, W, false>(a, b, (int64_t)blockIdx.x * 32, par, 0xffffffffu);
+}
+
+// the parts of the groups that were too large
+template <int DIM, bool PER, int W>
+__global__ void __launch_bounds__(W * 32, tile_blocks(W)) k_query_groups(QueryArgs a)
+{
+    __shared__ TileBuf<W> b;
+    tile_init(b);
+    int par = 0;
+    const unsigned long long len = *a.gr_len;
+    for (unsigned long long t = blockIdx.x; t < len; t += gridDim.x) {
+        const unsigned long long it = a.gr_list[t];
+        tile_tile<DIM, PER, W, true>(a, b, (int64_t)(it >> 32) * 32, par, (unsigned)it);
+        __syncthreads();                        // the buffers are reused by the next part
+    }
+}
+
+// Persistent form (LP_SCHED_QUEUE_QUERY): a grid of resident blocks that take
+// their next tile from a.queue until none is left.
+template <int DIM, bool PER, int W>
+__global__ void __launch_bounds__(W * 32, tile_blocks(W)) k_query_tile_q(QueryArgs a)
+{
+    __shared__ TileBuf<W> b;
+    tile_init(b);
+    int par = 0;
     for (;;) {
-        unsigned long long base = 0;
-        if (lane_id() == 0) base = atomicAdd(a.queue, 32ull);
-        base = __shfl_sync(0xffffffffu, base, 0);
+        if (threadIdx.x == 0) b.tile = atomicAdd(a.queue, 32ull);
+        __syncthreads();
+        const unsigned long long base = b.tile;
         if (base >= (unsigned long long)a.n) return;
-        tile_tile<DIM, PER>(a, b, (int64_t)base);
-        __syncwarp();                           // the buffer is reused by the next tile
+        tile_tile<DIM, PER, W, false>(a, b, (int64_t)base, par, 0xffffffffu);
+        __syncthreads();                        // b.tile and the buffers are reused by the next tile
     }
 }
 
@@ -1676,6 +2020,38 @@ __global__ void k_octant_coverage(int64_t n, DevCfg c, const float4* __restrict_
     if ((threadIdx.x & 31u) == 0u && b) atomicAdd(ngap, (unsigned long long)__popc(b));
 }
 
+namespace {
+
+template <int DIM, bool PER, int W>
+cudaError_t launch_tiles_w(const QueryArgs& a, bool queue, cudaStream_t s)
+{
+    const unsigned tiles = (unsigned)((a.n + 31) / 32), resident = 152u * tile_blocks(W);
+    if (queue) {
+        // as many blocks as are resident at once, never more than the tiles need
+        int dev = 0, sms = 0, per_sm = 0;
+        cudaError_t e;
+        if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+        if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+        if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_query_tile_q<DIM, PER, W>, W * 32, 0)) !=
+            cudaSuccess)
+            return e;
+        if (per_sm < 1) return cudaErrorInvalidConfiguration;
+        k_query_tile_q<DIM, PER, W><<<std::min((unsigned)(sms * per_sm), tiles), W * 32, 0, s>>>(a);
+    } else {
+        k_query_tile<DIM, PER, W><<<tiles, W * 32, 0, s>>>(a);
+    }
+    k_query_groups<DIM, PER, W><<<resident, W * 32, 0, s>>>(a);
+    return cudaGetLastError();
+}
+
+template <int DIM, bool PER>
+cudaError_t launch_tiles(const QueryArgs& a, bool queue, cudaStream_t s)
+{
+    return a.n < TQ_SMALL_N ? launch_tiles_w<DIM, PER, 4>(a, queue, s) : launch_tiles_w<DIM, PER, 2>(a, queue, s);
+}
+
+}  // namespace
+
 cudaError_t query_neighbors(lp_ctx* c, int64_t n, cudaStream_t s)
 {
     if (n == 0) return cudaSuccess;
@@ -1698,6 +2074,8 @@ cudaError_t query_neighbors(lp_ctx* c, int64_t n, cudaStream_t s)
     a.list_len = nullptr;
     a.fb_list = c->redo_list;                  // capacity n: each particle is appended at most once
     a.fb_len = c->counters + C_QFB_LEN;
+    a.gr_list = static_cast<unsigned long long*>(c->mid);   // (the fit's record: free until then, 8 bytes a particle or more)
+    a.gr_len = c->counters + C_GROUP_LEN;
     a.queue = nullptr;
     if (c->dc.radius_mode == LP_RADIUS_KSIDE) {
         k_query_kside<<<(unsigned)((n + 127) / 128), 128, 0, s>>>(a);
@@ -1708,7 +2086,8 @@ cudaError_t query_neighbors(lp_ctx* c, int64_t n, cudaStream_t s)
         k_query<1><<<(unsigned)((n + NB_WARPS - 1) / NB_WARPS), NB_WARPS * 32, 0, s>>>(a);
         return cudaGetLastError();
     }
-    cudaError_t e = cudaMemsetAsync(c->counters + C_QFB_LEN, 0, 8, s);
+    static_assert(C_GROUP_LEN == C_QFB_LEN + 1, "one memset for both lengths");
+    cudaError_t e = cudaMemsetAsync(c->counters + C_QFB_LEN, 0, 16, s);
     if (e != cudaSuccess) return e;
     const bool octant = c->dc.select == LP_SELECT_OCTANT;
     if (c->schedule & LP_SCHED_QUERY_WARP) {   // one warp per particle for every particle
@@ -1722,41 +2101,27 @@ cudaError_t query_neighbors(lp_ctx* c, int64_t n, cudaStream_t s)
         }
         return cudaGetLastError();
     }
-    // tiles first; the particles they leave go to the per-particle kernel
+    // tiles first, then the parts of the groups they found too large; the
+    // particles both leave go to the per-particle kernel
     const bool per = c->dc.periodic[0] || c->dc.periodic[1] || c->dc.periodic[2];
-    const int64_t tiles = (n + 31) / 32;
-    const unsigned tblocks = (unsigned)((tiles + TQ_WARPS - 1) / TQ_WARPS);
-    const size_t smem = sizeof(TileBuf) * TQ_WARPS;
-    if (c->schedule & LP_SCHED_QUEUE_QUERY) {
-        // as many blocks as are resident at once, never more than the tiles need
-        auto kq = dim == 3 ? (per ? k_query_tile_q<3, true> : k_query_tile_q<3, false>)
-                           : (per ? k_query_tile_q<2, true> : k_query_tile_q<2, false>);
-        int dev = 0, sms = 0, per_sm = 0;
-        if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-        if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-        if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kq, TQ_WARPS * 32, smem)) != cudaSuccess)
-            return e;
-        if (per_sm < 1) return cudaErrorInvalidConfiguration;
-        const unsigned qb = (unsigned)std::min<int64_t>((int64_t)sms * per_sm, (int64_t)tblocks);
+    const bool queue = (c->schedule & LP_SCHED_QUEUE_QUERY) != 0;
+    if (queue) {
         a.queue = c->counters + C_QUEUE_TILE;
         if ((e = cudaMemsetAsync(a.queue, 0, 8, s)) != cudaSuccess) return e;
-        kq<<<qb, TQ_WARPS * 32, smem, s>>>(a);
-    } else if (dim == 3) {
-        if (per) k_query_tile<3, true><<<tblocks, TQ_WARPS * 32, smem, s>>>(a);
-        else k_query_tile<3, false><<<tblocks, TQ_WARPS * 32, smem, s>>>(a);
-    } else {
-        if (per) k_query_tile<2, true><<<tblocks, TQ_WARPS * 32, smem, s>>>(a);
-        else k_query_tile<2, false><<<tblocks, TQ_WARPS * 32, smem, s>>>(a);
     }
+    if (dim == 3) e = per ? launch_tiles<3, true>(a, queue, s) : launch_tiles<3, false>(a, queue, s);
+    else e = per ? launch_tiles<2, true>(a, queue, s) : launch_tiles<2, false>(a, queue, s);
+    if (e != cudaSuccess) return e;
     a.list = c->redo_list;
     a.list_len = c->counters + C_QFB_LEN;
-    const unsigned fblocks = 152u * 4u;
     if (octant) {
+        const unsigned fblocks = 152u * 4u;
         if (dim == 3) k_query_octant<3><<<fblocks, NB_WARPS * 32, 0, s>>>(a);
         else k_query_octant<2><<<fblocks, NB_WARPS * 32, 0, s>>>(a);
     } else {
-        if (dim == 3) k_query<3><<<fblocks, NB_WARPS * 32, 0, s>>>(a);
-        else k_query<2><<<fblocks, NB_WARPS * 32, 0, s>>>(a);
+        const unsigned fblocks = 152u * 8u;
+        if (dim == 3) k_query_left<3><<<fblocks, QL_THREADS, 0, s>>>(a);
+        else k_query_left<2><<<fblocks, QL_THREADS, 0, s>>>(a);
     }
     return cudaGetLastError();
 }
@@ -1765,21 +2130,7 @@ int query_launches(const lp_ctx* c)
 {
     if (c->dc.radius_mode == LP_RADIUS_KSIDE) return 1;
     if (c->dc.dim == 1 || (c->schedule & LP_SCHED_QUERY_WARP)) return 1;
-    return 2;
-}
-
-cudaError_t query_init()
-{
-    const int smem = (int)(sizeof(TileBuf) * TQ_WARPS);
-    cudaError_t e;
-    if ((e = cudaFuncSetAttribute(k_query_tile<3, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(k_query_tile<3, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(k_query_tile<2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(k_query_tile<2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(k_query_tile_q<3, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(k_query_tile_q<3, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(k_query_tile_q<2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess) return e;
-    return cudaFuncSetAttribute(k_query_tile_q<2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    return 3;
 }
 
 }  // namespace lp
