@@ -72,7 +72,7 @@ void free_all(lp_ctx* c)
                     c->sV, c->su[0], c->su[1], c->su[2], c->sP, c->sm, c->sid, c->rec, c->pos4, c->cells, c->nb_count, c->nb_total,
                     c->nb_idx, c->nb_d2min, c->grid, c->dt_dev, c->dt_min, c->counters, c->redo_list,
                     c->plain_list, c->refine_list, c->mid, c->ext, c->grange, c->level_off_dev, c->sim_of,
-                    c->mlp_master, c->mlp_bf16, c->mlp_m1, c->mlp_m2, c->mlp_grad, c->mlp_loss, c->stage_buf,
+                    c->mlp_master, c->mlp_bf16, c->mlp_m1, c->mlp_m2, c->mlp_grad, c->mlp_work, c->stage_buf,
                     c->in_pattern, c->in_state, c->in_part};
     for (void* p : ptrs)
         if (p) cudaFree(p);
@@ -451,7 +451,7 @@ lp_status lp_create(const lp_config* cfg, lp_ctx** out)
     A(dalloc(&c->counters, C_COUNT * 8));
     A(dalloc(&c->mlp_master, MLP_NPARAM * 4)); A(dalloc(&c->mlp_bf16, MLP_NPARAM * 2));
     A(dalloc(&c->mlp_m1, MLP_NPARAM * 4)); A(dalloc(&c->mlp_m2, MLP_NPARAM * 4));
-    A(dalloc(&c->mlp_grad, MLP_NPARAM * 4)); A(dalloc(&c->mlp_loss, 4));
+    A(dalloc(&c->mlp_grad, MLP_NPARAM * 4)); A(dalloc(&c->mlp_work, MLP_WORK * sizeof(float)));
     if (ok) {
         A(cudaMemset(c->cells, 0, (size_t)c->table_entries * 8));
         A(cudaMemset(c->counters, 0, C_COUNT * 8));

@@ -33,6 +33,7 @@ constexpr uint32_t ST_CAPACITY = 1u << LP_ERR_CAPACITY;
 constexpr uint32_t ST_ILLCOND = 1u << LP_ERR_ILLCOND;
 constexpr uint32_t ST_NONFINITE = 1u << LP_ERR_NONFINITE;
 constexpr uint32_t ST_ARG = 1u << LP_ERR_ARG;
+constexpr uint32_t ST_TIMEOUT = 1u << LP_ERR_TIMEOUT;
 
 // per-particle fit flags (lp_gfd_derivs status output)
 constexpr uint32_t FIT_LINEAR = 1u, FIT_NONE = 2u, FIT_FP64 = 8u;
@@ -319,7 +320,7 @@ struct lp_ctx {
     float* mlp_m1;
     float* mlp_m2;
     float* mlp_grad;
-    float* mlp_loss;
+    float* mlp_work;              // training: epoch losses, gradient buffers, barrier (MLP_WORK)
     int64_t mlp_step;
     int mlp_ready;
     // reservoir inflow (lp_inflow): the in-plane lattice of a layer [in_npat][2],
