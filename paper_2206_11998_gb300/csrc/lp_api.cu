@@ -73,7 +73,7 @@ void free_all(lp_ctx* c)
                     c->nb_idx, c->nb_d2min, c->grid, c->dt_dev, c->dt_min, c->counters, c->redo_list,
                     c->plain_list, c->refine_list, c->mid, c->ext, c->grange, c->level_off_dev, c->sim_of,
                     c->mlp_master, c->mlp_bf16, c->mlp_m1, c->mlp_m2, c->mlp_grad, c->mlp_work, c->stage_buf,
-                    c->in_pattern, c->in_state, c->in_part};
+                    c->in_pattern, c->in_state, c->in_part, c->tickets};
     for (void* p : ptrs)
         if (p) cudaFree(p);
 }
@@ -145,29 +145,83 @@ __global__ void k_split_fields(int64_t n, int nf, int F, const double* f0, const
     for (int q = 0; q < nf; ++q) split(f[q][i], r[rec_fh(q, F)], r[rec_fl(q, F)]);
 }
 
+// the time step of simulation s from its smallest d2 / c^2 (bit pattern), and t
+__device__ inline void dt_finalize(int s, double cfl, double dt_fixed, double t_end, unsigned long long dtmin,
+                                   double* dt, double* t, unsigned long long* counters)
+{
+    double v;
+    if (dt_fixed > 0.0) v = dt_fixed;
+    else v = cfl * sqrt(__longlong_as_double((long long)dtmin));
+    if (!(v > 0.0) || isinf(v) || isnan(v)) {
+        atomicOr(reinterpret_cast<unsigned int*>(counters + C_STATUS), ST_NONFINITE);
+        v = 0.0;
+    }
+    if (s == 0) counters[C_STEPS] += 1;
+    // the last step ends at t_end (a simulation already there does not move)
+    if (t && t_end > 0.0) {
+        const double rem = fmax(__dsub_rn(t_end, t[s]), 0.0);
+        if (v >= rem) {
+            dt[s] = rem;
+            t[s] = fmax(t[s], t_end);
+            return;
+        }
+    }
+    dt[s] = v;
+    if (t) t[s] += v;
+}
+
 // dt_s = cfl * sqrt(min_i d2min_i / (gamma P_i V_i)) over the fluid particles of
-// simulation s (one simulation: a grid-stride loop; several: one particle per
-// thread, reduced over the warp when its particles share a simulation)
-__global__ void k_cfl(int64_t n, DevCfg c, const double* d2min, const double* P, const double* V,
-                      const uint32_t* id, const uint64_t* keys, int key_shift, unsigned long long* dtmin)
+// simulation s.  Each thread takes its block's next CFL_ITEMS particles (one
+// simulation: a grid-stride loop) with the smallest quotient so far in
+// registers; a change of simulation passes it on.  A block whose threads end in
+// one simulation reduces to one atomic: with an atomic per warp, on the few
+// addresses of the simulations, the 2D ensemble's 2.5M particles took 100 us.
+// The last block to finish sets the time steps and puts the minima back to
+// their initial value.
+constexpr int CFL_THREADS = 256;
+constexpr int CFL_ITEMS = 8;
+constexpr unsigned long long DTMIN_INIT = 0x7f7f7f7f7f7f7f7full;      // large positive
+__global__ void __launch_bounds__(CFL_THREADS) k_cfl(int64_t n, DevCfg c, const double* d2min, const double* P,
+                                                     const double* V, const uint32_t* id, const uint64_t* keys,
+                                                     int key_shift, unsigned long long* dtmin, int nsim, double cfl,
+                                                     double t_end, double* dt, double* t,
+                                                     unsigned long long* counters, unsigned int* ticket)
 {
     // The smallest quotient d2 / cs2 is kept as the pair (bn, bd) and compared
     // by cross-multiplication, d2 bd < bn cs2 (both sides positive): two FP64
     // multiplications per particle instead of a division, which is a sequence
     // of FP64 operations on a GPU with little FP64 throughput.  The one
-    // division comes at the end, per warp.  (The comparison rounds: between
-    // two quotients within a few ulp either may win, far inside the accuracy
-    // the step's Delta t is held to.)
+    // division comes at the end.  (The comparison rounds: between two quotients
+    // within a few ulp either may win, far inside the accuracy the step's
+    // Delta t is held to.)
     // The tests compare the bit patterns as integers: for doubles that are
     // not negative and not NaN the order of the patterns is the order of the
     // values, and an integer comparison does not occupy the FP64 units
     // (finite positive values below 2^1024 have patterns below 0x7ff0...).
     constexpr long long INF_BITS = 0x7ff0000000000000ll;
     double bn = INFINITY, bd = 1.0;
+    const bool many = c.nsim_max > 1;
     uint32_t sim = 0;
-    bool many = c.nsim_max > 1;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        if (many) sim = (uint32_t)(keys[i] >> key_shift);
+    bool any = false;
+    auto put = [&] {
+        const double best = bn / bd;
+        if (best >= 0.0 && best < INFINITY) atomicMin(dtmin + sim, (unsigned long long)__double_as_longlong(best));
+    };
+    const int64_t step = many ? CFL_THREADS : (int64_t)gridDim.x * CFL_THREADS;
+    const int64_t first = (many ? blockIdx.x * (int64_t)(CFL_THREADS * CFL_ITEMS) : blockIdx.x * (int64_t)CFL_THREADS)
+                          + threadIdx.x;
+    const int64_t end = many ? min(n, (blockIdx.x + (int64_t)1) * (CFL_THREADS * CFL_ITEMS)) : n;
+    for (int64_t i = first; i < end; i += step) {
+        if (many) {
+            const uint32_t si = (uint32_t)(keys[i] >> key_shift);
+            if (any && si != sim) {
+                put();
+                bn = INFINITY;
+                bd = 1.0;
+            }
+            sim = si;
+        }
+        any = true;
         const double d2 = d2min[i];
         const long long d2b = __double_as_longlong(d2);
         // fluid, 0 <= d2 < inf (-0 has the sign bit and is left out with the negatives)
@@ -177,45 +231,50 @@ __global__ void k_cfl(int64_t n, DevCfg c, const double* d2min, const double* P,
             if (cb > 0 && cb < INF_BITS &&
                 __double_as_longlong(d2 * bd) < __double_as_longlong(bn * cs2)) { bn = d2; bd = cs2; }
         }
-        if (many) break;
     }
-    uint32_t s0 = __shfl_sync(0xffffffffu, sim, 0);
-    if (__all_sync(0xffffffffu, sim == s0)) {
+    // over the block, when its threads end in one simulation
+    __shared__ double sn[CFL_THREADS / 32], sd[CFL_THREADS / 32];
+    __shared__ uint32_t ssim;
+    __shared__ bool last_block;
+    const int lane = (int)(threadIdx.x & 31u), wid = (int)(threadIdx.x >> 5);
+    if (threadIdx.x == 0) ssim = sim;
+    __syncthreads();
+    const bool one = __syncthreads_and(!any || sim == ssim);
+    if (one) {
         for (int o = 16; o > 0; o >>= 1) {
             const double on = __shfl_xor_sync(0xffffffffu, bn, o), od = __shfl_xor_sync(0xffffffffu, bd, o);
             if (__double_as_longlong(on * bd) < __double_as_longlong(bn * od)) { bn = on; bd = od; }
         }
-        if ((threadIdx.x & 31) != 0) return;
+        if (lane == 0) { sn[wid] = bn; sd[wid] = bd; }
+    } else if (any) {
+        put();
     }
-    const double best = bn / bd;
-    if (best >= 0.0 && best < INFINITY) atomicMin(dtmin + sim, (unsigned long long)__double_as_longlong(best));
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        if (one) {
+            for (int q = 1; q < CFL_THREADS / 32; ++q)
+                if (__double_as_longlong(sn[q] * bd) < __double_as_longlong(bn * sd[q])) { bn = sn[q]; bd = sd[q]; }
+            put();
+        }
+        __threadfence();
+        last_block = atomicAdd(ticket, 1u) == gridDim.x - 1u;
+    }
+    __syncthreads();
+    if (!last_block) return;
+    __threadfence();
+    for (int q = threadIdx.x; q < nsim; q += CFL_THREADS) {
+        const unsigned long long m = __ldcg(dtmin + q);
+        dtmin[q] = DTMIN_INIT;
+        dt_finalize(q, cfl, 0.0, t_end, m, dt, t, counters);
+    }
+    if (threadIdx.x == 0) *ticket = 0u;
 }
 
-__global__ void k_dt_finalize(int nsim, double cfl, double dt_fixed, double t_end, const unsigned long long* dtmin,
-                              double* dt, double* t, unsigned long long* counters)
+__global__ void k_dt_fixed(int nsim, double dt_fixed, double t_end, double* dt, double* t,
+                           unsigned long long* counters)
 {
-    int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= nsim) return;
-    double v;
-    if (dt_fixed > 0.0) v = dt_fixed;
-    else v = cfl * sqrt(__longlong_as_double((long long)dtmin[s]));
-    if (!(v > 0.0) || isinf(v) || isnan(v)) {
-        atomicOr(reinterpret_cast<unsigned int*>(counters + C_STATUS), ST_NONFINITE);
-        v = 0.0;
-    }
-    // the last step ends at t_end (a simulation already there does not move)
-    if (t && t_end > 0.0) {
-        const double rem = fmax(__dsub_rn(t_end, t[s]), 0.0);
-        if (v >= rem) {
-            dt[s] = rem;
-            t[s] = fmax(t[s], t_end);
-            if (s == 0) counters[C_STEPS] += 1;
-            return;
-        }
-    }
-    dt[s] = v;
-    if (t) t[s] += v;
-    if (s == 0) counters[C_STEPS] += 1;
+    const int s = blockIdx.x * blockDim.x + threadIdx.x;
+    if (s < nsim) dt_finalize(s, 0.0, dt_fixed, t_end, 0ull, dt, t, counters);
 }
 
 void fill_fit_args(lp_ctx* c, FitArgs& a, int64_t n)
@@ -295,17 +354,17 @@ namespace lp {
 
 cudaError_t run_cfl(lp_ctx* c, int64_t n, double cfl, double dt_fixed, double* t, cudaStream_t s)
 {
-    int nsim = c->nsim;
-    cudaError_t e = cudaMemsetAsync(c->dt_min, 0x7f, sizeof(unsigned long long) * nsim, s);   // large positive
-    if (e != cudaSuccess) return e;
-    if (dt_fixed <= 0.0 && n > 0) {
-        int64_t nb_ = (n + 255) / 256;
-        unsigned blocks = nsim > 1 ? (unsigned)nb_ : (unsigned)(nb_ < 152 * 8 ? nb_ : 152 * 8);
-        k_cfl<<<blocks, 256, 0, s>>>(n, c->dc, c->nb_d2min, c->sP, c->sV, c->sid, c->keys_sorted,
-                                     c->dc.dim * c->dc.mbits, c->dt_min);
+    const int nsim = c->nsim;
+    if (dt_fixed > 0.0) {
+        k_dt_fixed<<<(unsigned)((nsim + 127) / 128), 128, 0, s>>>(nsim, dt_fixed, c->cfg.t_end, c->dt_dev, t, c->counters);
+        return cudaGetLastError();
     }
-    k_dt_finalize<<<(unsigned)((nsim + 127) / 128), 128, 0, s>>>(nsim, cfl, dt_fixed, c->cfg.t_end, c->dt_min,
-                                                                c->dt_dev, t, c->counters);
+    const int64_t per = c->dc.nsim_max > 1 ? CFL_THREADS * CFL_ITEMS : CFL_THREADS;
+    const int64_t nb_ = n > 0 ? (n + per - 1) / per : 1;
+    const unsigned blocks = (unsigned)(c->dc.nsim_max > 1 || nb_ < 152 * 8 ? nb_ : 152 * 8);
+    k_cfl<<<blocks, CFL_THREADS, 0, s>>>(n, c->dc, c->nb_d2min, c->sP, c->sV, c->sid, c->keys_sorted,
+                                         c->dc.dim * c->dc.mbits, c->dt_min, nsim, cfl, c->cfg.t_end, c->dt_dev, t,
+                                         c->counters, c->tickets + 1);
     return cudaGetLastError();
 }
 
@@ -320,18 +379,20 @@ lp_status run_fit(lp_ctx* c, FitArgs a, const StepOut& o, int sched, cudaStream_
 {
     const bool split = (sched & LP_SCHED_SPLIT) != 0;
     const int dim = c->dc.dim;
-    if (split) LP_CUDA(cudaMemsetAsync(c->counters + C_PLAIN_LEN, 0, 8, s));
+    const bool fresh = c->fresh_fit != 0;       // the build zeroed the lists' lengths and counters
+    c->fresh_fit = 0;
+    a.fresh = fresh ? 1 : 0;
+    if (split && !fresh) LP_CUDA(cudaMemsetAsync(c->counters + C_PLAIN_LEN, 0, 8, s));
     // with no learned gate every fitted particle takes the plain stage: its
-    // slot is its index, and the plain kernel keeps the key order (slots of
-    // particles without a plain stage stay all ones)
+    // slot is its index, and the plain kernel keeps the key order (the central
+    // kernel sets the slots of particles without a plain stage to all ones)
     if (split && !o.features && c->dc.estimator != LP_EST_MLP && a.n > 0) {
         a.plain_ident = 1;
-        LP_CUDA(cudaMemsetAsync(c->plain_list, 0xff, (size_t)a.n * 4, s));
     }
     if (c->dc.precision == LP_PREC_FP32) {
-        LP_CUDA(cudaMemsetAsync(c->counters + C_REDO_LEN, 0, 8, s));
+        if (!fresh) LP_CUDA(cudaMemsetAsync(c->counters + C_REDO_LEN, 0, 8, s));
         const bool defer = split && c->dc.refine == LP_REFINE_AUTO;
-        if (defer) LP_CUDA(cudaMemsetAsync(c->counters + C_REFINE_LEN, 0, 8, s));
+        if (defer && !fresh) LP_CUDA(cudaMemsetAsync(c->counters + C_REFINE_LEN, 0, 8, s));
         {
             Phase ph(c, LP_PH_FIT, split ? (defer ? 3 : 2) : 1, s);
             if (split && (sched & LP_SCHED_QUEUE_FIT)) LP_CUDA(launch_step_split_queue_f32(dim, a, o, s));
@@ -448,7 +509,7 @@ lp_status lp_create(const lp_config* cfg, lp_ctx** out)
     A(dalloc(&c->grid, sizeof(Grid) * ns)); A(dalloc(&c->dt_dev, 8 * ns));
     A(dalloc(&c->dt_min, 8 * ns)); A(dalloc(&c->ext, 64 * (size_t)ns)); A(dalloc(&c->grange, 8));
     A(dalloc(&c->level_off_dev, sizeof(int64_t) * (MAX_LEVELS + 1)));
-    A(dalloc(&c->counters, C_COUNT * 8));
+    A(dalloc(&c->counters, C_COUNT * 8)); A(dalloc(&c->tickets, 2 * sizeof(unsigned int)));
     A(dalloc(&c->mlp_master, MLP_NPARAM * 4)); A(dalloc(&c->mlp_bf16, MLP_NPARAM * 2));
     A(dalloc(&c->mlp_m1, MLP_NPARAM * 4)); A(dalloc(&c->mlp_m2, MLP_NPARAM * 4));
     A(dalloc(&c->mlp_grad, MLP_NPARAM * 4)); A(dalloc(&c->mlp_work, MLP_WORK * sizeof(float)));
@@ -456,6 +517,10 @@ lp_status lp_create(const lp_config* cfg, lp_ctx** out)
         A(cudaMemset(c->cells, 0, (size_t)c->table_entries * 8));
         A(cudaMemset(c->counters, 0, C_COUNT * 8));
         A(cudaMemset(c->dt_dev, 0, 8 * ns));
+        A(cudaMemset(c->dt_min, 0x7f, 8 * (size_t)ns));      // (every k_cfl and k_begin puts its words back)
+        A(cudaMemset(c->tickets, 0, 2 * sizeof(unsigned int)));
+        A(sort_init());
+        A(init_extent(c, nullptr));
         A(cudaMemcpy(c->level_off_dev, c->level_off, sizeof(int64_t) * (MAX_LEVELS + 1), cudaMemcpyHostToDevice));
         for (int q = 0; q < 2 * EV_PAIRS && ok; ++q) A(cudaEventCreate(&c->ev[q]));
         A(cudaDeviceSynchronize());
@@ -514,20 +579,21 @@ static lp_status build(lp_ctx* c, lp_particles* p, cudaStream_t s)
 {
     int64_t n = p->n;
     bool tables = c->dc.dim > 1;
-    if (c->tables_dirty) {   // clear the previous build's table entries
-        Phase ph(c, LP_PH_TABLES, tables && c->n_lists > 0 ? 1 : 0, s);
-        LP_CUDA(fill_tables(c, c->n_lists, true, s));
-        c->tables_dirty = 0;
-    }
+    const int64_t n_old = c->tables_dirty ? c->n_lists : 0;   // the previous build's table entries are cleared first
+    c->tables_dirty = 0;
     c->n_lists = 0;
     c->lists_stale = 0;
-    if (n == 0) return LP_OK;
-    {
-        Phase ph(c, LP_PH_GRID, 4 + (c->nsim > 1 ? 1 : 0), s);
-        LP_CUDA(build_grid(c, p, s));
-        LP_CUDA(make_keys(c, p, s));
+    if (n == 0) {
+        Phase ph(c, LP_PH_TABLES, tables && n_old > 0 ? 1 : 0, s);
+        LP_CUDA(fill_tables(c, n_old, true, s));
+        return LP_OK;
     }
+    const bool small = front_is_small(c, n);
     {
+        Phase ph(c, LP_PH_GRID, front_launches(c, n), s);
+        LP_CUDA(build_front(c, p, n_old, s));
+    }
+    if (!small) {
         Phase ph(c, LP_PH_SORT, 3 * radix_passes(c), s);
         LP_CUDA(radix_sort(c, n, s));
     }
@@ -700,7 +766,7 @@ lp_status step_prologue(lp_ctx* c, lp_particles* p, const int64_t* offsets, int3
     if (st != LP_OK) return st;
     int64_t n = p->n;
     {
-        Phase ph(c, LP_PH_CFL, (dt <= 0.0 && n > 0) ? 2 : 1, s);
+        Phase ph(c, LP_PH_CFL, 1, s);
         LP_CUDA(run_cfl(c, n, cfl, dt, t, s));
     }
     if (n == 0) return LP_OK;

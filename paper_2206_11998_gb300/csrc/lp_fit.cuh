@@ -361,6 +361,7 @@ struct FitArgs {
     void* mid;
     int64_t mid_cap;
     int plain_ident;
+    int fresh;                // the queue's counters are zero
     // split schedule, FP32: the central fits that need the correction pass,
     // listed by the first kernel for a kernel of their own
     uint32_t* refine_list;

@@ -26,8 +26,8 @@ cudaError_t split_queue(const FitArgs& a, const StepOut& o, cudaStream_t s)
     const unsigned bc = resident_grid(k_step_central_q<float, DIM, GATE, DEFER>, FIT_THREADS);
     const unsigned bp = resident_grid(k_step_plain_q<float, DIM>, FIT_THREADS);
     if (bc == 0 || bp == 0) return cudaErrorInvalidConfiguration;
-    cudaError_t e = cudaMemsetAsync(a.queue, 0, 2 * sizeof(unsigned long long), s);
-    if (e != cudaSuccess) return e;
+    cudaError_t e = cudaSuccess;
+    if (!a.fresh && (e = cudaMemsetAsync(a.queue, 0, 2 * sizeof(unsigned long long), s)) != cudaSuccess) return e;
     k_step_central_q<float, DIM, GATE, DEFER><<<bc, FIT_THREADS, 0, s>>>(a, o);
     if (DEFER) {
         FitArgs r = a;

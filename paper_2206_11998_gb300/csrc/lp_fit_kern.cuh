@@ -469,6 +469,8 @@ __device__ __forceinline__ void central_one(const FitArgs& a, const StepOut& o, 
 {
     constexpr int F = DIM + 2;
     Loaded<DIM> L;
+    // (overwritten below, or by the correction kernel, where there is a plain stage)
+    if (a.plain_ident) a.plain_list[i] = 0xffffffffu;
     if (step_load<T, DIM>(a, o, i, L)) return;
     Src<T, DIM, F> src(a, i);
     const int cnt = (int)a.count[i];

@@ -287,6 +287,8 @@ struct lp_ctx {
     double* dt_dev;               // one per simulation
     unsigned long long* dt_min;   // per simulation: bit pattern of min(d2 / c^2)
     unsigned long long* ext;      // per simulation: 8 extent words
+    unsigned int* tickets;        // [2] blocks done, of kernels whose last block finishes up (zero between launches)
+    int fresh_query, fresh_fit;   // the build's lengths and counters are zero: not yet used by a query, a fit pass
     int* grange;                  // [2] table levels in use over all simulations
     int64_t* level_off_dev;
     uint32_t* sim_of;             // simulation of each particle (input order)
@@ -348,8 +350,11 @@ struct lp_ctx {
 
 namespace lp {
 // launchers implemented in the .cu files
-cudaError_t build_grid(lp_ctx* c, const lp_particles* p, cudaStream_t s);
-cudaError_t make_keys(lp_ctx* c, const lp_particles* p, cudaStream_t s);
+cudaError_t sort_init();                                  // kernel attributes on the current device
+cudaError_t init_extent(lp_ctx* c, cudaStream_t s);      // once per context
+bool front_is_small(const lp_ctx* c, int64_t n);          // build_front sorts as well
+int front_launches(const lp_ctx* c, int64_t n);
+cudaError_t build_front(lp_ctx* c, const lp_particles* p, int64_t n_old, cudaStream_t s);
 int radix_passes(const lp_ctx* c);
 cudaError_t radix_sort(lp_ctx* c, int64_t n, cudaStream_t s);
 cudaError_t gather(lp_ctx* c, const lp_particles* p, cudaStream_t s);

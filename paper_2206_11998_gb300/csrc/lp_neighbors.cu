@@ -2087,8 +2087,10 @@ cudaError_t query_neighbors(lp_ctx* c, int64_t n, cudaStream_t s)
         return cudaGetLastError();
     }
     static_assert(C_GROUP_LEN == C_QFB_LEN + 1, "one memset for both lengths");
-    cudaError_t e = cudaMemsetAsync(c->counters + C_QFB_LEN, 0, 16, s);
-    if (e != cudaSuccess) return e;
+    cudaError_t e = cudaSuccess;
+    const bool fresh = c->fresh_query != 0;       // the build zeroed the lengths and the counter
+    c->fresh_query = 0;
+    if (!fresh && (e = cudaMemsetAsync(c->counters + C_QFB_LEN, 0, 16, s)) != cudaSuccess) return e;
     const bool octant = c->dc.select == LP_SELECT_OCTANT;
     if (c->schedule & LP_SCHED_QUERY_WARP) {   // one warp per particle for every particle
         const unsigned wb = (unsigned)((n + NB_WARPS - 1) / NB_WARPS);
@@ -2107,7 +2109,7 @@ cudaError_t query_neighbors(lp_ctx* c, int64_t n, cudaStream_t s)
     const bool queue = (c->schedule & LP_SCHED_QUEUE_QUERY) != 0;
     if (queue) {
         a.queue = c->counters + C_QUEUE_TILE;
-        if ((e = cudaMemsetAsync(a.queue, 0, 8, s)) != cudaSuccess) return e;
+        if (!fresh && (e = cudaMemsetAsync(a.queue, 0, 8, s)) != cudaSuccess) return e;
     }
     if (dim == 3) e = per ? launch_tiles<3, true>(a, queue, s) : launch_tiles<3, false>(a, queue, s);
     else e = per ? launch_tiles<2, true>(a, queue, s) : launch_tiles<2, false>(a, queue, s);

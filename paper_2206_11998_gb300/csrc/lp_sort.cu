@@ -156,19 +156,89 @@ __device__ __forceinline__ void block_w_extent(bool valid, double w, uint32_t si
     }
 }
 
-// ext[8 s + 0..2] min x_k, [8 s + 3..5] max x_k (order keys) of simulation s
-// (the extent of m V, ext[8 s + 6..7], is taken by the gather, which reads m
-// and V anyway: the keys need only the positions).  One simulation:
-// grid-stride accumulation and a warp reduction; several: EXT_ITEMS particles
-// per thread, reduced over the warp when the warp's particles share a
-// simulation (they are stored by simulation), with atomics per run otherwise.
-// The comparisons are integer ones on the order keys (FP64 min / max would
-// run on the scarce FP64 units).
-template <int DIM>
-__global__ void k_reduce_extent(int64_t n, const double* __restrict__ x0,
-                                const double* __restrict__ x1, const double* __restrict__ x2,
-                                const uint32_t* __restrict__ sim_of, unsigned long long* ext)
+__global__ void k_init_extent(unsigned long long* ext, int nsim)
 {
+    int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t < 8 * nsim) {
+        int w = t & 7;
+        ext[t] = (w < 3 || w == 6) ? ~0ull : 0ull;
+    }
+}
+
+// Bounding cube of a simulation (what the keys need) from its extent lo, hi
+// (order keys).
+__device__ inline void finalize_cube(const DevCfg& c, const unsigned long long (&lo)[3],
+                                     const unsigned long long (&hi)[3], Grid* g)
+{
+    double L = 0.0, org[3] = {0.0, 0.0, 0.0};
+    for (int k = 0; k < c.dim; ++k) {
+        double ext_k;
+        if (c.periodic[k]) { org[k] = c.box_lo[k]; ext_k = c.Lper[k]; }
+        else { org[k] = from_order_key(lo[k]); ext_k = __dsub_rn(from_order_key(hi[k]), org[k]); }
+        L = fmax(L, ext_k);
+    }
+    if (!(L > 0.0)) L = 1.0;
+    g->L = L;
+    g->inv = __ddiv_rn(ldexp(1.0, c.mbits), L);
+    for (int k = 0; k < 3; ++k) {
+        g->lo[k] = org[k];
+        split(org[k], g->lo_h[k], g->lo_l[k]);
+    }
+    g->inv_f = (float)g->inv;
+    g->L_f = (float)L;
+}
+
+// one particle's entries of the cell tables (see k_tables)
+struct TableArgs {
+    int dim, mbits;
+    int64_t n;                    // 0: no tables
+    const uint64_t* keys;
+    const int* grange;
+    const int64_t* level_off;
+    unsigned long long* cells;
+};
+template <bool CLEAR>
+__device__ __forceinline__ void table_entries(const TableArgs& a, int64_t i)
+{
+    const uint64_t k = a.keys[i];
+    const uint64_t kp = i > 0 ? a.keys[i - 1] : 0;
+    const uint64_t kn = i + 1 < a.n ? a.keys[i + 1] : 0;
+    uint32_t* half = reinterpret_cast<uint32_t*>(a.cells);
+    for (int l = a.grange[0]; l <= a.grange[1]; ++l) {
+        const int sh = a.dim * (a.mbits - l);
+        const uint64_t c = k >> sh;
+        const bool first = i == 0 || (kp >> sh) != c;
+        const int64_t e = a.level_off[l] + (int64_t)c;
+        if (CLEAR) {
+            if (first) a.cells[e] = 0ull;
+        } else {
+            const bool last = i + 1 == a.n || (kn >> sh) != c;
+            if (first) half[2 * e] = (uint32_t)i;
+            if (last) half[2 * e + 1] = (uint32_t)(i + 1);
+        }
+    }
+}
+
+// The start of a build: the last build's table entries cleared (old), and the
+// extent of the positions, ext[8 s + 0..2] min x_k, [8 s + 3..5] max x_k (order
+// keys) of simulation s, from which the last block to finish forms the bounding
+// cubes (the extent of m V, ext[8 s + 6..7], is taken by the gather, which
+// reads m and V anyway: the keys need only the positions).  The extent words
+// are at their initial values on entry and are put back for the next build.
+// One simulation: grid-stride accumulation and a warp reduction; several:
+// EXT_ITEMS particles per thread, reduced over the warp when the warp's
+// particles share a simulation (they are stored by simulation), with atomics
+// per run otherwise.  The comparisons are integer ones on the order keys (FP64
+// min / max would run on the scarce FP64 units).  As kernels of their own the
+// clearing, the words' initialisation and the cubes cost a launch each (2 to 3
+// us, and as much between launches).
+template <int DIM>
+__global__ void k_begin(int64_t n, const double* __restrict__ x0, const double* __restrict__ x1,
+                        const double* __restrict__ x2, const uint32_t* __restrict__ sim_of, unsigned long long* ext,
+                        DevCfg c, int nsim, Grid* grids, unsigned int* ticket, TableArgs old)
+{
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < old.n; i += (int64_t)gridDim.x * blockDim.x)
+        table_entries<true>(old, i);
     ExtKeys r;
     r.init();
     const double* const xs[3] = {x0, x1, x2};
@@ -220,103 +290,113 @@ __global__ void k_reduce_extent(int64_t n, const double* __restrict__ x0,
         for (int k = 0; k < DIM; ++k) { slo[wid][k] = r.lo[k]; shi[wid][k] = r.hi[k]; }
     }
     __syncthreads();
-    if (threadIdx.x != 0) return;
-    const int nw = (int)((blockDim.x + 31) / 32);
-    uint32_t sb = 0xffffffffu;
-    bool one = true;
-    for (int q = 0; q < nw; ++q) {
-        const uint32_t sq = ssim[q];
-        if (sq == 0xffffffffu) continue;                    // no particle
-        if (sq == 0xfffffffeu || (sb != 0xffffffffu && sq != sb)) { one = false; break; }
-        sb = sq;
-    }
-    for (int q = 0; q < nw; ++q) {
-        const uint32_t sq = ssim[q];
-        if (sq >= 0xfffffffeu) continue;
-        ExtKeys t;
-        t.init();
-#pragma unroll
-        for (int k = 0; k < DIM; ++k) { t.lo[k] = slo[q][k]; t.hi[k] = shi[q][k]; }
-        if (one) {
-            // merge every warp into the first, flushed once at the end
-            for (int q2 = q + 1; q2 < nw; ++q2) {
-                if (ssim[q2] != sb) continue;
-#pragma unroll
-                for (int k = 0; k < DIM; ++k) {
-                    t.lo[k] = slo[q2][k] < t.lo[k] ? slo[q2][k] : t.lo[k];
-                    t.hi[k] = shi[q2][k] > t.hi[k] ? shi[q2][k] : t.hi[k];
-                }
-            }
-            t.flush<DIM>(ext + 8 * (int64_t)sb);
-            break;
+    if (threadIdx.x == 0) {
+        const int nw = (int)((blockDim.x + 31) / 32);
+        uint32_t sb = 0xffffffffu;
+        bool one = true;
+        for (int q = 0; q < nw; ++q) {
+            const uint32_t sq = ssim[q];
+            if (sq == 0xffffffffu) continue;                    // no particle
+            if (sq == 0xfffffffeu || (sb != 0xffffffffu && sq != sb)) { one = false; break; }
+            sb = sq;
         }
-        t.flush<DIM>(ext + 8 * (int64_t)sq);
+        for (int q = 0; q < nw; ++q) {
+            const uint32_t sq = ssim[q];
+            if (sq >= 0xfffffffeu) continue;
+            ExtKeys t;
+            t.init();
+    #pragma unroll
+            for (int k = 0; k < DIM; ++k) { t.lo[k] = slo[q][k]; t.hi[k] = shi[q][k]; }
+            if (one) {
+                // merge every warp into the first, flushed once at the end
+                for (int q2 = q + 1; q2 < nw; ++q2) {
+                    if (ssim[q2] != sb) continue;
+    #pragma unroll
+                    for (int k = 0; k < DIM; ++k) {
+                        t.lo[k] = slo[q2][k] < t.lo[k] ? slo[q2][k] : t.lo[k];
+                        t.hi[k] = shi[q2][k] > t.hi[k] ? shi[q2][k] : t.hi[k];
+                    }
+                }
+                t.flush<DIM>(ext + 8 * (int64_t)sb);
+                break;
+            }
+            t.flush<DIM>(ext + 8 * (int64_t)sq);
+        }
     }
+    // the last block: every block's words are in
+    __shared__ bool last_block;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        last_block = atomicAdd(ticket, 1u) == gridDim.x - 1u;
+    }
+    __syncthreads();
+    if (!last_block) return;
+    __threadfence();
+    for (int q = threadIdx.x; q < nsim; q += blockDim.x) {
+        unsigned long long* e = ext + 8 * (int64_t)q;
+        unsigned long long lo[3], hi[3];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) { lo[k] = __ldcg(e + k); hi[k] = __ldcg(e + 3 + k); }
+#pragma unroll
+        for (int k = 0; k < 3; ++k) { e[k] = ~0ull; e[3 + k] = 0ull; }
+        e[6] = ~0ull;
+        e[7] = 0ull;
+        finalize_cube(c, lo, hi, grids + q);
+    }
+    if (threadIdx.x == 0) *ticket = 0u;
 }
 
-__global__ void k_init_extent(unsigned long long* ext, int nsim)
-{
-    int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t < 8 * nsim) {
-        int w = t & 7;
-        ext[t] = (w < 3 || w == 6) ? ~0ull : 0ull;
-    }
-}
+// floor(log2(v)) of a positive normal value
+__device__ __forceinline__ int exponent_of(double v) { return (int)((__double_as_longlong(v) >> 52) & 0x7ff) - 1023; }
 
-// Bounding cube of each simulation (what the keys need).
-__global__ void k_finalize_cube(DevCfg c, int nsim, const unsigned long long* ext_all, Grid* grids)
+// floor(log2(A / r)) for the radius r = (k^dim w)^(1/dim): with q = A^dim / (k^dim w)
+// it is floor(floor(log2 q) / dim), so the exponent of q gives it (FP64 pow and
+// log2 took a single block 11 us).  Outside the range where the powers are
+// normal numbers, the functions.
+__device__ inline int level_of(int dim, double A, double k, double w)
 {
-    int sim = blockIdx.x * blockDim.x + threadIdx.x;
-    if (sim >= nsim) return;
-    const unsigned long long* ext = ext_all + 8 * sim;
-    Grid* g = grids + sim;
-    double L = 0.0;
-    for (int k = 0; k < c.dim; ++k) {
-        double lo, ext_k;
-        if (c.periodic[k]) { lo = c.box_lo[k]; ext_k = c.Lper[k]; }
-        else { lo = from_order_key(ext[k]); ext_k = __dsub_rn(from_order_key(ext[3 + k]), lo); }
-        g->lo[k] = lo;
-        L = fmax(L, ext_k);
-    }
-    for (int k = c.dim; k < 3; ++k) g->lo[k] = 0.0;
-    if (!(L > 0.0)) L = 1.0;
-    g->L = L;
-    g->inv = __ddiv_rn(ldexp(1.0, c.mbits), L);
-    for (int k = 0; k < 3; ++k) split(g->lo[k], g->lo_h[k], g->lo_l[k]);
-    g->inv_f = (float)g->inv;
-    g->L_f = (float)L;
+    double a = A, b = k;
+    for (int d = 1; d < dim; ++d) { a *= A; b *= k; }
+    const double q = a / (b * w);
+    if (!(q >= 0x1p-1000) || !(q <= 0x1p1000) || !(a <= 0x1p1000) || !(a >= 0x1p-1000) || !(b * w >= 0x1p-1000))
+        return (int)floor(log2(A / (k * pow(w, 1.0 / dim))));
+    const int e = exponent_of(q);
+    return e >= 0 ? e / dim : -((dim - 1 - e) / dim);
 }
 
 // The range of cell levels of each simulation, and over all of them (one
 // block).  lmin is the finest level whose cell edge L / 2^l is at least the
 // largest radius present; lmax the finest whose edge is at least half the
-// smallest radius (the queries use cells down to half a radius).
+// smallest radius (the queries use cells down to half a radius).  Also zeroes
+// the lengths and work counters of the query and the fit pass that follow
+// (fresh_query, fresh_fit: they need no memsets of their own).
 constexpr int LEVEL_THREADS = 256;
 __global__ void __launch_bounds__(LEVEL_THREADS) k_finalize_levels(DevCfg c, int lmax_cap, int nsim,
                                                                    const unsigned long long* ext_all, Grid* grids,
-                                                                   int* grange)
+                                                                   int* grange, unsigned long long* counters)
 {
     __shared__ int slo[LEVEL_THREADS], shi[LEVEL_THREADS];
+    if (threadIdx.x < 8) {
+        const int zero[8] = {C_QFB_LEN, C_GROUP_LEN, C_QUEUE_TILE, C_REDO_LEN, C_PLAIN_LEN, C_REFINE_LEN,
+                             C_QUEUE_CENTRAL, C_QUEUE_PLAIN};
+        counters[zero[threadIdx.x]] = 0ull;
+    }
     int lo_all = 1 << 20, hi_all = 0;
     for (int sim = threadIdx.x; sim < nsim; sim += LEVEL_THREADS) {
         const unsigned long long* ext = ext_all + 8 * sim;
         Grid* g = grids + sim;
         const double L = g->L;
-        double rmin, rmax;
-        if (c.radius_mode == LP_RADIUS_FIXED) { rmin = rmax = c.radius; }
-        else {
-            double wlo = from_order_key(ext[6]), whi = from_order_key(ext[7]);
-            rmin = c.kappa * pow(wlo, 1.0 / c.dim);
-            rmax = c.kappa * pow(whi, 1.0 / c.dim);
-        }
-        // margins wider than the per-particle float radius margin (1e-5) keep every
-        // particle's level inside [lmin, lmax]
-        rmin *= 1.0 - 1e-4;
-        rmax *= 1.0 + 1e-4;
-        if (!(rmin > 0.0)) rmin = L * ldexp(1.0, -lmax_cap);   // empty or degenerate simulation
-        if (!(rmax > 0.0) || isinf(rmax)) rmax = L;
-        int lmax = (int)floor(log2(2.0 * L / rmin));
-        int lmin = (int)floor(log2(L / rmax));
+        const bool fixed = c.radius_mode == LP_RADIUS_FIXED;
+        // the radius is k w^(1/dim), the fixed one with w = 1.  Margins wider than
+        // the per-particle float radius margin (1e-5) keep every particle's level
+        // inside [lmin, lmax]
+        const double k = fixed ? c.radius : c.kappa;
+        const double wlo = fixed ? 1.0 : from_order_key(ext[6]), whi = fixed ? 1.0 : from_order_key(ext[7]);
+        const bool some = wlo > 0.0 && k > 0.0, bounded = whi > 0.0 && k > 0.0 && !isinf(whi) && !isinf(k);
+        int lmax = some ? level_of(c.dim, 2.0 * L, k * (1.0 - 1e-4), wlo)
+                        : lmax_cap + 1;               // empty or degenerate simulation: the finest
+        int lmin = bounded ? level_of(c.dim, L, k * (1.0 + 1e-4), whi) : 0;
         lmax = max(0, min(lmax, lmax_cap));
         lmin = max(0, min(lmin, lmax));
         g->lmax = lmax;
@@ -340,7 +420,26 @@ __global__ void __launch_bounds__(LEVEL_THREADS) k_finalize_levels(DevCfg c, int
     }
 }
 
-// key = simulation << (DIM mbits) | Morton code of the quantised position
+// key = simulation << (DIM mbits) | Morton code of the quantised position (1D:
+// the order key of x)
+template <int DIM>
+__device__ __forceinline__ uint64_t key_of(const double* const (&xs)[3], int64_t i, const Grid* g, uint32_t sim, int mbits)
+{
+    if (DIM == 1) return order_key(xs[0][i]);
+    const double inv = g->inv;
+    const uint32_t qmax = (1u << mbits) - 1u;
+    uint32_t q[3] = {0, 0, 0};
+#pragma unroll
+    for (int k = 0; k < DIM; ++k) {
+        // floor(t) clamped to [0, qmax] (negative and NaN give 0, +inf gives
+        // qmax), read from t's bits: the conversion instruction would run on
+        // the FP64 units, which the subtraction and the product already keep busy
+        const double t = __dmul_rn(__dsub_rn(xs[k][i], g->lo[k]), inv);
+        q[k] = floor_clamped(t, qmax);
+    }
+    return ((uint64_t)sim << (DIM * mbits)) | morton<DIM>(q);
+}
+
 template <int DIM>
 __global__ void k_keys(int64_t n, const double* __restrict__ x0, const double* __restrict__ x1,
                        const double* __restrict__ x2, const Grid* __restrict__ grids,
@@ -349,29 +448,13 @@ __global__ void k_keys(int64_t n, const double* __restrict__ x0, const double* _
 {
     int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= n) return;
-    if (DIM == 1) {
-        keys[i] = order_key(x0[i]);
-        vals[i] = (uint32_t)i;
-        return;
-    }
     const double* xs[3] = {x0, x1, x2};
-    uint32_t sim = sim_of ? sim_of[i] : 0u;
-    const Grid* g = grids + sim;
-    double inv = g->inv;
-    const uint32_t qmax = (1u << mbits) - 1u;
-    uint32_t q[3] = {0, 0, 0};
-    for (int k = 0; k < DIM; ++k) {
-        // floor(t) clamped to [0, qmax] (negative and NaN give 0, +inf gives
-        // qmax), read from t's bits: the conversion instruction would run on
-        // the FP64 units, which the subtraction and the product already keep busy
-        const double t = __dmul_rn(__dsub_rn(xs[k][i], g->lo[k]), inv);
-        q[k] = floor_clamped(t, qmax);
-    }
-    keys[i] = ((uint64_t)sim << (DIM * mbits)) | morton<DIM>(q);
+    const uint32_t sim = sim_of ? sim_of[i] : 0u;
+    keys[i] = key_of<DIM>(xs, i, grids + sim, sim, mbits);
     vals[i] = (uint32_t)i;
 }
 
-// ---- LSD radix sort, 8-bit digits ----------------------------------------
+// ---- LSD radix sort, RS_BITS-bit digits ----------------------------------
 
 __global__ void k_rs_upsweep(int64_t n, const uint64_t* __restrict__ keys, int shift,
                              uint32_t* __restrict__ counts, int64_t nblocks)
@@ -505,6 +588,191 @@ k_rs_downsweep(int64_t n, const uint64_t* __restrict__ kin, const uint32_t* __re
     }
 }
 
+// The whole front of a build for one simulation of at most FS_MAX particles, by
+// one block: the last build's table entries cleared, the extent, the cube, the
+// keys and every pass of the radix sort, keys and indices in shared memory.
+// Launched one by one these are 4 + 3 launches per digit, 28 for the 64-bit keys
+// of 1D, each a few microseconds whatever n is: of a 1D step of 1000 particles
+// they were 180 of 218 us.  Keys already in order (1D particles keep theirs)
+// need no pass; with more particles than FS_MAX the passes of one SM cost more
+// than the launches of all.  The order is that of the general path: stable, by
+// the same digits.
+constexpr int FS_THREADS = 1024;
+constexpr int FS_ITEMS = 8;
+constexpr int FS_MAX = FS_THREADS * FS_ITEMS;
+constexpr int FS_WARPS = FS_THREADS / 32;
+struct FrontShared {
+    uint64_t key[FS_MAX];
+    uint16_t val[FS_MAX];
+    uint16_t wc[FS_WARPS][RS_BINS];       // per warp digit counts, then places
+    uint32_t wsum[FS_WARPS];
+    uint64_t lo[3][FS_WARPS], hi[3][FS_WARPS];
+    Grid grid;
+};
+static_assert(FS_MAX <= 65535 && RS_BINS <= FS_THREADS, "16-bit places, a thread per digit");
+
+template <int DIM>
+__global__ void __launch_bounds__(FS_THREADS) k_front_small(int n, const double* __restrict__ x0,
+                                                            const double* __restrict__ x1,
+                                                            const double* __restrict__ x2, DevCfg c, Grid* grid,
+                                                            unsigned long long* ext, TableArgs old, int lo_bit,
+                                                            int hi_bit, uint64_t* __restrict__ keys,
+                                                            uint32_t* __restrict__ vals)
+{
+    extern __shared__ __align__(16) unsigned char fs_smem[];
+    FrontShared& sm = *reinterpret_cast<FrontShared*>(fs_smem);
+    const int t = (int)threadIdx.x, w = t >> 5, lane = t & 31;
+    const unsigned lt = (1u << lane) - 1u;
+    for (int64_t i = t; i < old.n; i += FS_THREADS) table_entries<true>(old, i);
+    if (t < 2) ext[6 + t] = t == 0 ? ~0ull : 0ull;        // the gather takes the extent of m V
+    const double* const xs[3] = {x0, x1, x2};
+    ExtKeys r;
+    r.init();
+    for (int i = t; i < n; i += FS_THREADS) r.add<DIM>(xs, i);
+#pragma unroll
+    for (int k = 0; k < DIM; ++k) {
+        for (int o = 16; o > 0; o >>= 1) {
+            const uint64_t a = __shfl_xor_sync(0xffffffffu, r.lo[k], o);
+            const uint64_t b = __shfl_xor_sync(0xffffffffu, r.hi[k], o);
+            r.lo[k] = a < r.lo[k] ? a : r.lo[k];
+            r.hi[k] = b > r.hi[k] ? b : r.hi[k];
+        }
+        if (lane == 0) { sm.lo[k][w] = r.lo[k]; sm.hi[k][w] = r.hi[k]; }
+    }
+    __syncthreads();
+    if (w == 0) {
+        unsigned long long lo[3] = {~0ull, ~0ull, ~0ull}, hi[3] = {0ull, 0ull, 0ull};
+#pragma unroll
+        for (int k = 0; k < DIM; ++k) {
+            uint64_t a = sm.lo[k][lane], b = sm.hi[k][lane];
+            for (int o = 16; o > 0; o >>= 1) {
+                const uint64_t a2 = __shfl_xor_sync(0xffffffffu, a, o), b2 = __shfl_xor_sync(0xffffffffu, b, o);
+                a = a2 < a ? a2 : a;
+                b = b2 > b ? b2 : b;
+            }
+            lo[k] = a;
+            hi[k] = b;
+        }
+        if (lane == 0) {
+            finalize_cube(c, lo, hi, &sm.grid);
+            // (the levels are set after the gather)
+            for (int k = 0; k < 3; ++k) {
+                grid->lo[k] = sm.grid.lo[k];
+                grid->lo_h[k] = sm.grid.lo_h[k];
+                grid->lo_l[k] = sm.grid.lo_l[k];
+            }
+            grid->L = sm.grid.L;
+            grid->inv = sm.grid.inv;
+            grid->inv_f = sm.grid.inv_f;
+            grid->L_f = sm.grid.L_f;
+        }
+    }
+    __syncthreads();
+    // warp w holds positions [w 32 items, (w + 1) 32 items), 32 per round
+    const int items = (n + FS_THREADS - 1) / FS_THREADS;
+    const int base = w * 32 * items + lane;
+    uint64_t key[FS_ITEMS];
+    uint32_t val[FS_ITEMS];
+#pragma unroll
+    for (int q = 0; q < FS_ITEMS; ++q) {
+        const int i = base + 32 * q;
+        if (q >= items || i >= n) continue;
+        key[q] = key_of<DIM>(xs, i, &sm.grid, 0u, c.mbits);
+        val[q] = (uint32_t)i;
+        sm.key[i] = key[q];
+    }
+    __syncthreads();
+    bool sorted = true;
+#pragma unroll
+    for (int q = 0; q < FS_ITEMS; ++q) {
+        const int i = base + 32 * q;
+        if (q < items && i + 1 < n) sorted = sorted && (key[q] >> lo_bit) <= (sm.key[i + 1] >> lo_bit);
+    }
+    if (!__syncthreads_and(sorted)) {
+        for (int shift = lo_bit; shift < hi_bit; shift += RS_BITS) {
+            for (int d = lane; d < RS_BINS; d += 32) sm.wc[w][d] = 0;
+            __syncwarp();
+            uint32_t loc[FS_ITEMS];
+#pragma unroll
+            for (int q = 0; q < FS_ITEMS; ++q) {
+                if (q >= items) break;
+                const bool valid = base + 32 * q < n;
+                const uint32_t d = valid ? (uint32_t)((key[q] >> shift) & RS_MASK) : RS_BINS + lane;
+                const unsigned peers = __match_any_sync(0xffffffffu, d);
+                const bool leader = (__ffs(peers) - 1) == lane;
+                loc[q] = valid ? sm.wc[w][d] + __popc(peers & lt) : 0u;
+                __syncwarp();
+                if (valid && leader) sm.wc[w][d] += (uint16_t)__popc(peers);
+                __syncwarp();
+            }
+            __syncthreads();
+            // digit t: its warps' counts to places, after the smaller digits
+            uint32_t total = 0;
+            if (t < RS_BINS)
+                for (int u = 0; u < FS_WARPS; ++u) total += sm.wc[u][t];
+            uint32_t x = total;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+                if (lane >= o) x += y;
+            }
+            if (lane == 31) sm.wsum[w] = x;
+            __syncthreads();
+            if (t < RS_BINS) {
+                uint32_t run = x - total;
+                for (int u = 0; u < w; ++u) run += sm.wsum[u];
+                for (int u = 0; u < FS_WARPS; ++u) {
+                    const uint32_t k = sm.wc[u][t];
+                    sm.wc[u][t] = (uint16_t)run;
+                    run += k;
+                }
+            }
+            __syncthreads();
+#pragma unroll
+            for (int q = 0; q < FS_ITEMS; ++q) {
+                if (q >= items || base + 32 * q >= n) continue;
+                const uint32_t pos = sm.wc[w][(uint32_t)((key[q] >> shift) & RS_MASK)] + loc[q];
+                sm.key[pos] = key[q];
+                sm.val[pos] = (uint16_t)val[q];
+            }
+            __syncthreads();
+#pragma unroll
+            for (int q = 0; q < FS_ITEMS; ++q) {
+                const int i = base + 32 * q;
+                if (q >= items || i >= n) continue;
+                key[q] = sm.key[i];
+                val[q] = sm.val[i];
+            }
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < FS_ITEMS; ++q) {
+        const int i = base + 32 * q;
+        if (q >= items || i >= n) continue;
+        keys[i] = key[q];
+        vals[i] = val[q];
+    }
+}
+
+template <int DIM>
+cudaError_t launch_front_small(int n, const double* x0, const double* x1, const double* x2, const DevCfg& c, Grid* grid,
+                               unsigned long long* ext, const TableArgs& old, int lo_bit, int hi_bit, uint64_t* keys,
+                               uint32_t* vals, cudaStream_t s)
+{
+    k_front_small<DIM><<<1, FS_THREADS, sizeof(FrontShared), s>>>(n, x0, x1, x2, c, grid, ext, old, lo_bit, hi_bit, keys,
+                                                                  vals);
+    return cudaGetLastError();
+}
+
+cudaError_t front_small(int dim, int n, const double* x0, const double* x1, const double* x2, const DevCfg& c, Grid* grid,
+                        unsigned long long* ext, const TableArgs& old, int lo_bit, int hi_bit, uint64_t* keys,
+                        uint32_t* vals, cudaStream_t s)
+{
+    if (dim == 3) return launch_front_small<3>(n, x0, x1, x2, c, grid, ext, old, lo_bit, hi_bit, keys, vals, s);
+    if (dim == 2) return launch_front_small<2>(n, x0, x1, x2, c, grid, ext, old, lo_bit, hi_bit, keys, vals, s);
+    return launch_front_small<1>(n, x0, x1, x2, c, grid, ext, old, lo_bit, hi_bit, keys, vals, s);
+}
+
 // gather the state into key order and split it into float hi/lo pairs
 template <int DIM>
 __global__ void k_gather(int64_t n, const uint32_t* __restrict__ perm, lp_particles p, DevCfg c,
@@ -617,29 +885,11 @@ __global__ void k_gather_fields(int64_t n, const uint32_t* __restrict__ perm, lp
 }
 
 // cell tables: entry = start | end << 32 of the key-sorted particles in the cell
-__global__ void k_tables(int dim, int mbits, int64_t n, const uint64_t* __restrict__ keys,
-                         const int* __restrict__ grange, const int64_t* __restrict__ level_off,
-                         unsigned long long* cells, int clear)
+template <bool CLEAR>
+__global__ void k_tables(TableArgs a)
 {
-    int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    uint64_t k = keys[i];
-    uint64_t kp = i > 0 ? keys[i - 1] : 0;
-    uint64_t kn = i + 1 < n ? keys[i + 1] : 0;
-    uint32_t* half = reinterpret_cast<uint32_t*>(cells);
-    for (int l = grange[0]; l <= grange[1]; ++l) {
-        int sh = dim * (mbits - l);
-        uint64_t c = k >> sh;
-        bool first = i == 0 || (kp >> sh) != c;
-        bool last = i + 1 == n || (kn >> sh) != c;
-        int64_t e = level_off[l] + (int64_t)c;
-        if (clear) {
-            if (first) cells[e] = 0ull;
-        } else {
-            if (first) half[2 * e] = (uint32_t)i;
-            if (last) half[2 * e + 1] = (uint32_t)(i + 1);
-        }
-    }
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (i < a.n) table_entries<CLEAR>(a, i);
 }
 
 __global__ void k_scatter_back(int dim, int64_t n, lp_particles p, const double* sx0, const double* sx1,
@@ -676,38 +926,67 @@ __global__ void k_sim_of(int64_t n, const int64_t* __restrict__ offsets, int nsi
 
 }  // namespace
 
-cudaError_t build_grid(lp_ctx* c, const lp_particles* p, cudaStream_t s)
+cudaError_t sort_init()
 {
-    int64_t n = p->n;
-    int nsim = c->nsim;
+    const cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    cudaError_t e;
+    if ((e = cudaFuncSetAttribute(k_front_small<1>, at, (int)sizeof(FrontShared))) != cudaSuccess) return e;
+    if ((e = cudaFuncSetAttribute(k_front_small<2>, at, (int)sizeof(FrontShared))) != cudaSuccess) return e;
+    return cudaFuncSetAttribute(k_front_small<3>, at, (int)sizeof(FrontShared));
+}
+
+static TableArgs table_args(const lp_ctx* c, int64_t n)
+{
+    return TableArgs{c->dc.dim, c->dc.mbits, c->dc.dim == 1 ? 0 : n, c->keys_sorted, c->grange, c->level_off_dev, c->cells};
+}
+
+cudaError_t init_extent(lp_ctx* c, cudaStream_t s)
+{
+    const int ns = c->dc.nsim_max;
+    k_init_extent<<<(unsigned)((8 * (int64_t)ns + 255) / 256), 256, 0, s>>>(c->ext, ns);
+    return cudaGetLastError();
+}
+
+bool front_is_small(const lp_ctx* c, int64_t n) { return c->nsim == 1 && n <= FS_MAX; }
+
+int front_launches(const lp_ctx* c, int64_t n)
+{
+    return front_is_small(c, n) ? 1 : 2 + (c->nsim > 1 ? 1 : 0);
+}
+
+// everything up to the sort; for small n the sort too (one kernel)
+cudaError_t build_front(lp_ctx* c, const lp_particles* p, int64_t n_old, cudaStream_t s)
+{
+    const int64_t n = p->n;
+    const int nsim = c->nsim, dim = c->dc.dim, mb = c->dc.mbits;
+    const TableArgs old = table_args(c, n_old);
+    const double* x1 = p->x[1] ? p->x[1] : p->x[0];
+    const double* x2 = p->x[2] ? p->x[2] : p->x[0];
+    if (front_is_small(c, n)) {
+        // the buffers radix_sort ends in, so that a captured step finds the keys of
+        // the one before it where the capture did.  (They may hold the last build's
+        // keys: those are read before the block's barriers, the new ones written
+        // after them.)
+        const int out = radix_passes(c) & 1;
+        c->keys_sorted = c->keys[out];
+        c->perm_sorted = c->vals[out];
+        return front_small(dim, (int)n, p->x[0], x1, x2, c->dc, c->grid, c->ext, old, c->sort_lo_bit, c->sort_hi_bit,
+                           c->keys_sorted, c->perm_sorted, s);
+    }
     const uint32_t* sim_of = nullptr;
     if (nsim > 1) {
         k_sim_of<<<grid_for(n, 256), 256, 0, s>>>(n, c->offsets, nsim, c->sim_of);
         sim_of = c->sim_of;
     }
-    k_init_extent<<<(unsigned)((8 * nsim + 255) / 256), 256, 0, s>>>(c->ext, nsim);
-    int64_t nb_ = grid_for(n, 256);
-    unsigned blocks = nsim > 1 ? (unsigned)((n + 256 * EXT_ITEMS - 1) / (256 * EXT_ITEMS))
-                               : (unsigned)(nb_ < 152 * 8 ? nb_ : 152 * 8);
-    if (blocks == 0) blocks = 1;
-    const double* x1 = p->x[1] ? p->x[1] : p->x[0];
-    const double* x2 = p->x[2] ? p->x[2] : p->x[0];
-    if (c->dc.dim == 3) k_reduce_extent<3><<<blocks, 256, 0, s>>>(n, p->x[0], x1, x2, sim_of, c->ext);
-    else if (c->dc.dim == 2) k_reduce_extent<2><<<blocks, 256, 0, s>>>(n, p->x[0], x1, x2, sim_of, c->ext);
-    else k_reduce_extent<1><<<blocks, 256, 0, s>>>(n, p->x[0], x1, x2, sim_of, c->ext);
-    k_finalize_cube<<<(unsigned)((nsim + 127) / 128), 128, 0, s>>>(c->dc, nsim, c->ext, c->grid);
-    return cudaGetLastError();
-}
-
-cudaError_t make_keys(lp_ctx* c, const lp_particles* p, cudaStream_t s)
-{
-    int64_t n = p->n;
-    int dim = c->dc.dim;
-    const double* x1 = p->x[1] ? p->x[1] : p->x[0];
-    const double* x2 = p->x[2] ? p->x[2] : p->x[0];
-    const uint32_t* sim_of = c->nsim > 1 ? c->sim_of : nullptr;
-    int mb = c->dc.mbits;
-    unsigned gb = grid_for(n, 256);
+    const int64_t nb_ = grid_for(n, 256);
+    const unsigned blocks = nsim > 1 ? (unsigned)((n + 256 * EXT_ITEMS - 1) / (256 * EXT_ITEMS))
+                                     : (unsigned)(nb_ < 152 * 8 ? nb_ : 152 * 8);
+#define LP_BEGIN_ARGS n, p->x[0], x1, x2, sim_of, c->ext, c->dc, nsim, c->grid, c->tickets, old
+    if (dim == 3) k_begin<3><<<blocks, 256, 0, s>>>(LP_BEGIN_ARGS);
+    else if (dim == 2) k_begin<2><<<blocks, 256, 0, s>>>(LP_BEGIN_ARGS);
+    else k_begin<1><<<blocks, 256, 0, s>>>(LP_BEGIN_ARGS);
+#undef LP_BEGIN_ARGS
+    const unsigned gb = grid_for(n, 256);
     if (dim == 3) k_keys<3><<<gb, 256, 0, s>>>(n, p->x[0], x1, x2, c->grid, sim_of, mb, c->keys[0], c->vals[0]);
     else if (dim == 2) k_keys<2><<<gb, 256, 0, s>>>(n, p->x[0], x1, x2, c->grid, sim_of, mb, c->keys[0], c->vals[0]);
     else k_keys<1><<<gb, 256, 0, s>>>(n, p->x[0], x1, x2, c->grid, sim_of, mb, c->keys[0], c->vals[0]);
@@ -749,7 +1028,8 @@ cudaError_t gather(lp_ctx* c, const lp_particles* p, cudaStream_t s)
     else k_gather<1><<<gb, 256, 0, s>>>(LP_GATHER_ARGS);
 #undef LP_GATHER_ARGS
     // the cell levels need the m V extent the gather took
-    k_finalize_levels<<<1, LEVEL_THREADS, 0, s>>>(c->dc, c->lmax_cap, c->nsim, c->ext, c->grid, c->grange);
+    k_finalize_levels<<<1, LEVEL_THREADS, 0, s>>>(c->dc, c->lmax_cap, c->nsim, c->ext, c->grid, c->grange, c->counters);
+    c->fresh_query = c->fresh_fit = 1;
     return cudaGetLastError();
 }
 
@@ -767,7 +1047,8 @@ cudaError_t gather_geometry(lp_ctx* c, const lp_particles* p, cudaStream_t s)
     else if (dim == 2) k_gather_geom<2><<<gb, 256, 0, s>>>(LP_GATHER_ARGS);
     else k_gather_geom<1><<<gb, 256, 0, s>>>(LP_GATHER_ARGS);
 #undef LP_GATHER_ARGS
-    k_finalize_levels<<<1, LEVEL_THREADS, 0, s>>>(c->dc, c->lmax_cap, c->nsim, c->ext, c->grid, c->grange);
+    k_finalize_levels<<<1, LEVEL_THREADS, 0, s>>>(c->dc, c->lmax_cap, c->nsim, c->ext, c->grid, c->grange, c->counters);
+    c->fresh_query = c->fresh_fit = 1;
     return cudaGetLastError();
 }
 
@@ -794,8 +1075,8 @@ cudaError_t gather_fields(lp_ctx* c, const lp_particles* p, cudaStream_t s)
 cudaError_t fill_tables(lp_ctx* c, int64_t n, bool clear, cudaStream_t s)
 {
     if (c->dc.dim == 1 || n == 0) return cudaSuccess;
-    k_tables<<<grid_for(n, 256), 256, 0, s>>>(c->dc.dim, c->dc.mbits, n, c->keys_sorted, c->grange,
-                                               c->level_off_dev, c->cells, clear ? 1 : 0);
+    if (clear) k_tables<true><<<grid_for(n, 256), 256, 0, s>>>(table_args(c, n));
+    else k_tables<false><<<grid_for(n, 256), 256, 0, s>>>(table_args(c, n));
     return cudaGetLastError();
 }
 
@@ -866,7 +1147,7 @@ cudaError_t noalloc_setup(cudaStream_t s, unsigned char** out)
     if (cs == cudaStreamCaptureStatusNone) {
         void* p = nullptr;
         e = cudaGetSymbolAddress(&p, noalloc_scratch);
-        if (e != cudaSuccess) return e;
+        if (e != cudaSuccess || (e = sort_init()) != cudaSuccess) return e;
         na_ptr[dev] = static_cast<unsigned char*>(p);
     } else if (!na_ptr[dev]) {
         return cudaErrorStreamCaptureUnsupported;
@@ -916,14 +1197,18 @@ extern "C" lp_status lp_sort_keys_noalloc(int32_t dim, int64_t n, const double* 
     int lmax_cap = dim == 3 ? 9 : (dim == 2 ? 13 : 0);
     int lo_bit = 0, hi_bit = 64;
     sort_bit_range(dim, MORTON_BITS, lmax_cap, 0, lo_bit, hi_bit);
+    const TableArgs none = {};
+    if (n <= FS_MAX)
+        return front_small(dim, (int)n, x0, p1, p2, dc, grid, ext, none, lo_bit, hi_bit, keys_out, perm_out, s) ==
+                       cudaSuccess ? LP_OK : LP_ERR_CUDA;
     unsigned gb = grid_for(n, 256);
     int64_t nb_ = gb;
     unsigned rblocks = (unsigned)(nb_ < 152 * 8 ? nb_ : 152 * 8);
+    unsigned int* ticket = reinterpret_cast<unsigned int*>(ext + 8);     // (zero at load, put back by k_begin)
     k_init_extent<<<1, 32, 0, s>>>(ext, 1);
-    if (dim == 3) k_reduce_extent<3><<<rblocks, 256, 0, s>>>(n, x0, p1, p2, nullptr, ext);
-    else if (dim == 2) k_reduce_extent<2><<<rblocks, 256, 0, s>>>(n, x0, p1, p2, nullptr, ext);
-    else k_reduce_extent<1><<<rblocks, 256, 0, s>>>(n, x0, p1, p2, nullptr, ext);
-    k_finalize_cube<<<1, 1, 0, s>>>(dc, 1, ext, grid);
+    if (dim == 3) k_begin<3><<<rblocks, 256, 0, s>>>(n, x0, p1, p2, nullptr, ext, dc, 1, grid, ticket, none);
+    else if (dim == 2) k_begin<2><<<rblocks, 256, 0, s>>>(n, x0, p1, p2, nullptr, ext, dc, 1, grid, ticket, none);
+    else k_begin<1><<<rblocks, 256, 0, s>>>(n, x0, p1, p2, nullptr, ext, dc, 1, grid, ticket, none);
     if (dim == 3) k_keys<3><<<gb, 256, 0, s>>>(n, x0, p1, p2, grid, nullptr, MORTON_BITS, keys[0], vals[0]);
     else if (dim == 2) k_keys<2><<<gb, 256, 0, s>>>(n, x0, p1, p2, grid, nullptr, MORTON_BITS, keys[0], vals[0]);
     else k_keys<1><<<gb, 256, 0, s>>>(n, x0, p1, p2, grid, nullptr, MORTON_BITS, keys[0], vals[0]);
