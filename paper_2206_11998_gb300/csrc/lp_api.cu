@@ -689,9 +689,10 @@ lp_status lp_gfd_derivs(lp_ctx* c, const lp_particles* p, const double* const* f
                 k_split_fields<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(
                     n, F, F, a.fd[0], a.fd[1], a.fd[2], a.fd[3], a.fd[4], c->rec);
             }
-            LP_CUDA(cudaMemsetAsync(c->counters + C_REDO_LEN, 0, 8, s));
+            static_assert(C_REFINE_LEN == C_REDO_LEN + 1, "one memset for both lengths");
+            LP_CUDA(cudaMemsetAsync(c->counters + C_REDO_LEN, 0, 16, s));
             {
-                Phase ph(c, LP_PH_FIT, 1, s);
+                Phase ph(c, LP_PH_FIT, c->dc.refine == LP_REFINE_AUTO ? 2 : 1, s);
                 LP_CUDA(launch_derivs_f32(dim, F, a, o, s));
             }
             a.list = c->redo_list;
@@ -728,9 +729,9 @@ lp_status lp_onesided_derivs(lp_ctx* c, const lp_particles* p, const double* con
             k_split_fields<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(
                 n, 5, 5, a.fd[0], a.fd[1], a.fd[2], a.fd[3], a.fd[4], c->rec);
         }
-        LP_CUDA(cudaMemsetAsync(c->counters + C_REDO_LEN, 0, 8, s));
+        LP_CUDA(cudaMemsetAsync(c->counters + C_REDO_LEN, 0, 16, s));
         {
-            Phase ph(c, LP_PH_FIT, 1, s);
+            Phase ph(c, LP_PH_FIT, 3, s);
             LP_CUDA(launch_onesided_f32(dim, a, derivs, nfields, s));
         }
         a.list = c->redo_list;

@@ -271,8 +271,34 @@ struct NormalEqPacked {
         for (int q = 0; q < NP; ++q) P[q] = make_float2(0.0f, 0.0f);
     }
 
-    __device__ void add(const float (&a)[N], const float (&b)[F])
+    // (F = 0) the row without right-hand sides
+    __device__ void add_gram(const float (&a)[N])
     {
+        static_assert(F == 0, "the Gram matrix alone");
+        float2 v[VP];
+#pragma unroll
+        for (int p = 0; p < VP; ++p) v[p] = make_float2(a[2 * p], 2 * p + 1 < N ? a[2 * p + 1 < N ? 2 * p + 1 : 0] : 0.0f);
+#pragma unroll
+        for (int k = 0; k < N; ++k) {
+            const float2 ak = make_float2(a[k], a[k]);
+#pragma unroll
+            for (int p = k / 2; p < VP; ++p) P[off(k) + p - k / 2] = __ffma2_rn(ak, v[p], P[off(k) + p - k / 2]);
+        }
+    }
+
+    template <int F1>
+    __device__ void store_gram(NormalEq<float, N, F1>& E) const
+    {
+#pragma unroll
+        for (int k = 0; k < N; ++k)
+#pragma unroll
+            for (int l = k; l < N; ++l) E.Gm[NormalEq<float, N, F1>::id(k, l)] = at(k, l);
+    }
+
+    template <int F1 = F>
+    __device__ void add(const float (&a)[N], const float (&b)[F1])
+    {
+        static_assert(F1 == F && F > 0, "a row with its right-hand sides");
         float2 v[VP];
 #pragma unroll
         for (int p = 0; p < VP; ++p) {
@@ -815,9 +841,12 @@ __device__ int linear_fit(const Src<T, DIM, F>& src, const NB& nb, int cnt, T in
 // tailn and finds them by a scan of the list's tail.  ok[k][s] = false where
 // fewer than DIM members or rank deficient.  ill = true when a system with
 // enough members is below tau (FP32: redo in FP64).
+//
+// onesided_fits leaves component f of fit q = 2k + s at osm[q F + f][threadIdx.x]
+// (shared memory; only where bit q of the returned mask is set).
 template <typename T, int DIM, int F, class NB>
-__device__ __forceinline__ void onesided_all(const Src<T, DIM, F>& src, const NB& nb, int cnt, int ks, T invS, T tau,
-                             T tau_rank, T (&out)[DIM][2][F], bool (&ok)[DIM][2], bool& ill)
+__device__ __forceinline__ unsigned onesided_fits(const Src<T, DIM, F>& src, const NB& nb, int cnt, int ks, T invS,
+                                                  T tau, T tau_rank, T (*osm)[FIT_THREADS], bool& ill)
 {
     uint64_t m[DIM][2];
     int c[DIM][2];
@@ -853,7 +882,6 @@ __device__ __forceinline__ void onesided_all(const Src<T, DIM, F>& src, const NB
     }
     // the 2 DIM fits in one rolled loop (one copy of its code); fit q = 2k + s
     // leaves its k-component in shared memory and a bit in okb
-    __shared__ T osm[2 * DIM * F][FIT_THREADS];
     unsigned okb = 0;
 #pragma unroll 1
     for (int q = 0; q < 2 * DIM; ++q) {
@@ -918,6 +946,15 @@ __device__ __forceinline__ void onesided_all(const Src<T, DIM, F>& src, const NB
         }
         okb |= 1u << q;
     }
+    return okb;
+}
+
+template <typename T, int DIM, int F, class NB>
+__device__ __forceinline__ void onesided_all(const Src<T, DIM, F>& src, const NB& nb, int cnt, int ks, T invS, T tau,
+                             T tau_rank, T (&out)[DIM][2][F], bool (&ok)[DIM][2], bool& ill)
+{
+    __shared__ T osm[2 * DIM * F][FIT_THREADS];
+    const unsigned okb = onesided_fits<T, DIM, F>(src, nb, cnt, ks, invS, tau, tau_rank, osm, ill);
 #pragma unroll
     for (int k = 0; k < DIM; ++k)
 #pragma unroll
@@ -926,6 +963,48 @@ __device__ __forceinline__ void onesided_all(const Src<T, DIM, F>& src, const NB
 #pragma unroll
             for (int f = 0; f < F; ++f) out[k][s][f] = ok[k][s] ? osm[(2 * k + s) * F + f][threadIdx.x] : T(0);
         }
+}
+
+// Whether the FP32 central fit would be ill-conditioned (central_fit's result
+// 1): the Gram matrix, its factor and, below NE_RATIO_MIN, the rotations,
+// without right-hand sides.  The matrix's sums, and so the ratio, are bit for
+// bit those of central_fit; half of each record and half of the sums suffice.
+template <int DIM, int F, class NB>
+__device__ __forceinline__ bool central_ill(const Src<float, DIM, F>& src, const NB& nb, int cnt, float invS, float tau)
+{
+    constexpr int N = NU<DIM>::v;
+    using Rec = typename Src<float, DIM, F>::Rec;
+    if (cnt < N) return true;
+    NormalEqPacked<N, 0> EP;
+    EP.zero();
+    for_neighbors<true>(src, nb, cnt, [&](uint32_t, const Rec& rec) {
+        float d[DIM], a[N], bl;
+        src.unpack_last(rec, d, bl);
+#pragma unroll
+        for (int k = 0; k < DIM; ++k) d[k] *= invS;
+        gfd_row<float, DIM>(d, a);
+        EP.add_gram(a);
+        return true;
+    });
+    NormalEq<float, N, 1> E;
+    Givens<float, N, 1> G;
+    EP.store_gram(E);
+    E.factor(G);
+    float ratio = G.ratio();
+    if (!(ratio >= NE_RATIO_MIN)) {
+        G.zero();
+        for_neighbors<true>(src, nb, cnt, [&](uint32_t, const Rec& rec) {
+            float d[DIM], a[N], b[1];
+            src.unpack_last(rec, d, b[0]);
+#pragma unroll
+            for (int k = 0; k < DIM; ++k) d[k] *= invS;
+            gfd_row<float, DIM>(d, a);
+            G.add(a, b);
+            return true;
+        });
+        ratio = G.ratio();
+    }
+    return !(ratio >= tau);
 }
 
 // ---------------------------------------------------------------------------

@@ -631,19 +631,23 @@ struct DerivOut {
     uint32_t* status;
 };
 
-template <typename T, int DIM, int F>
-__device__ void derivs_one(const FitArgs& a, const DerivOut& o, int64_t i)
+template <typename T, int DIM, int F, bool DEFER = false, class NB>
+__device__ __forceinline__ void derivs_one(const FitArgs& a, const DerivOut& o, int64_t i, const NB& nb)
 {
     constexpr int N = NU<DIM>::v;
     const DevCfg& c = a.c;
     Src<T, DIM, F> src(a, i);
     const int cnt = (int)a.count[i];
-    const NbGlobal nb{a.idx + i * (int64_t)c.k_max};
     const T invS = (T)inv_scale(last_d2(src, nb, cnt));
     const T tau = IsF32<T>::v ? (T)c.tau32 : (T)c.tau64;
     T cd[N][F];
     uint32_t st = IsF32<T>::v ? 0u : (a.list ? FIT_FP64 : 0u);
-    if (central_fit<T, DIM, F>(src, nb, cnt, invS, tau, c, cd)) {
+    const int ill = central_fit<T, DIM, F, false, DEFER>(src, nb, cnt, invS, tau, c, cd);
+    if (DEFER && ill == 2) {
+        a.refine_list[atomicAdd(a.refine_len, 1ull)] = (uint32_t)i;
+        return;
+    }
+    if (ill) {
         if (IsF32<T>::v) { push_redo(a, i); return; }
         st |= FIT_LINEAR;
 #pragma unroll
@@ -674,29 +678,53 @@ __device__ void derivs_one(const FitArgs& a, const DerivOut& o, int64_t i)
     if (o.status && o.f_first == 0) o.status[i] = st;
 }
 
-template <typename T, int DIM, int F>
-__global__ void __launch_bounds__(FIT_THREADS) k_derivs(FitArgs a, DerivOut o)
+// The warp's list rows staged as in k_step_central; DEFER (FP32, correction
+// where the ratio asks for it): the fits that need the correction pass go to
+// k_derivs_refine.  One field needs half of each record and under 100 registers,
+// so more blocks fit an SM.
+template <typename T, int F> struct DerivOcc { static constexpr int v = 1; };
+template <> struct DerivOcc<float, 1> { static constexpr int v = 5; };
+template <> struct DerivOcc<float, 5> { static constexpr int v = 3; };
+template <typename T, int DIM, int F, bool DEFER>
+__global__ void __launch_bounds__(FIT_THREADS, DerivOcc<T, F>::v) k_derivs(FitArgs a, DerivOut o)
 {
-    int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i < a.n) derivs_one<T, DIM, F>(a, o, i);
+    constexpr int SD = DEFER ? 64 : 32;
+    __shared__ uint32_t stage[SD][NB_PITCH];
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    stage_rows<SD>(stage, a.idx, a.c.k_max, i < a.n ? i : -1);
+    if (i >= a.n) return;
+    derivs_one<T, DIM, F, DEFER>(a, o, i, NbStaged<SD>{a.idx + i * (int64_t)a.c.k_max, &stage[0][threadIdx.x]});
+}
+
+// the fits k_derivs deferred, with the correction pass on (the caller passes
+// refine = LP_REFINE_ALWAYS)
+template <typename T, int DIM, int F>
+__global__ void __launch_bounds__(FIT_THREADS) k_derivs_refine(FitArgs a, DerivOut o)
+{
+    const unsigned long long len = *a.refine_len;
+    for (unsigned long long t = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; t < len;
+         t += (unsigned long long)gridDim.x * blockDim.x) {
+        const int64_t i = a.refine_list[t];
+        derivs_one<T, DIM, F>(a, o, i, NbGlobal{a.idx + i * (int64_t)a.c.k_max});
+    }
 }
 
 // ---------------------------------------------------------------------------
 // one-sided derivatives (lp_onesided_derivs), out[i][k][s][f] float64
 // ---------------------------------------------------------------------------
-template <typename T, int DIM, int F>
+template <int DIM, int F>
 __device__ void onesided_one(const FitArgs& a, double* out, int f_real, int64_t i)
 {
+    using T = double;
     constexpr int N = NU<DIM>::v;
     const DevCfg& c = a.c;
     Src<T, DIM, F> src(a, i);
     const int cnt = (int)a.count[i];
     const NbGlobal nb{a.idx + i * (int64_t)c.k_max};
     const T invS = (T)inv_scale(last_d2(src, nb, cnt));
-    const T tau = IsF32<T>::v ? (T)c.tau32 : (T)c.tau64;
+    const T tau = c.tau64;
     T cd[N][F];
     if (central_fit<T, DIM, F>(src, nb, cnt, invS, tau, c, cd)) {
-        if (IsF32<T>::v) { push_redo(a, i); return; }
 #pragma unroll
         for (int u = 0; u < N; ++u)
 #pragma unroll
@@ -722,7 +750,6 @@ __device__ void onesided_one(const FitArgs& a, double* out, int f_real, int64_t 
 #pragma unroll
                 for (int f = 0; f < F; ++f) os[k][s][f] = ok[k][s] ? o2[k][s][f] : cd[k][f];
     }
-    if (IsF32<T>::v && ill) { push_redo(a, i); return; }
 #pragma unroll
     for (int k = 0; k < DIM; ++k)
 #pragma unroll
@@ -732,11 +759,101 @@ __device__ void onesided_one(const FitArgs& a, double* out, int f_real, int64_t 
                 if (f < f_real) out[((i * DIM + k) * 2 + s) * f_real + f] = (double)os[k][s][f];
 }
 
-template <typename T, int DIM, int F>
+template <int DIM, int F>
 __global__ void __launch_bounds__(FIT_THREADS) k_onesided(FitArgs a, double* out, int f_real)
 {
     int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i < a.n) onesided_one<T, DIM, F>(a, out, f_real, i);
+    if (i < a.n) onesided_one<DIM, F>(a, out, f_real, i);
+}
+
+// The FP32 path in three kernels.  k_onesided_sides runs the one-sided fits (the
+// warp's list rows staged, results written coalesced: 30 doubles a particle, one
+// line per lane and store otherwise) and lists the particles that lack a side,
+// which need central derivatives; k_onesided_check tests the others' central
+// fits (an ill-conditioned one sends the whole particle to the FP64 redo) from
+// the Gram matrix alone; k_onesided_fill runs the listed particles' central
+// fits.  In one kernel every particle ran the whole central fit, for 10 % of
+// them on a 59^3 lattice to use it: 334 us at 205k particles, against 190 us.
+// state[i] (plain_list): nothing more to do, or the FP64 redo has it
+// (SIDES_REDO); else SIDES_CHECK or the mask of the fits it has.
+constexpr uint32_t SIDES_REDO = 0xffffffffu, SIDES_CHECK = 0xfffffffeu;
+template <int DIM, int F>
+__global__ void __launch_bounds__(FIT_THREADS, 5) k_onesided_sides(FitArgs a, double* out, int f_real)
+{
+    __shared__ uint32_t stage[32][NB_PITCH];
+    __shared__ float osm[2 * DIM * F][FIT_THREADS];
+    const DevCfg& c = a.c;
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    stage_rows<32>(stage, a.idx, c.k_max, i < a.n ? i : -1);
+    if (i < a.n) {
+        Src<float, DIM, F> src(a, i);
+        const int cnt = (int)a.count[i];
+        const NbStaged<32> nb{a.idx + i * (int64_t)c.k_max, &stage[0][threadIdx.x]};
+        const float invS = inv_scale(last_d2(src, nb, cnt));
+        bool ill = false;
+        const unsigned okb = onesided_fits<float, DIM, F>(src, nb, cnt, c.k_side, invS, (float)c.tau32, (float)c.tau64,
+                                                          osm, ill);
+        constexpr unsigned ALL = (1u << (2 * DIM)) - 1u;
+        a.plain_list[i] = ill ? SIDES_REDO : (okb == ALL ? SIDES_CHECK : okb);
+        if (ill) push_redo(a, i);
+        const bool lacks = !ill && okb != ALL;
+        const unsigned long long t = warp_append(a.refine_len, lacks);
+        if (lacks) a.refine_list[t] = (uint32_t)i;
+    }
+    __syncwarp();
+    // the warp's particles are one run of the output; entries of sides without a
+    // fit are filled in later
+    const int w0 = (int)(threadIdx.x & ~31u), lane = (int)(threadIdx.x & 31u);
+    const int64_t i0 = i - lane;
+    if (i0 >= a.n) return;
+    const int per = 2 * DIM * f_real, np = (int)(a.n - i0 < 32 ? a.n - i0 : 32);
+    for (int e = lane; e < np * per; e += 32) {
+        const int p = e / per, r = e - p * per, q = r / f_real, f = r - q * f_real;
+        out[i0 * per + e] = (double)osm[q * F + f][w0 + p];
+    }
+}
+
+template <int DIM, int F>
+__global__ void __launch_bounds__(FIT_THREADS, 5) k_onesided_check(FitArgs a)
+{
+    __shared__ uint32_t stage[64][NB_PITCH];
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    const bool mine = i < a.n && a.plain_list[i] == SIDES_CHECK;
+    stage_rows<64>(stage, a.idx, a.c.k_max, mine ? i : -1);
+    if (!mine) return;
+    Src<float, DIM, F> src(a, i);
+    const int cnt = (int)a.count[i];
+    const NbStaged<64> nb{a.idx + i * (int64_t)a.c.k_max, &stage[0][threadIdx.x]};
+    const float invS = inv_scale(last_d2(src, nb, cnt));
+    if (central_ill<DIM, F>(src, nb, cnt, invS, (float)a.c.tau32)) push_redo(a, i);
+}
+
+template <int DIM, int F>
+__global__ void __launch_bounds__(FIT_THREADS) k_onesided_fill(FitArgs a, double* out, int f_real)
+{
+    const unsigned long long len = *a.refine_len;
+    for (unsigned long long t = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; t < len;
+         t += (unsigned long long)gridDim.x * blockDim.x) {
+        const int64_t i = a.refine_list[t];
+        Src<float, DIM, F> src(a, i);
+        const int cnt = (int)a.count[i];
+        const NbGlobal nb{a.idx + i * (int64_t)a.c.k_max};
+        const float invS = inv_scale(last_d2(src, nb, cnt));
+        float cd[NU<DIM>::v][F];
+        if (central_fit<float, DIM, F>(src, nb, cnt, invS, (float)a.c.tau32, a.c, cd)) {
+            push_redo(a, i);
+            continue;
+        }
+        const unsigned okb = a.plain_list[i];
+#pragma unroll
+        for (int k = 0; k < DIM; ++k)
+#pragma unroll
+            for (int s = 0; s < 2; ++s)
+                if (!((okb >> (2 * k + s)) & 1u))
+#pragma unroll
+                    for (int f = 0; f < F; ++f)
+                        if (f < f_real) out[((i * DIM + k) * 2 + s) * f_real + f] = (double)cd[k][f];
+    }
 }
 
 // launchers, defined once per precision in lp_fit_f32.cu / lp_fit_f64.cu
@@ -784,6 +901,23 @@ inline bool split_defers_t(const FitArgs& a)
 inline unsigned fit_blocks(const FitArgs& a)
 {
     return (unsigned)((a.n + FIT_THREADS - 1) / FIT_THREADS);
+}
+
+template <typename T, int DIM, int F>
+cudaError_t launch_derivs(const FitArgs& a, const DerivOut& o, cudaStream_t s)
+{
+    const unsigned b = fit_blocks(a);
+    if constexpr (IsF32<T>::v) {
+        if (split_defers_t<T>(a)) {
+            FitArgs r = a;
+            r.c.refine = LP_REFINE_ALWAYS;
+            k_derivs<T, DIM, F, true><<<b, FIT_THREADS, 0, s>>>(a, o);
+            k_derivs_refine<T, DIM, F><<<152u * 4u, FIT_THREADS, 0, s>>>(r, o);
+            return cudaGetLastError();
+        }
+    }
+    k_derivs<T, DIM, F, false><<<b, FIT_THREADS, 0, s>>>(a, o);
+    return cudaGetLastError();
 }
 
 #define LP_DEFINE_FIT_LAUNCHERS(T, SUF)                                                         \
@@ -850,23 +984,11 @@ inline unsigned fit_blocks(const FitArgs& a)
     cudaError_t launch_derivs_##SUF(int dim, int F, const FitArgs& a, const DerivOut& o,        \
                                     cudaStream_t s)                                             \
     {                                                                                           \
-        unsigned b = fit_blocks(a);                                                             \
-        if (b == 0) return cudaSuccess;                                                         \
-        if (dim == 3 && F == 1) k_derivs<T, 3, 1><<<b, FIT_THREADS, 0, s>>>(a, o);                     \
-        else if (dim == 3) k_derivs<T, 3, 5><<<b, FIT_THREADS, 0, s>>>(a, o);                          \
-        else if (dim == 2) k_derivs<T, 2, 5><<<b, FIT_THREADS, 0, s>>>(a, o);                          \
-        else k_derivs<T, 1, 5><<<b, FIT_THREADS, 0, s>>>(a, o);                                        \
-        return cudaGetLastError();                                                              \
-    }                                                                                           \
-    cudaError_t launch_onesided_##SUF(int dim, const FitArgs& a, double* out, int f_real,       \
-                                      cudaStream_t s)                                           \
-    {                                                                                           \
-        unsigned b = fit_blocks(a);                                                             \
-        if (b == 0) return cudaSuccess;                                                         \
-        if (dim == 3) k_onesided<T, 3, 5><<<b, FIT_THREADS, 0, s>>>(a, out, f_real);                   \
-        else if (dim == 2) k_onesided<T, 2, 5><<<b, FIT_THREADS, 0, s>>>(a, out, f_real);              \
-        else k_onesided<T, 1, 5><<<b, FIT_THREADS, 0, s>>>(a, out, f_real);                            \
-        return cudaGetLastError();                                                              \
+        if (a.n == 0) return cudaSuccess;                                                       \
+        if (dim == 3 && F == 1) return launch_derivs<T, 3, 1>(a, o, s);                         \
+        if (dim == 3) return launch_derivs<T, 3, 5>(a, o, s);                                   \
+        if (dim == 2) return launch_derivs<T, 2, 5>(a, o, s);                                   \
+        return launch_derivs<T, 1, 5>(a, o, s);                                                 \
     }
 
 }  // namespace lp

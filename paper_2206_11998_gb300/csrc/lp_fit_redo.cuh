@@ -491,7 +491,7 @@ __global__ void __launch_bounds__(FIT_THREADS) k_derivs_redo(FitArgs a, DerivOut
     }
     for (unsigned long long t = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; t < len;
          t += (unsigned long long)gridDim.x * blockDim.x)
-        derivs_one<double, DIM, F>(a, o, a.list[t]);
+        derivs_one<double, DIM, F>(a, o, a.list[t], NbGlobal{a.idx + (int64_t)a.list[t] * (int64_t)a.c.k_max});
 }
 
 template <int DIM, int F>
@@ -513,7 +513,7 @@ __global__ void __launch_bounds__(FIT_THREADS) k_onesided_redo(FitArgs a, double
     }
     for (unsigned long long t = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; t < len;
          t += (unsigned long long)gridDim.x * blockDim.x)
-        onesided_one<double, DIM, F>(a, out, f_real, a.list[t]);
+        onesided_one<DIM, F>(a, out, f_real, a.list[t]);
 }
 
 }  // namespace lp
