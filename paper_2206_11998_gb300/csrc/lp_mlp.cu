@@ -207,8 +207,8 @@ struct MlpTrainArgs {
     float* m1;
     float* m2;
     __nv_bfloat16* wb;
-    float* gbuf;                  // [3][MLP_NPARAM], zero
-    float* loss;                  // [epochs], zero: sums of the batch losses
+    float* gbuf;                  // [3][MLP_NPARAM + 1], zero: gradient, batch loss
+    float* loss;                  // [epochs]: sums of the batch losses
     unsigned int* arrived;        // zero
     int64_t step;                 // Adam steps taken before
     unsigned int* lost;           // set (and ST_TIMEOUT in the status word) where the barrier gave up
@@ -241,12 +241,14 @@ __global__ void __launch_bounds__(MT_THREADS) k_mlp_train(MlpTrainArgs a)
     MlpSample v = mlp_load(a.X, a.y, size(0), t0);
     unsigned it = 0;
     for (int ep = 0; ep < a.epochs; ++ep) {
+        double total = 0.0;                     // (of block 0's first thread)
         for (int64_t b0 = 0; b0 < a.n; b0 += a.batch, ++it) {
-            float* g = a.gbuf + (it % 3u) * MLP_NPARAM;
+            float* g = a.gbuf + (it % 3u) * (MLP_NPARAM + 1);
             if (blockIdx.x == 0)
-                for (int q = tid; q < MLP_NPARAM; q += MT_THREADS) a.gbuf[((it + 1u) % 3u) * MLP_NPARAM + q] = 0.0f;
+                for (int q = tid; q <= MLP_NPARAM; q += MT_THREADS)
+                    a.gbuf[((it + 1u) % 3u) * (MLP_NPARAM + 1) + q] = 0.0f;
             const int64_t nb = size(b0);
-            mlp_block_grad(sm, v, a.X + b0 * MLP_IN, a.y + b0, nb, nb, a.pos_weight, g, a.loss + ep);
+            mlp_block_grad(sm, v, a.X + b0 * MLP_IN, a.y + b0, nb, nb, a.pos_weight, g, g + MLP_NPARAM);
             // the next minibatch's samples, in flight over the barrier
             const int64_t b1 = b0 + a.batch < a.n ? b0 + a.batch : 0;
             v = mlp_load(a.X + b1 * MLP_IN, a.y + b1, size(b1), t0);
@@ -270,6 +272,7 @@ __global__ void __launch_bounds__(MT_THREADS) k_mlp_train(MlpTrainArgs a)
             }
             __syncthreads();
             if (lost) return;
+            if (blockIdx.x == 0 && tid == 0) total += (double)__ldcg(g + MLP_NPARAM);
             float gq[PER];
 #pragma unroll
             for (int u = 0; u < PER; ++u) gq[u] = tid + u * MT_THREADS < MLP_NPARAM ? __ldcg(g + tid + u * MT_THREADS) : 0.0f;
@@ -282,6 +285,7 @@ __global__ void __launch_bounds__(MT_THREADS) k_mlp_train(MlpTrainArgs a)
             }
             __syncthreads();
         }
+        if (blockIdx.x == 0 && tid == 0) a.loss[ep] = (float)total;
     }
     if (blockIdx.x != 0) return;
 #pragma unroll
@@ -403,7 +407,7 @@ lp_status lp_mlp_train(lp_ctx* c, const float* X, const float* y, int64_t n, int
     a.lost = reinterpret_cast<unsigned int*>(c->mlp_work);
     a.loss = c->mlp_work + 1;
     a.gbuf = a.loss + MLP_EPOCHS;
-    a.arrived = reinterpret_cast<unsigned int*>(a.gbuf + 3 * MLP_NPARAM);
+    a.arrived = reinterpret_cast<unsigned int*>(a.gbuf + 3 * (MLP_NPARAM + 1));
     a.status = reinterpret_cast<unsigned int*>(c->counters + C_STATUS);
     const int64_t nbatches = (n + batch - 1) / batch, most = n < batch ? n : batch;
     // launches of at most MLP_EPOCHS epochs, whose losses the work area holds

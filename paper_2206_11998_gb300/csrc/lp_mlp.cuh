@@ -16,7 +16,7 @@ constexpr int OFF_W2 = OFF_B1 + MLP_H;
 constexpr int OFF_B2 = OFF_W2 + MLP_H;
 constexpr int MLP_NPARAM = OFF_B2 + 1;
 constexpr int MLP_EPOCHS = 1024;                                 // epochs of one training launch
-constexpr int MLP_WORK = 2 + MLP_EPOCHS + 3 * MLP_NPARAM;        // floats: a flag, epoch losses, gradients, barrier
+constexpr int MLP_WORK = 2 + MLP_EPOCHS + 3 * (MLP_NPARAM + 1);        // floats: a flag, epoch losses, gradients, barrier
 
 // logit of the network for features x
 __device__ inline float mlp_logit(const float (&x)[MLP_IN], const __nv_bfloat16* __restrict__ w)
