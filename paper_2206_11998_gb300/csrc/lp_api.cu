@@ -350,6 +350,10 @@ struct Phase {
 
 }  // namespace
 
+namespace {
+lp_status order_fp64(lp_ctx* c, FitArgs& a, cudaStream_t s);
+}
+
 namespace lp {
 
 cudaError_t run_cfl(lp_ctx* c, int64_t n, double cfl, double dt_fixed, double* t, cudaStream_t s)
@@ -371,6 +375,17 @@ cudaError_t run_cfl(lp_ctx* c, int64_t n, double cfl, double dt_fixed, double* t
 }  // namespace lp
 
 namespace {
+
+// FP64 passes over all particles take them by list length, where a warp's worth
+// of lists is long enough to pay for the ordering's launches
+lp_status order_fp64(lp_ctx* c, FitArgs& a, cudaStream_t s)
+{
+    if (c->dc.dim == 1 || a.n < 2048) return LP_OK;
+    // (the sort's histogram and the corrections' list are free here)
+    LP_CUDA(order_by_count(a.n, c->nb_count, c->hist, c->refine_list, s));
+    a.order = c->refine_list;
+    return LP_OK;
+}
 
 // the fit + update pass of one step: the main pass over all particles (fused,
 // or split into central and plain kernels), then, after an FP32 pass, the FP64
@@ -402,7 +417,9 @@ lp_status run_fit(lp_ctx* c, FitArgs a, const StepOut& o, int sched, cudaStream_
         Phase ph(c, LP_PH_FIT64, 1, s);
         LP_CUDA(launch_step_redo(dim, a, o, s));
     } else {
-        Phase ph(c, LP_PH_FIT64, split ? 2 : 1, s);
+        Phase ph(c, LP_PH_FIT64, split ? 4 : 3, s);
+        const lp_status st = order_fp64(c, a, s);
+        if (st != LP_OK) return st;
         LP_CUDA(split ? launch_step_split_f64(dim, a, o, s) : launch_step_f64(dim, a, o, s));
     }
     return LP_OK;
@@ -699,7 +716,9 @@ lp_status lp_gfd_derivs(lp_ctx* c, const lp_particles* p, const double* const* f
             Phase ph(c, LP_PH_FIT64, 1, s);
             LP_CUDA(launch_derivs_redo(dim, F, a, o, s));
         } else {
-            Phase ph(c, LP_PH_FIT64, 1, s);
+            Phase ph(c, LP_PH_FIT64, 3, s);
+            const lp_status st = order_fp64(c, a, s);
+            if (st != LP_OK) return st;
             LP_CUDA(launch_derivs_f64(dim, F, a, o, s));
         }
         f0 += real;
@@ -738,7 +757,9 @@ lp_status lp_onesided_derivs(lp_ctx* c, const lp_particles* p, const double* con
         Phase ph(c, LP_PH_FIT64, 1, s);
         LP_CUDA(launch_onesided_redo(dim, a, derivs, nfields, s));
     } else {
-        Phase ph(c, LP_PH_FIT64, 1, s);
+        Phase ph(c, LP_PH_FIT64, 3, s);
+        const lp_status st = order_fp64(c, a, s);
+        if (st != LP_OK) return st;
         LP_CUDA(launch_onesided_f64(dim, a, derivs, nfields, s));
     }
     return LP_OK;

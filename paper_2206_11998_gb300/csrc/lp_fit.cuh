@@ -44,6 +44,8 @@ template <> struct RN<float> {
     static __device__ __forceinline__ float div(float a, float b) { return __fdiv_rn(a, b); }
     // the hardware reciprocal (a few ulp), as fast as the square root it replaces
     static __device__ __forceinline__ float rcp(float a) { return __fdividef(1.0f, a); }
+    static __device__ __forceinline__ bool nonzero(float a) { return a != 0.0f; }
+    static __device__ __forceinline__ bool positive(float a) { return a > 0.0f; }
 };
 template <> struct RN<double> {
     static __device__ __forceinline__ double mul(double a, double b) { return __dmul_rn(a, b); }
@@ -51,7 +53,29 @@ template <> struct RN<double> {
     static __device__ __forceinline__ double sub(double a, double b) { return __dsub_rn(a, b); }
     static __device__ __forceinline__ double fma(double a, double b, double c) { return __fma_rn(a, b, c); }
     static __device__ __forceinline__ double div(double a, double b) { return __ddiv_rn(a, b); }
-    static __device__ __forceinline__ double rcp(double a) { return __drcp_rn(a); }
+    // 1 / a to within an ulp.  An FP64 instruction holds a scheduler's FP64 unit
+    // for 64 cycles (19 cycles an SM when all four issue them), so the fits in
+    // FP64 are bound by their count, and a rotation takes a reciprocal per column:
+    // the hardware's approximation y (relative error e below 2^-18, from another
+    // unit) and one step of the third-order iteration y (1 + e + e^2), whose error
+    // is e^3, take three FMAs, the rounded reciprocal six.  Where y could be
+    // denormal or infinite, the rounded reciprocal.
+    static __device__ __forceinline__ double rcp(double a)
+    {
+        const unsigned ex = (unsigned)(__double_as_longlong(a) >> 52) & 0x7ffu;
+        if (ex - 4u >= 0x7f0u) return __drcp_rn(a);
+        double y;
+        asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
+        const double e = __fma_rn(-a, y, 1.0);
+        return __fma_rn(y, __fma_rn(e, e, e), y);
+    }
+    // a != 0 and a > 0 from the bits, off the FP64 unit (NaN: as the comparisons)
+    static __device__ __forceinline__ bool nonzero(double a) { return (__double_as_longlong(a) << 1) != 0; }
+    static __device__ __forceinline__ bool positive(double a)
+    {
+        const long long b = __double_as_longlong(a);
+        return b > 0 && b <= 0x7ff0000000000000ll;
+    }
 };
 
 
@@ -100,7 +124,7 @@ struct Givens {
             const T wa = O::mul(w, ak);
             const T dn = O::fma(wa, ak, d[k]);
             // a row absorbed by an empty column keeps weight 0 (live = false: no change)
-            const bool live = wa != T(0) && dn > T(0);
+            const bool live = O::nonzero(wa) && O::positive(dn);
             const T inv = live ? O::rcp(dn) : T(0);
             const T sk = O::mul(wa, inv);                     // 0 when not live
             const T ck = live ? O::mul(d[k], inv) : T(1);     // 1 when not live: U, Z unchanged
@@ -371,6 +395,7 @@ struct FitArgs {
     const double* sm;
     unsigned long long* counters;
     uint32_t* redo_list;      // FP32 pass: particles to redo in FP64
+    const uint32_t* order;    // thread t's particle (null: t)
     const uint32_t* list;     // FP64 redo: the particles of the list
     const unsigned long long* list_len;
     const __nv_bfloat16* mlp_w;   // learned-estimator weights (BF16)
@@ -547,7 +572,7 @@ struct Src<double, DIM, F> {
     __device__ int side(const Rec& r, uint32_t, int k) const
     {
         const double dk = offset64(a.c, k, xi[k], r.x[k]);
-        return dk > 0.0 ? 1 : (dk < 0.0 ? -1 : 0);
+        return RN<double>::positive(dk) ? 1 : (RN<double>::positive(-dk) ? -1 : 0);
     }
     __device__ int unpack_side(const Rec& r, uint32_t, int k, double (&d)[DIM], double (&b)[F]) const
     {

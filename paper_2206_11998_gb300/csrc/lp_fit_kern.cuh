@@ -6,6 +6,18 @@
 
 namespace lp {
 
+// threads per block of the thread-per-particle kernels.  FP64: a warp, since a
+// warp's time is its count of FP64 instructions, and blocks of four left the SMs
+// 30 % apart at 60k particles (3.1 blocks an SM, in whole blocks)
+template <typename T> struct FitBlock { static constexpr int v = FIT_THREADS; };
+template <> struct FitBlock<double> { static constexpr int v = 32; };
+
+__device__ __forceinline__ int64_t fit_particle(const FitArgs& a)
+{
+    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    return t < a.n && a.order ? (int64_t)a.order[t] : t;
+}
+
 struct StepOut {
     double* x[3];
     double* V;
@@ -411,7 +423,7 @@ __device__ void step_one(const FitArgs& a, const StepOut& o, int64_t i)
 template <typename T, int DIM, bool GATE>
 __global__ void __launch_bounds__(FIT_THREADS, FitOcc<T>::fused) k_step(FitArgs a, StepOut o)
 {
-    int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    const int64_t i = fit_particle(a);
     if (i < a.n) step_one<T, DIM, GATE>(a, o, i);
 }
 
@@ -495,7 +507,7 @@ __global__ void __launch_bounds__(FIT_THREADS, FitOcc<T>::central) k_step_centra
     // keep the block below 48 KB of static shared memory
     constexpr int SD = DEFER ? 64 : 32;
     __shared__ uint32_t stage[SD][NB_PITCH];
-    int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    const int64_t i = fit_particle(a);
     stage_rows<SD>(stage, a.idx, a.c.k_max, i < a.n ? i : -1);
     if (i >= a.n) return;
     central_one<T, DIM, GATE, DEFER>(a, o, i, NbStaged<SD>{a.idx + i * (int64_t)a.c.k_max, &stage[0][threadIdx.x]});
@@ -569,7 +581,8 @@ __global__ void __launch_bounds__(FIT_THREADS, FitOcc<T>::plain) k_step_plain(Fi
 {
     __shared__ uint32_t stage[32][NB_PITCH];
     const unsigned long long len = a.plain_ident ? (unsigned long long)a.n : *a.plain_len;
-    const unsigned long long t = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x;
+    const unsigned long long t0 = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x;
+    const unsigned long long t = a.plain_ident ? (unsigned long long)fit_particle(a) : t0;
     stage_rows<32>(stage, a.idx, a.c.k_max, plain_particle(a, t, len));
     if (t < len) plain_one<T, DIM>(a, o, t, &stage[0][threadIdx.x]);
 }
@@ -690,7 +703,7 @@ __global__ void __launch_bounds__(FIT_THREADS, DerivOcc<T, F>::v) k_derivs(FitAr
 {
     constexpr int SD = DEFER ? 64 : 32;
     __shared__ uint32_t stage[SD][NB_PITCH];
-    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    const int64_t i = fit_particle(a);
     stage_rows<SD>(stage, a.idx, a.c.k_max, i < a.n ? i : -1);
     if (i >= a.n) return;
     derivs_one<T, DIM, F, DEFER>(a, o, i, NbStaged<SD>{a.idx + i * (int64_t)a.c.k_max, &stage[0][threadIdx.x]});
@@ -762,7 +775,7 @@ __device__ void onesided_one(const FitArgs& a, double* out, int f_real, int64_t 
 template <int DIM, int F>
 __global__ void __launch_bounds__(FIT_THREADS) k_onesided(FitArgs a, double* out, int f_real)
 {
-    int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    const int64_t i = fit_particle(a);
     if (i < a.n) onesided_one<DIM, F>(a, out, f_real, i);
 }
 
@@ -865,6 +878,8 @@ cudaError_t launch_derivs_f32(int dim, int F, const FitArgs& a, const DerivOut& 
 cudaError_t launch_derivs_f64(int dim, int F, const FitArgs& a, const DerivOut& o, cudaStream_t s);
 cudaError_t launch_onesided_f32(int dim, const FitArgs& a, double* out, int f_real, cudaStream_t s);
 cudaError_t launch_onesided_f64(int dim, const FitArgs& a, double* out, int f_real, cudaStream_t s);
+// FP64 fits: the particles by falling list length to order[n] (bins: 2 (KMAX + 1) words)
+cudaError_t order_by_count(int64_t n, const uint32_t* count, unsigned int* bins, uint32_t* order, cudaStream_t s);
 // the FP64 redo of the particles a.list (a.list_len of them, on the device) that
 // an FP32 pass listed (lp_fit_f64_redo.cu)
 cudaError_t launch_step_redo(int dim, const FitArgs& a, const StepOut& o, cudaStream_t s);
@@ -898,43 +913,46 @@ inline bool split_defers_t(const FitArgs& a)
     return IsF32<T>::v && a.refine_list && a.c.refine == LP_REFINE_AUTO;
 }
 
+template <typename T>
 inline unsigned fit_blocks(const FitArgs& a)
 {
-    return (unsigned)((a.n + FIT_THREADS - 1) / FIT_THREADS);
+    return (unsigned)((a.n + FitBlock<T>::v - 1) / FitBlock<T>::v);
 }
 
 template <typename T, int DIM, int F>
 cudaError_t launch_derivs(const FitArgs& a, const DerivOut& o, cudaStream_t s)
 {
-    const unsigned b = fit_blocks(a);
+    const unsigned b = fit_blocks<T>(a);
+    constexpr int B = FitBlock<T>::v;
     if constexpr (IsF32<T>::v) {
         if (split_defers_t<T>(a)) {
             FitArgs r = a;
             r.c.refine = LP_REFINE_ALWAYS;
-            k_derivs<T, DIM, F, true><<<b, FIT_THREADS, 0, s>>>(a, o);
+            k_derivs<T, DIM, F, true><<<b, B, 0, s>>>(a, o);
             k_derivs_refine<T, DIM, F><<<152u * 4u, FIT_THREADS, 0, s>>>(r, o);
             return cudaGetLastError();
         }
     }
-    k_derivs<T, DIM, F, false><<<b, FIT_THREADS, 0, s>>>(a, o);
+    k_derivs<T, DIM, F, false><<<b, B, 0, s>>>(a, o);
     return cudaGetLastError();
 }
 
 #define LP_DEFINE_FIT_LAUNCHERS(T, SUF)                                                         \
     cudaError_t launch_step_##SUF(int dim, const FitArgs& a, const StepOut& o, cudaStream_t s)  \
     {                                                                                           \
-        unsigned b = fit_blocks(a);                                                             \
+        const unsigned b = fit_blocks<T>(a);                                                    \
+        constexpr int B = FitBlock<T>::v;                                                       \
         if (b == 0) return cudaSuccess;                                                         \
         const bool gate = o.features || a.c.estimator == LP_EST_MLP;                           \
         if (dim == 3) {                                                                         \
-            if (gate) k_step<T, 3, true><<<b, FIT_THREADS, 0, s>>>(a, o);                               \
-            else k_step<T, 3, false><<<b, FIT_THREADS, 0, s>>>(a, o);                                   \
+            if (gate) k_step<T, 3, true><<<b, B, 0, s>>>(a, o);                               \
+            else k_step<T, 3, false><<<b, B, 0, s>>>(a, o);                                   \
         } else if (dim == 2) {                                                                  \
-            if (gate) k_step<T, 2, true><<<b, FIT_THREADS, 0, s>>>(a, o);                               \
-            else k_step<T, 2, false><<<b, FIT_THREADS, 0, s>>>(a, o);                                   \
+            if (gate) k_step<T, 2, true><<<b, B, 0, s>>>(a, o);                               \
+            else k_step<T, 2, false><<<b, B, 0, s>>>(a, o);                                   \
         } else {                                                                                \
-            if (gate) k_step<T, 1, true><<<b, FIT_THREADS, 0, s>>>(a, o);                               \
-            else k_step<T, 1, false><<<b, FIT_THREADS, 0, s>>>(a, o);                                   \
+            if (gate) k_step<T, 1, true><<<b, B, 0, s>>>(a, o);                               \
+            else k_step<T, 1, false><<<b, B, 0, s>>>(a, o);                                   \
         }                                                                                       \
         return cudaGetLastError();                                                              \
     }                                                                                           \
@@ -942,42 +960,43 @@ cudaError_t launch_derivs(const FitArgs& a, const DerivOut& o, cudaStream_t s)
                                         cudaStream_t s)                                         \
     {                                                                                           \
         auto split_defers = [](const FitArgs& x) { return split_defers_t<T>(x); };              \
-        unsigned b = (unsigned)((a.n + FIT_THREADS - 1) / FIT_THREADS);                                             \
+        const unsigned b = fit_blocks<T>(a);                                                    \
+        constexpr int B = FitBlock<T>::v;                                                       \
         if (b == 0) return cudaSuccess;                                                         \
         const bool gate = o.features || a.c.estimator == LP_EST_MLP;                           \
         if (split_defers(a)) {                                                                  \
             FitArgs r = a;                                                                      \
             r.c.refine = LP_REFINE_ALWAYS;                                                      \
             if (dim == 3) {                                                                     \
-                if (gate) k_step_central<T, 3, true, true><<<b, FIT_THREADS, 0, s>>>(a, o);    \
-                else k_step_central<T, 3, false, true><<<b, FIT_THREADS, 0, s>>>(a, o);        \
+                if (gate) k_step_central<T, 3, true, true><<<b, B, 0, s>>>(a, o);    \
+                else k_step_central<T, 3, false, true><<<b, B, 0, s>>>(a, o);        \
                 launch_central_refine<T>(3, gate, r, o, s);                             \
-                k_step_plain<T, 3><<<b, FIT_THREADS, 0, s>>>(a, o);                             \
+                k_step_plain<T, 3><<<b, B, 0, s>>>(a, o);                             \
             } else if (dim == 2) {                                                              \
-                if (gate) k_step_central<T, 2, true, true><<<b, FIT_THREADS, 0, s>>>(a, o);    \
-                else k_step_central<T, 2, false, true><<<b, FIT_THREADS, 0, s>>>(a, o);        \
+                if (gate) k_step_central<T, 2, true, true><<<b, B, 0, s>>>(a, o);    \
+                else k_step_central<T, 2, false, true><<<b, B, 0, s>>>(a, o);        \
                 launch_central_refine<T>(2, gate, r, o, s);                             \
-                k_step_plain<T, 2><<<b, FIT_THREADS, 0, s>>>(a, o);                             \
+                k_step_plain<T, 2><<<b, B, 0, s>>>(a, o);                             \
             } else {                                                                            \
-                if (gate) k_step_central<T, 1, true, true><<<b, FIT_THREADS, 0, s>>>(a, o);    \
-                else k_step_central<T, 1, false, true><<<b, FIT_THREADS, 0, s>>>(a, o);        \
+                if (gate) k_step_central<T, 1, true, true><<<b, B, 0, s>>>(a, o);    \
+                else k_step_central<T, 1, false, true><<<b, B, 0, s>>>(a, o);        \
                 launch_central_refine<T>(1, gate, r, o, s);                             \
-                k_step_plain<T, 1><<<b, FIT_THREADS, 0, s>>>(a, o);                             \
+                k_step_plain<T, 1><<<b, B, 0, s>>>(a, o);                             \
             }                                                                                   \
             return cudaGetLastError();                                                          \
         }                                                                                       \
         if (dim == 3) {                                                                         \
-            if (gate) k_step_central<T, 3, true, false><<<b, FIT_THREADS, 0, s>>>(a, o);               \
-            else k_step_central<T, 3, false, false><<<b, FIT_THREADS, 0, s>>>(a, o);                   \
-            k_step_plain<T, 3><<<b, FIT_THREADS, 0, s>>>(a, o);                                         \
+            if (gate) k_step_central<T, 3, true, false><<<b, B, 0, s>>>(a, o);               \
+            else k_step_central<T, 3, false, false><<<b, B, 0, s>>>(a, o);                   \
+            k_step_plain<T, 3><<<b, B, 0, s>>>(a, o);                                         \
         } else if (dim == 2) {                                                                  \
-            if (gate) k_step_central<T, 2, true, false><<<b, FIT_THREADS, 0, s>>>(a, o);               \
-            else k_step_central<T, 2, false, false><<<b, FIT_THREADS, 0, s>>>(a, o);                   \
-            k_step_plain<T, 2><<<b, FIT_THREADS, 0, s>>>(a, o);                                         \
+            if (gate) k_step_central<T, 2, true, false><<<b, B, 0, s>>>(a, o);               \
+            else k_step_central<T, 2, false, false><<<b, B, 0, s>>>(a, o);                   \
+            k_step_plain<T, 2><<<b, B, 0, s>>>(a, o);                                         \
         } else {                                                                                \
-            if (gate) k_step_central<T, 1, true, false><<<b, FIT_THREADS, 0, s>>>(a, o);               \
-            else k_step_central<T, 1, false, false><<<b, FIT_THREADS, 0, s>>>(a, o);                   \
-            k_step_plain<T, 1><<<b, FIT_THREADS, 0, s>>>(a, o);                                         \
+            if (gate) k_step_central<T, 1, true, false><<<b, B, 0, s>>>(a, o);               \
+            else k_step_central<T, 1, false, false><<<b, B, 0, s>>>(a, o);                   \
+            k_step_plain<T, 1><<<b, B, 0, s>>>(a, o);                                         \
         }                                                                                       \
         return cudaGetLastError();                                                              \
     }                                                                                           \

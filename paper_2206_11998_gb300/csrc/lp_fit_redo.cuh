@@ -58,14 +58,6 @@ struct RedoShared {
     int ok[2 * DIM];
 };
 
-// d > 0 and x != 0 from the bits, off the FP64 unit (NaN: as the comparisons)
-__device__ __forceinline__ bool pos_bits(double v)
-{
-    const long long b = __double_as_longlong(v);
-    return b > 0 && b <= 0x7ff0000000000000ll;
-}
-__device__ __forceinline__ bool nonzero_bits(double v) { return (__double_as_longlong(v) << 1) != 0; }
-
 // one stage of Givens::add: the rotation that takes entry ak of weight w into a column with diagonal d
 struct Rotation { double c, s; };
 __device__ __forceinline__ Rotation rotate(double ak, double& w, double& d)
@@ -73,7 +65,7 @@ __device__ __forceinline__ Rotation rotate(double ak, double& w, double& d)
     using O = RN<double>;
     const double wa = O::mul(w, ak);
     const double dn = O::fma(wa, ak, d);
-    const bool live = nonzero_bits(wa) && pos_bits(dn);
+    const bool live = O::nonzero(wa) && O::positive(dn);
     const double inv = live ? O::rcp(dn) : 0.0;
     Rotation q;
     q.s = O::mul(wa, inv);
