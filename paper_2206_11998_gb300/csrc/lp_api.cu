@@ -376,13 +376,14 @@ cudaError_t run_cfl(lp_ctx* c, int64_t n, double cfl, double dt_fixed, double* t
 
 namespace {
 
-// FP64 passes over all particles take them by list length, where a warp's worth
-// of lists is long enough to pay for the ordering's launches
+// FP64 passes over all particles take them by cost, where a warp's worth of
+// lists is long enough to pay for the ordering's launches
 lp_status order_fp64(lp_ctx* c, FitArgs& a, cudaStream_t s)
 {
     if (c->dc.dim == 1 || a.n < 2048) return LP_OK;
-    // (the sort's histogram and the corrections' list are free here)
-    LP_CUDA(order_by_count(a.n, c->nb_count, c->hist, c->refine_list, s));
+    // (the sort's histogram and the FP32 path's lists are free here; the records
+    // hold the positions of the last build)
+    LP_CUDA(order_by_cost(c->dc.dim, a, c->hist, c->redo_list, c->refine_list, s));
     a.order = c->refine_list;
     return LP_OK;
 }

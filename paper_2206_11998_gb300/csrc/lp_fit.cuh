@@ -990,16 +990,14 @@ __device__ __forceinline__ void onesided_all(const Src<T, DIM, F>& src, const NB
         }
 }
 
-// Whether the FP32 central fit would be ill-conditioned (central_fit's result
-// 1): the Gram matrix, its factor and, below NE_RATIO_MIN, the rotations,
-// without right-hand sides.  The matrix's sums, and so the ratio, are bit for
-// bit those of central_fit; half of each record and half of the sums suffice.
+// The ratio of the FP32 central fit from the Gram matrix and its factor, without
+// right-hand sides: its sums, and so the ratio, are bit for bit those of
+// central_fit; half of each record and half of the sums suffice.
 template <int DIM, int F, class NB>
-__device__ __forceinline__ bool central_ill(const Src<float, DIM, F>& src, const NB& nb, int cnt, float invS, float tau)
+__device__ __forceinline__ float gram_ratio(const Src<float, DIM, F>& src, const NB& nb, int cnt, float invS)
 {
     constexpr int N = NU<DIM>::v;
     using Rec = typename Src<float, DIM, F>::Rec;
-    if (cnt < N) return true;
     NormalEqPacked<N, 0> EP;
     EP.zero();
     for_neighbors<true>(src, nb, cnt, [&](uint32_t, const Rec& rec) {
@@ -1015,8 +1013,20 @@ __device__ __forceinline__ bool central_ill(const Src<float, DIM, F>& src, const
     Givens<float, N, 1> G;
     EP.store_gram(E);
     E.factor(G);
-    float ratio = G.ratio();
+    return G.ratio();
+}
+
+// Whether the FP32 central fit would be ill-conditioned (central_fit's result
+// 1): the ratio, from the rotations below NE_RATIO_MIN
+template <int DIM, int F, class NB>
+__device__ __forceinline__ bool central_ill(const Src<float, DIM, F>& src, const NB& nb, int cnt, float invS, float tau)
+{
+    constexpr int N = NU<DIM>::v;
+    using Rec = typename Src<float, DIM, F>::Rec;
+    if (cnt < N) return true;
+    float ratio = gram_ratio(src, nb, cnt, invS);
     if (!(ratio >= NE_RATIO_MIN)) {
+        Givens<float, N, 1> G;
         G.zero();
         for_neighbors<true>(src, nb, cnt, [&](uint32_t, const Rec& rec) {
             float d[DIM], a[N], b[1];

@@ -878,8 +878,8 @@ cudaError_t launch_derivs_f32(int dim, int F, const FitArgs& a, const DerivOut& 
 cudaError_t launch_derivs_f64(int dim, int F, const FitArgs& a, const DerivOut& o, cudaStream_t s);
 cudaError_t launch_onesided_f32(int dim, const FitArgs& a, double* out, int f_real, cudaStream_t s);
 cudaError_t launch_onesided_f64(int dim, const FitArgs& a, double* out, int f_real, cudaStream_t s);
-// FP64 fits: the particles by falling list length to order[n] (bins: 2 (KMAX + 1) words)
-cudaError_t order_by_count(int64_t n, const uint32_t* count, unsigned int* bins, uint32_t* order, cudaStream_t s);
+// FP64 fits: the particles by falling cost to order[n] (cost[n]; bins: 512 words)
+cudaError_t order_by_cost(int dim, const FitArgs& a, unsigned int* bins, uint32_t* cost, uint32_t* order, cudaStream_t s);
 // the FP64 redo of the particles a.list (a.list_len of them, on the device) that
 // an FP32 pass listed (lp_fit_f64_redo.cu)
 cudaError_t launch_step_redo(int dim, const FitArgs& a, const StepOut& o, cudaStream_t s);

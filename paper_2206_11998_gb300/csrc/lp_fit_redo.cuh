@@ -132,12 +132,15 @@ __device__ void systolic_givens(RedoShared<DIM, F>& sm, int cnt)
     __syncwarp();
 }
 
-// the ratio test's value, and x = U^{-1} Z of field f, from the factor in sm
+// The ratio test's value, and x = U^{-1} Z of field f, from the factor in sm.
+// Rolled loops over shared memory here and in the solves below: each runs once
+// per particle, and unrolled the warp waited for instructions (50,000 cycles for
+// the ratio and this solve, most of them for code fetched once).
 template <int NN, int DIM, int F>
 __device__ double factor_ratio(const RedoShared<DIM, F>& sm)
 {
     double lo = sm.d[0], hi = sm.d[0];
-#pragma unroll
+#pragma unroll 1
     for (int k = 1; k < NN; ++k) {
         lo = sm.d[k] < lo ? sm.d[k] : lo;
         hi = sm.d[k] > hi ? sm.d[k] : hi;
@@ -148,16 +151,13 @@ __device__ double factor_ratio(const RedoShared<DIM, F>& sm)
 template <int NN, int DIM, int F>
 __device__ void back_solve(RedoShared<DIM, F>& sm, int f)
 {
-    double x[NN];
-#pragma unroll
+#pragma unroll 1
     for (int k = NN - 1; k >= 0; --k) {
         double s = sm.U[k][NN + f];
-#pragma unroll
-        for (int l = k + 1; l < NN; ++l) s = RN<double>::fma(-sm.U[k][l], x[l], s);
-        x[k] = s;
+#pragma unroll 1
+        for (int l = k + 1; l < NN; ++l) s = RN<double>::fma(-sm.U[k][l], sm.x[l][f], s);
+        sm.x[k][f] = s;
     }
-#pragma unroll
-    for (int k = 0; k < NN; ++k) sm.x[k][f] = x[k];
 }
 
 // The one-sided fits of axis k (one warp; half a warp per side, lane l of it
@@ -321,25 +321,24 @@ __device__ void redo_fits(const FitArgs& a, int64_t i, RedoShared<DIM, F>& sm)
             }
             __syncthreads();
             if (tid < F) {
-                double g[N];
-#pragma unroll
+#pragma unroll 1
                 for (int k = 0; k < N; ++k) {
                     double s = sm.g[k][tid];
-#pragma unroll
-                    for (int l = 0; l < k; ++l) s = O::fma(-sm.U[l][k], g[l], s);
-                    g[k] = s;
+#pragma unroll 1
+                    for (int l = 0; l < k; ++l) s = O::fma(-sm.U[l][k], sm.g[l][tid], s);
+                    sm.g[k][tid] = s;
                 }
-#pragma unroll
-                for (int k = 0; k < N; ++k) g[k] = O::mul(g[k], O::rcp(sm.d[k]));
-#pragma unroll
+#pragma unroll 1
+                for (int k = 0; k < N; ++k) sm.g[k][tid] = O::mul(sm.g[k][tid], O::rcp(sm.d[k]));
+#pragma unroll 1
                 for (int k = N - 1; k >= 0; --k) {
-                    double s = g[k];
-#pragma unroll
-                    for (int l = k + 1; l < N; ++l) s = O::fma(-sm.U[k][l], g[l], s);
-                    g[k] = s;
+                    double s = sm.g[k][tid];
+#pragma unroll 1
+                    for (int l = k + 1; l < N; ++l) s = O::fma(-sm.U[k][l], sm.g[l][tid], s);
+                    sm.g[k][tid] = s;
                 }
-#pragma unroll
-                for (int k = 0; k < N; ++k) sm.x[k][tid] += g[k];
+#pragma unroll 1
+                for (int k = 0; k < N; ++k) sm.x[k][tid] += sm.g[k][tid];
             }
         }
         __syncthreads();
@@ -383,9 +382,26 @@ __device__ void redo_step_block(const FitArgs& a, const StepOut& o, int64_t i, R
         if (sm.state) atomicAdd(a.counters + C_LINEAR, 1ull);
         if (sm.state == 2) atomicAdd(a.counters + C_NOFIT, 1ull);
     }
-    int skip = 0;
-    if (GATE && lane == 0) skip = central_gate<double, DIM, GATE>(a, o, i, L, cd, sm.st) ? 1 : 0;
-    const bool mlp_skip = GATE && __shfl_sync(0xffffffffu, skip, 0) != 0;
+    bool mlp_skip = false;
+    if (GATE && (o.features || c.estimator == LP_EST_MLP)) {
+        // (central_gate's steps, the hidden units a lane each)
+        float xf[MLP_IN];
+        mlp_features<double, DIM>(cd, sm.st, sqrt(a.d2min[i]), L.s0[0], L.s0[F - 1], c.gamma, xf);
+        if (o.features && lane < MLP_IN) {
+            float v = xf[0];
+#pragma unroll
+            for (int k = 1; k < MLP_IN; ++k) v = lane == k ? xf[k] : v;
+            o.features[i * MLP_IN + lane] = v;
+        }
+        if (c.estimator == LP_EST_MLP) {
+            const float pg = mlp_prob_warp(xf, a.mlp_w);
+            mlp_skip = pg < c.mlp_tau_lo;
+            if (lane == 0) {
+                if (o.gate_p) o.gate_p[i] = pg;
+                atomicAdd(a.counters + (mlp_skip ? C_MLP_SKIP : C_MLP_UNCERTAIN), 1ull);
+            }
+        }
+    }
     central_rates<double, DIM>(a, L, cd, cdf, lw);
     const bool plain = !mlp_skip || c.mlp_audit;
     double os[DIM][2][F];
