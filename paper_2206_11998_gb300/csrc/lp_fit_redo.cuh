@@ -134,8 +134,8 @@ __device__ void systolic_givens(RedoShared<DIM, F>& sm, int cnt)
 
 // The ratio test's value, and x = U^{-1} Z of field f, from the factor in sm.
 // Rolled loops over shared memory here and in the solves below: each runs once
-// per particle, and unrolled the warp waited for instructions (50,000 cycles for
-// the ratio and this solve, most of them for code fetched once).
+// per particle, and unrolled they are code that is fetched for one use (the whole
+// kernel 109 us with rolled loops, 113 unrolled, two particles at 131k).
 template <int NN, int DIM, int F>
 __device__ double factor_ratio(const RedoShared<DIM, F>& sm)
 {

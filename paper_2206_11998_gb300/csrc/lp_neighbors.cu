@@ -853,55 +853,68 @@ __global__ void __launch_bounds__(NB_WARPS * 32) k_query(QueryArgs a)
     if (i < a.n) query_one<DIM>(a, bufs[w], i);
 }
 
-// The particles the tiles left, a block each.  They are few (0.3 % of the 2M
-// cloud, 5 % of a cloud of 20k), most with some ten neighbours more than a
-// tile's column holds, some with hundreds among thousands of candidates, so the
-// chain of one particle's work sets the time: by a warp (query_one) it took 100
-// us, two thirds of it in the sort of 64-bit keys in shared memory.  Here the
-// 128 threads of a block test the candidates of all start cells, four each in
-// flight, keep every hit in shared memory, leave out the hits beyond the
-// histogram bin of d2 that holds the NB_CAP-th, and give each of the others its
-// place by counting those that sort before it; the NB_CAP nearest are kept.
-// Particles with more candidates or hits than QL_CAND, QL_HITS, and lists whose
-// last entries tie past the buffer, go through query_one (which prunes by the
-// k_max-th distance) on the first warp.
-constexpr int QL_THREADS = 128;
-constexpr int QL_HITS = 1024;
+// The particles the tiles left, a block each: 4 % of the 2M cloud, whose 65 to 80
+// hits are a few more than a tile's column holds, 8 % of a cloud of 20k, and a
+// few outliers with up to 18,000 candidates.  The threads of a block test the
+// candidates of all start cells, LOADS each in flight, count the hits by bin of
+// d2 and keep them in shared memory; a full buffer is pruned to the hits up to
+// the bin that holds the NB_CAP-th so far, and later ones beyond it are only
+// counted.  Each remaining hit then gets its place by counting those that sort
+// before it; the NB_CAP nearest are kept.  Particles with more candidates than
+// QL_CAND, and lists whose last entries tie past the buffer, go through
+// query_one (which prunes by the k_max-th distance) on the first warp.
+//
+// What bounds it: in small sets the chain of one outlier (20k: 9,600 candidates,
+// 178,000 cycles with 128 threads), so 256 threads with four loads each: 56 us at
+// 20k and 58 at 60k, against 92 and 84 with 128 threads, 169 and 138 with 64; two
+// passes over the candidates of an outlier, without the pruning, took 158 at 20k.
+// In large sets the latency of the many small ones (14,000 cycles each), so 128
+// threads in 14 KB and 12 blocks an SM: 98 us at 2M and 55 at 131k, against 188
+// and 62 with 256 threads, 103 and 65 with 64, 132 and 55 with the two passes.
+template <int THREADS_, int LOADS_, int HITS_, int BLOCKS_>
+struct LeftShape {
+    static constexpr int THREADS = THREADS_, LOADS = LOADS_, HITS = HITS_, BLOCKS = BLOCKS_;   // (blocks an SM)
+};
+using LeftChain = LeftShape<256, 4, 1024, 8>;
+using LeftMany = LeftShape<128, 2, 512, 12>;
+constexpr int QL_SMALL_N = 100000;    // below: LeftChain
 constexpr uint32_t QL_CAND = 32768;
-constexpr int QL_LOADS = 4;           // candidates a thread has in flight
 constexpr int QL_BINS = 256;
-static_assert(QL_BINS == 2 * QL_THREADS, "two bins a thread");
-static_assert(FCAP == 2 * QL_THREADS && NB_CAP == QL_THREADS, "two start cells and one kept hit a thread");
+template <class S>
 struct LeftBuf {
     WarpBuf w;
-    alignas(16) unsigned long long key[QL_HITS + 2];  // float bits of d2 << 32 | id
-    uint32_t j[QL_HITS];
-    uint32_t cstart[FCAP], cexcl[FCAP];
-    uint32_t wsum[QL_THREADS / 32];
-    uint32_t hits, near, last_bin;
+    alignas(16) unsigned long long key[S::HITS + 2];  // float bits of d2 << 32 | id
+    uint32_t j[S::HITS];
+    uint32_t wsum[S::THREADS / 32];
+    uint32_t hits, last_bin;
     uint32_t hist[QL_BINS];           // hits by d2 / R2
 };
 
-template <int DIM>
-__device__ void query_left(const QueryArgs& a, LeftBuf& b, int64_t i)
+template <int DIM, class S>
+__device__ void query_left(const QueryArgs& a, LeftBuf<S>& b, int64_t i)
 {
+    constexpr int QL_THREADS = S::THREADS, QL_LOADS = S::LOADS, QL_HITS = S::HITS;
+    constexpr int QL_CELLS = FCAP / QL_THREADS;      // start cells a thread looks up
+    static_assert(QL_BINS % QL_THREADS == 0 && FCAP % QL_THREADS == 0 && QL_HITS % QL_THREADS == 0, "whole shares");
     const unsigned lane = lane_id();
     const int tid = (int)threadIdx.x, wid = tid >> 5;
     const DevCfg& c = a.c;
     const int mb = c.mbits;
     QueryStart st;
     query_start<DIM, QL_THREADS>(a, b.w, i, st);
-    if (tid == 0) { b.hits = 0; b.near = 0; }
-    b.hist[tid] = 0;
-    b.hist[tid + QL_THREADS] = 0;
+    // the cells' first particles and running counts, where only query_one needs the room
+    uint32_t* const cstart = reinterpret_cast<uint32_t*>(b.w.front[1]);
+    uint32_t* const cexcl = cstart + FCAP;
+    if (tid == 0) b.hits = 0;
+    for (int e = tid; e < QL_BINS; e += QL_THREADS) b.hist[e] = 0;
     __syncthreads();
     const float bin_scale = st.R2f > 0.0f ? (float)QL_BINS / st.R2f : 0.0f;
     auto bin_of = [&](float d2f) { return min(QL_BINS - 1, (int)(d2f * bin_scale)); };   // (monotonic in d2f)
-    // the particles of the start cells within reach, two cells a thread
-    uint32_t cs[2] = {0, 0}, cn[2] = {0, 0};
+    // the particles of the start cells within reach, QL_CELLS cells a thread
+    uint32_t cs[QL_CELLS] = {}, cn[QL_CELLS] = {};
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        const int e = 2 * tid + h;
+    for (int h = 0; h < QL_CELLS; ++h) {
+        const int e = QL_CELLS * tid + h;
         if (e >= st.ncells) continue;
         int l, wv[3], shv[3];
         unpack_cell(b.w.front[0][e], l, wv, shv);
@@ -922,140 +935,165 @@ __device__ void query_left(const QueryArgs& a, LeftBuf& b, int64_t i)
         const uint32_t ce = (uint32_t)(ent >> 32);
         cn[h] = ce > cs[h] ? ce - cs[h] : 0;
     }
-    uint32_t incl = cn[0] + cn[1];
+    uint32_t own = 0;
+#pragma unroll
+    for (int h = 0; h < QL_CELLS; ++h) own += cn[h];
+    uint32_t upto = own;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t v = __shfl_up_sync(0xffffffffu, incl, o);
-        if ((int)lane >= o) incl += v;
+        const uint32_t v = __shfl_up_sync(0xffffffffu, upto, o);
+        if ((int)lane >= o) upto += v;
     }
-    if (lane == 31) b.wsum[wid] = incl;
+    if (lane == 31) b.wsum[wid] = upto;
     __syncthreads();
-    uint32_t before = incl - cn[0] - cn[1], T = 0;
+    uint32_t before = upto - own, T = 0;
 #pragma unroll
     for (int w = 0; w < QL_THREADS / 32; ++w) {
         if (w < wid) before += b.wsum[w];
         T += b.wsum[w];
     }
-    b.cstart[2 * tid] = cs[0];
-    b.cexcl[2 * tid] = before;
-    b.cstart[2 * tid + 1] = cs[1];
-    b.cexcl[2 * tid + 1] = before + cn[0];
+#pragma unroll
+    for (int h = 0; h < QL_CELLS; ++h) {
+        cstart[QL_CELLS * tid + h] = cs[h];
+        cexcl[QL_CELLS * tid + h] = before;
+        before += cn[h];
+    }
     __syncthreads();
-    // pass 0: every hit counted, and kept while there is room; with more than
-    // NB_CAP of them, the bin that holds the NB_CAP-th.  Pass 1, where they did
-    // not all fit: the hits up to that bin.  (T, total and the bins are uniform
-    // over the block.)
+    // The hits are counted by their bin of d2 and kept while there is room; when
+    // the buffer is full, and at the end, those beyond the bin that holds the
+    // NB_CAP-th so far are dropped, and later ones beyond it are only counted.
+    // (T, last and the number of hits kept are uniform over the block.)
     bool small = T <= QL_CAND;
     uint32_t total = 0;
     int last = QL_BINS;
-    for (int pass = 0; small && pass < 2; ++pass) {
-        uint32_t* const kept = pass == 0 ? &b.hits : &b.near;
-        for (uint32_t base = 0; base < T; base += QL_THREADS * QL_LOADS) {
-            uint32_t j[QL_LOADS];
-            float4 ph[QL_LOADS], pl[QL_LOADS];
+    auto prune = [&] {
+        const uint32_t kept = min(b.hits, (uint32_t)QL_HITS);
+        unsigned long long k[QL_HITS / QL_THREADS];
+        uint32_t jk[QL_HITS / QL_THREADS];
 #pragma unroll
-            for (int u = 0; u < QL_LOADS; ++u) {
-                const uint32_t t = base + (uint32_t)(u * QL_THREADS + tid);
-                j[u] = 0xffffffffu;
-                ph[u] = pl[u] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-                if (t >= T) continue;
-                int lo = 0;                                 // the last cell with cexcl <= t
-#pragma unroll
-                for (int s = FCAP / 2; s > 0; s >>= 1)
-                    if (b.cexcl[lo + s] <= t) lo += s;
-                j[u] = b.cstart[lo] + (t - b.cexcl[lo]);
-                ldg256(a.pos4 + 2 * (int64_t)j[u], ph[u], pl[u]);
-            }
-#pragma unroll
-            for (int u = 0; u < QL_LOADS; ++u) {
-                const bool test = j[u] != 0xffffffffu && (int64_t)j[u] != i;
-                const float hj[3] = {ph[u].x, ph[u].y, ph[u].z}, lj[3] = {pl[u].x, pl[u].y, pl[u].z};
-                float d2f = 0.0f;
-#pragma unroll
-                for (int k = 0; k < DIM; ++k) {
-                    float dh = hj[k] - st.hxi[k];
-                    float dl = lj[k] - st.lxi[k];
-                    if (c.periodic[k]) {
-                        if (dh > 0.5f * c.Lper_h[k]) { dh -= c.Lper_h[k]; dl -= c.Lper_l[k]; }
-                        else if (dh < -0.5f * c.Lper_h[k]) { dh += c.Lper_h[k]; dl += c.Lper_l[k]; }
-                    }
-                    const float d = dh + dl;
-                    d2f = fmaf(d, d, d2f);
-                }
-                bool in = test && d2f <= st.R2f * (1.0f - TOL_R);
-                if (test && !in && d2f <= st.R2f * (1.0f + TOL_R))
-                    in = inside64(c, DIM, exact_d2<DIM>(a, i, j[u]), __dmul_rn(a.sm[i], a.sV[i]));
-                const int bin = bin_of(d2f);
-                if (pass == 0) { if (in) atomicAdd(&b.hist[bin], 1u); }
-                else in = in && bin <= last;
-                // (one atomic a warp)
-                const unsigned im = __ballot_sync(0xffffffffu, in);
-                if (!im) continue;
-                uint32_t pos = 0;
-                if (lane == 0) pos = atomicAdd(kept, (uint32_t)__popc(im));
-                pos = __shfl_sync(0xffffffffu, pos, 0) + (uint32_t)__popc(im & ((1u << lane) - 1u));
-                if (in && pos < (uint32_t)QL_HITS) {
-                    b.key[pos] = (unsigned long long)__float_as_uint(d2f) << 32;
-                    b.j[pos] = j[u];
-                }
-            }
+        for (int u = 0; u < QL_HITS / QL_THREADS; ++u) {
+            const uint32_t e = (uint32_t)(u * QL_THREADS + tid);
+            k[u] = e < kept ? b.key[e] : ~0ull;
+            jk[u] = e < kept ? b.j[e] : 0u;
         }
-        __syncthreads();
-        if (pass == 1) break;
-        total = b.hits;
-        if (total <= (uint32_t)NB_CAP) break;
-        const uint32_t h0 = b.hist[2 * tid], h1 = b.hist[2 * tid + 1];
-        uint32_t inc = h0 + h1;
+        uint32_t h[QL_BINS / QL_THREADS], sum = 0;
+#pragma unroll
+        for (int u = 0; u < QL_BINS / QL_THREADS; ++u) {
+            h[u] = b.hist[tid * (QL_BINS / QL_THREADS) + u];
+            sum += h[u];
+        }
+        uint32_t inc = sum;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
             const uint32_t v = __shfl_up_sync(0xffffffffu, inc, o);
             if ((int)lane >= o) inc += v;
         }
         if (lane == 31) b.wsum[wid] = inc;
-        __syncthreads();
-        for (int w = 0; w < wid; ++w) inc += b.wsum[w];
-        const uint32_t exc = inc - h0 - h1, want = (uint32_t)NB_CAP;
-        if (exc < want && want <= exc + h0) b.last_bin = 2 * tid;
-        else if (exc + h0 < want && want <= inc) b.last_bin = 2 * tid + 1;
+        __syncthreads();                    // (all have read the buffer too)
+        total = 0;
+#pragma unroll
+        for (int w = 0; w < QL_THREADS / 32; ++w) {
+            if (w < wid) inc += b.wsum[w];
+            total += b.wsum[w];
+        }
+        uint32_t exc = inc - sum;
+#pragma unroll
+        for (int u = 0; u < QL_BINS / QL_THREADS; ++u) {
+            if (exc < (uint32_t)NB_CAP && (uint32_t)NB_CAP <= exc + h[u])
+                b.last_bin = tid * (QL_BINS / QL_THREADS) + u;
+            exc += h[u];
+        }
+        if (tid == 0) b.hits = 0;
         __syncthreads();
         last = (int)b.last_bin;
-        if (total <= (uint32_t)QL_HITS) break;
-    }
-    uint32_t near = small && total > (uint32_t)QL_HITS ? b.near : total;      // hits in b.key
-    small = small && near <= (uint32_t)QL_HITS;
-    const int m = (int)min(total, (uint32_t)NB_CAP), kmax = c.k_max;
-    if (small && last == QL_BINS) {
-        if (tid < near) b.key[tid] |= a.sid[b.j[tid]];      // (at most NB_CAP hits: their ids)
-    } else if (small) {
-        // their ids, and only those up to the bin: read by all before any is written
-        unsigned long long k[QL_HITS / QL_THREADS];
-        uint32_t jk[QL_HITS / QL_THREADS];
-        unsigned mine = 0;
 #pragma unroll
         for (int u = 0; u < QL_HITS / QL_THREADS; ++u) {
-            const uint32_t e = (uint32_t)(u * QL_THREADS + tid);
-            k[u] = 0;
-            jk[u] = 0;
-            if (e >= near) continue;
-            const unsigned long long kk = b.key[e];
-            if (bin_of(key_d2(kk)) > last) continue;
-            jk[u] = b.j[e];
-            k[u] = kk | a.sid[jk[u]];
-            mine |= 1u << u;
+            const bool in = k[u] != ~0ull && bin_of(key_d2(k[u])) <= last;
+            const unsigned im = __ballot_sync(0xffffffffu, in);
+            if (!im) continue;
+            uint32_t pos = 0;
+            if (lane == 0) pos = atomicAdd(&b.hits, (uint32_t)__popc(im));
+            pos = __shfl_sync(0xffffffffu, pos, 0) + (uint32_t)__popc(im & ((1u << lane) - 1u));
+            if (in) { b.key[pos] = k[u]; b.j[pos] = jk[u]; }
         }
         __syncthreads();
-        if (tid == 0) b.near = 0;
-        __syncthreads();
+    };
+    for (uint32_t base = 0; small && base < T; base += QL_THREADS * QL_LOADS) {
+        uint32_t j[QL_LOADS];
+        float4 ph[QL_LOADS], pl[QL_LOADS];
+        float d2[QL_LOADS];
 #pragma unroll
-        for (int u = 0; u < QL_HITS / QL_THREADS; ++u)
-            if ((mine >> u) & 1u) {
-                const uint32_t pos = atomicAdd(&b.near, 1u);
-                b.key[pos] = k[u];
-                b.j[pos] = jk[u];
+        for (int u = 0; u < QL_LOADS; ++u) {
+            const uint32_t t = base + (uint32_t)(u * QL_THREADS + tid);
+            j[u] = 0xffffffffu;
+            ph[u] = pl[u] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            if (t >= T) continue;
+            int lo = 0;                                 // the last cell with cexcl <= t
+#pragma unroll
+            for (int s = FCAP / 2; s > 0; s >>= 1)
+                if (cexcl[lo + s] <= t) lo += s;
+            j[u] = cstart[lo] + (t - cexcl[lo]);
+            ldg256(a.pos4 + 2 * (int64_t)j[u], ph[u], pl[u]);
+        }
+        unsigned keep = 0;                              // bit u: hit u is to be stored
+#pragma unroll
+        for (int u = 0; u < QL_LOADS; ++u) {
+            const bool test = j[u] != 0xffffffffu && (int64_t)j[u] != i;
+            const float hj[3] = {ph[u].x, ph[u].y, ph[u].z}, lj[3] = {pl[u].x, pl[u].y, pl[u].z};
+            float d2f = 0.0f;
+#pragma unroll
+            for (int k = 0; k < DIM; ++k) {
+                float dh = hj[k] - st.hxi[k];
+                float dl = lj[k] - st.lxi[k];
+                if (c.periodic[k]) {
+                    if (dh > 0.5f * c.Lper_h[k]) { dh -= c.Lper_h[k]; dl -= c.Lper_l[k]; }
+                    else if (dh < -0.5f * c.Lper_h[k]) { dh += c.Lper_h[k]; dl += c.Lper_l[k]; }
+                }
+                const float d = dh + dl;
+                d2f = fmaf(d, d, d2f);
             }
-        __syncthreads();
-        near = b.near;
+            d2[u] = d2f;
+            bool in = test && d2f <= st.R2f * (1.0f - TOL_R);
+            if (test && !in && d2f <= st.R2f * (1.0f + TOL_R))
+                in = inside64(c, DIM, exact_d2<DIM>(a, i, j[u]), __dmul_rn(a.sm[i], a.sV[i]));
+            if (!in) continue;
+            const int bin = bin_of(d2f);
+            atomicAdd(&b.hist[bin], 1u);
+            if (bin <= last) keep |= 1u << u;
+        }
+        for (int tries = 0; ; ++tries) {
+            // (one atomic a warp)
+            uint32_t mine = (uint32_t)__popc(keep), incl = mine;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t v = __shfl_up_sync(0xffffffffu, incl, o);
+                if ((int)lane >= o) incl += v;
+            }
+            uint32_t pos = 0;
+            if (lane == 31 && incl) pos = atomicAdd(&b.hits, incl);
+            pos = __shfl_sync(0xffffffffu, pos, 31) + incl - mine;
+#pragma unroll
+            for (int u = 0; u < QL_LOADS; ++u)
+                if (((keep >> u) & 1u) && pos < (uint32_t)QL_HITS) {
+                    b.key[pos] = (unsigned long long)__float_as_uint(d2[u]) << 32;
+                    b.j[pos++] = j[u];
+                    keep &= ~(1u << u);
+                }
+            if (!__syncthreads_or(keep != 0)) break;
+            if (tries == 1) { small = false; break; }   // one bin holds more than the buffer
+            prune();
+#pragma unroll
+            for (int u = 0; u < QL_LOADS; ++u)
+                if (((keep >> u) & 1u) && bin_of(d2[u]) > last) keep &= ~(1u << u);
+        }
     }
+    __syncthreads();
+    if (small && (last < QL_BINS || b.hits > (uint32_t)NB_CAP)) prune();
+    else total = b.hits;
+    const uint32_t near = b.hits;                                   // hits in b.key
+    const int m = (int)min(total, (uint32_t)NB_CAP), kmax = c.k_max;
+    if (small)
+        for (uint32_t e = tid; e < near; e += QL_THREADS) b.key[e] |= a.sid[b.j[e]];
     if (small) {
         if (tid < 2) b.key[near + tid] = ~0ull;             // pads the last pair
         __syncthreads();
@@ -1099,15 +1137,22 @@ __device__ void query_left(const QueryArgs& a, LeftBuf& b, int64_t i)
     }
 }
 
-template <int DIM>
-__global__ void __launch_bounds__(QL_THREADS) k_query_left(QueryArgs a)
+template <int DIM, class S>
+__global__ void __launch_bounds__(S::THREADS) k_query_left(QueryArgs a)
 {
-    __shared__ LeftBuf b;
+    __shared__ LeftBuf<S> b;
     const unsigned long long len = *a.list_len;
     for (unsigned long long t = blockIdx.x; t < len; t += gridDim.x) {
-        query_left<DIM>(a, b, (int64_t)a.list[t]);
+        query_left<DIM, S>(a, b, (int64_t)a.list[t]);
         __syncthreads();                    // the buffers are reused by the next particle
     }
+}
+
+template <int DIM>
+void launch_left(const QueryArgs& a, cudaStream_t s)
+{
+    if (a.n < QL_SMALL_N) k_query_left<DIM, LeftChain><<<152u * LeftChain::BLOCKS, LeftChain::THREADS, 0, s>>>(a);
+    else k_query_left<DIM, LeftMany><<<152u * LeftMany::BLOCKS, LeftMany::THREADS, 0, s>>>(a);
 }
 
 // the octant-balanced selection (LP_SELECT_OCTANT), warp per particle: every
@@ -2121,9 +2166,8 @@ cudaError_t query_neighbors(lp_ctx* c, int64_t n, cudaStream_t s)
         if (dim == 3) k_query_octant<3><<<fblocks, NB_WARPS * 32, 0, s>>>(a);
         else k_query_octant<2><<<fblocks, NB_WARPS * 32, 0, s>>>(a);
     } else {
-        const unsigned fblocks = 152u * 8u;
-        if (dim == 3) k_query_left<3><<<fblocks, QL_THREADS, 0, s>>>(a);
-        else k_query_left<2><<<fblocks, QL_THREADS, 0, s>>>(a);
+        if (dim == 3) launch_left<3>(a, s);
+        else launch_left<2>(a, s);
     }
     return cudaGetLastError();
 }

@@ -64,6 +64,13 @@ def _cases():
     yield "periodic-3d", _points(r.uniform(0, 1, (3, 4000)), r.uniform(0.05, 0.3, 4000)), dict(
         dim=3, kappa=1.0, k_max=64, periodic=(1, 1, 1), box_hi=(1, 1, 1))
     yield "kh", inputs.kh_2d(30000, 0.03, seed=9), dict(dim=2, kappa=2.2, k_max=40, periodic=(1, 1, 0), box_hi=(1, 1, 1))
+    # as above past the size where the left-over particles change to the smaller blocks
+    p = np.concatenate([r.normal(0, 0.02, (3, 12000)), r.uniform(-1, 1, (3, 89000))], 1)
+    yield "dense-core-many", _points(p, r.uniform(0.01, 0.2, 101000)), dict(dim=3, kappa=1.0, k_max=64)
+    g = np.stack(np.meshgrid(*[np.arange(47.0)] * 3, indexing="ij")).reshape(3, -1)
+    for rad, km in ((3.3, 80), (4.2, 50), (5.1, 20)):
+        yield "lattice-many-%g" % rad, _points(g), dict(dim=3, radius_mode=lp.RADIUS_FIXED, radius=rad, k_max=km)
+    yield "few-kept-2d-many", _points(r.uniform(0, 1, (2, 100000)), 0.03), dict(dim=2, kappa=1.0, k_max=9)
     yield "scattered-2d", _points(r.normal(size=(2, 3000)) ** 5, r.uniform(0.01, 3.0, 3000)), dict(dim=2, kappa=1.0, k_max=33)
 
 
