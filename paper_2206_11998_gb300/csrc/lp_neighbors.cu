@@ -1212,7 +1212,12 @@ constexpr float TQ_GAP = 2.0f;        // in radii
 // a warp per tile; 158 and 162 us at 131k.
 constexpr int TQ_SMALL_N = 200000;
 constexpr int tile_blocks(int W) { return 32 / W; }      // resident blocks per SM
-constexpr int TQ_DENSE_MAX = 4;       // largest group that is not halved when GROUP_DENSE
+// Groups and parts with a region too large and no more particles than this go to the
+// per-particle kernel, whose blocks all run at once, where halving down to single
+// particles is a chain in one block: groups and left-over particles together
+// 98 us at 20k, 124 at 131k, 243 at 2M; with 1 (4 when dense) 109, 139 and 250, with
+// 16 as good on small sets and 260 at 2M, with 32 106, 147 and 379.
+constexpr int TQ_FEW = 8;
 
 template <int W>
 struct TileBuf {
@@ -1340,7 +1345,7 @@ __device__ inline void bitonic_keys(uint32_t (&key)[2])
 // group uses (zero on entry; the other set is zeroed for the next group).
 // Returns 0 when done; otherwise the group's region spans too many cells or
 // candidates, nothing was written, and the caller splits the group into
-// 2^result parts or, GROUP_DENSE and few, hands it to the per-particle kernel
+// 2^result parts or, of a few particles, hands it to the per-particle kernel
 enum { GROUP_DONE = 0, GROUP_DENSE = 3 };
 constexpr uint32_t NO_ENTRY = 0xffffffffu, HANDED = 0xfffffffeu;   // TileBuf::near_j
 template <int DIM, bool PER, int W>
@@ -1854,7 +1859,7 @@ __device__ inline void groups_append(const QueryArgs& a, int64_t i0, unsigned g,
 // the tile of 32 key-ordered particles starting at i0 (< n), one block; par: the
 // parity of the counters of its first group, updated for the next tile.  only:
 // the lanes to take (LISTED: a part of a group that was too large; it is halved
-// here down to single particles, where the whole tile's too-large groups are
+// here down to a few particles, where the whole tile's too-large groups are
 // listed, so that no block works through a long series of halves while the
 // others are done: on the 131k cloud such tiles ran for 300 us)
 template <int DIM, bool PER, int W, bool LISTED>
@@ -1898,13 +1903,12 @@ __device__ __forceinline__ void tile_tile(const QueryArgs& a, TileBuf<W>& b, int
             const int r = tile_group<DIM, PER, W>(a, b, i, ((grp >> lane) & 1u) != 0u, sim, t, par);
             const int pc = __popc(grp);
             if (r == GROUP_DONE || threadIdx.x >= 32) continue;
-            if (pc > TQ_DENSE_MAX || (r != GROUP_DENSE && pc >= 2)) groups_append(a, i0, grp, max(1, pc >> (r + 1)));
+            if (pc > TQ_FEW) groups_append(a, i0, grp, max(1, pc >> (r + 1)));
             else list_append(a, ((grp >> lane) & 1u) != 0u, (uint32_t)i);
             continue;
         }
         // the part, halved (by key order: the halves are smaller regions) while
-        // its region is too large; single particles, and few particles among
-        // several times too many candidates, go to the per-particle kernel
+        // its region is too large; parts of a few go to the per-particle kernel
         unsigned stk[8];
         int sp = 0;
         stk[sp++] = grp;
@@ -1913,7 +1917,7 @@ __device__ __forceinline__ void tile_tile(const QueryArgs& a, TileBuf<W>& b, int
             const int r = tile_group<DIM, PER, W>(a, b, i, ((g >> lane) & 1u) != 0u, sim, t, par);
             if (r == GROUP_DONE) continue;
             const int pc = __popc(g);
-            if (pc > TQ_DENSE_MAX || (r != GROUP_DENSE && pc >= 2)) {
+            if (pc > TQ_FEW) {
                 unsigned lo = 0, gg = g;                // the first pc / 2 members
                 for (int q = 0; q < pc / 2; ++q) { lo |= gg & (0u - gg); gg &= gg - 1; }
                 stk[sp++] = g & ~lo;
