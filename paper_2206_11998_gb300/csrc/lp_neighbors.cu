@@ -538,6 +538,37 @@ __device__ inline void octant_ranks(const QueryArgs& a, WarpBuf& b, int m, int64
     }
 }
 
+// The selection from the entries b.key/b.j[0..m), sorted by (d2, id), which hold
+// all members of a rank up to R: ranks below R and the first rem of rank R, in
+// (d2, id) order, and the particle's counts.  One warp.
+template <int DIM>
+__device__ inline void octant_store(const QueryArgs& a, WarpBuf& b, int m, int64_t i, const float (&hi)[3],
+                                    const float (&li)[3], uint32_t R, uint32_t rem, uint32_t total)
+{
+    const unsigned lane = lane_id(), lt = (1u << lane) - 1u;
+    const uint32_t kmax = (uint32_t)a.c.k_max;
+    int w = 0;
+    uint32_t taken_r = 0;
+    octant_ranks<DIM>(a, b, m, i, hi, li, [&](int e0, bool valid, int, uint32_t rank) {
+        const int e = e0 + (int)lane;
+        const bool atR = valid && rank == R;
+        const unsigned bR = __ballot_sync(0xffffffffu, atR);
+        const bool keep = valid && (rank < R || (atR && taken_r + (uint32_t)__popc(bR & lt) < rem));
+        taken_r += (uint32_t)__popc(bR);
+        const unsigned km = __ballot_sync(0xffffffffu, keep);
+        if (keep) a.idx[i * (int64_t)kmax + w + __popc(km & lt)] = b.j[e];
+        w += __popc(km);
+    });
+    if (lane == 0) {
+        a.count[i] = (uint32_t)w;
+        a.total[i] = min(total, 4u * kmax);
+        // the nearest member is kept (rank 0, nearest of the rank-0 members)
+        a.d2min[i] = w > 0 ? exact_d2<DIM>(a, i, b.j[0]) : INFINITY;
+        if (total > kmax) atomicAdd(a.counters + C_OVERFLOW, 1ull);
+        atomicMax(a.counters + C_MAXCOUNT, (unsigned long long)total);
+    }
+}
+
 // Octant-balanced selection (LP_SELECT_OCTANT; Sec. 2.2 step 4: the top
 // members of a neighbour list cover all directions).  When more than k_max
 // particles lie inside the radius, the k_max kept are the first by (rank, d2,
@@ -819,27 +850,7 @@ __device__ void query_one_octant(const QueryArgs& a, WarpBuf& b, int64_t i)
             if (m > 0) compact();          // bounds for the next level
         });
     compact();                                               // m <= sum_o q_o, sorted
-    // ---- the selection, in (d2, id) order: ranks below R, and the first rem of rank R
-    int w = 0;
-    uint32_t taken_r = 0;
-    octant_ranks<DIM>(a, b, m, i, st.hxi, st.lxi, [&](int e0, bool valid, int, uint32_t rank) {
-        const int e = e0 + (int)lane;
-        const bool atR = valid && rank == R;
-        const unsigned bR = __ballot_sync(0xffffffffu, atR);
-        const bool keep = valid && (rank < R || (atR && taken_r + (uint32_t)__popc(bR & lt) < rem));
-        taken_r += (uint32_t)__popc(bR);
-        const unsigned km = __ballot_sync(0xffffffffu, keep);
-        if (keep) a.idx[i * (int64_t)kmax + w + __popc(km & lt)] = b.j[e];
-        w += __popc(km);
-    });
-    if (lane == 0) {
-        a.count[i] = (uint32_t)w;
-        a.total[i] = min(total, 4u * kmax);
-        // the nearest member is kept (rank 0, nearest of the rank-0 members)
-        a.d2min[i] = w > 0 ? exact_d2<DIM>(a, i, b.j[0]) : INFINITY;
-        if (total > kmax) atomicAdd(a.counters + C_OVERFLOW, 1ull);
-        atomicMax(a.counters + C_MAXCOUNT, (unsigned long long)total);
-    }
+    octant_store<DIM>(a, b, m, i, st.hxi, st.lxi, R, rem, total);
     __syncwarp();
 }
 
@@ -869,33 +880,52 @@ __global__ void __launch_bounds__(NB_WARPS * 32) k_query(QueryArgs a)
 // 20k and 58 at 60k, against 92 and 84 with 128 threads, 169 and 138 with 64; two
 // passes over the candidates of an outlier, without the pruning, took 158 at 20k.
 // In large sets the latency of the many small ones (14,000 cycles each), so 128
-// threads in 14 KB and 12 blocks an SM: 98 us at 2M and 55 at 131k, against 188
-// and 62 with 256 threads, 103 and 65 with 64, 132 and 55 with the two passes.
-template <int THREADS_, int LOADS_, int HITS_, int BLOCKS_>
+// threads in 14 KB and 12 blocks an SM, at the price of a few spills: 84 us at 2M
+// and 52 at 131k, against 103 and 55 with 8 blocks of 56 registers, and before
+// that 188 and 62 with 256 threads, 103 and 65 with 64, 132 and 55 with two passes.
+template <int THREADS_, int LOADS_, int HITS_, int BLOCKS_, int RESIDENT_>
 struct LeftShape {
-    static constexpr int THREADS = THREADS_, LOADS = LOADS_, HITS = HITS_, BLOCKS = BLOCKS_;   // (blocks an SM)
+    static constexpr int THREADS = THREADS_, LOADS = LOADS_, HITS = HITS_;
+    static constexpr int BLOCKS = BLOCKS_, RESIDENT = RESIDENT_;   // blocks launched and resident an SM
 };
-using LeftChain = LeftShape<256, 4, 1024, 8>;
-using LeftMany = LeftShape<128, 2, 512, 12>;
+using LeftChain = LeftShape<256, 4, 1024, 8, 4>;
+using LeftMany = LeftShape<128, 2, 512, 12, 12>;
+using LeftOct = LeftShape<256, 4, 1024, 24, 4>;   // LP_SELECT_OCTANT
 constexpr int QL_SMALL_N = 100000;    // below: LeftChain
-constexpr uint32_t QL_CAND = 32768;
+constexpr uint32_t QL_CAND = 32768, QL_OCT_CAND = 131072;   // (octants: where a warp would take as long)
 constexpr int QL_BINS = 256;
-template <class S>
+constexpr int QL_OCT_BINS = 128;      // an octant's, with LP_SELECT_OCTANT
+template <class S, bool OCT>
 struct LeftBuf {
     WarpBuf w;
-    alignas(16) unsigned long long key[S::HITS + 2];  // float bits of d2 << 32 | id
+    alignas(16) unsigned long long key[S::HITS + 2];  // float bits of d2 << 32 | id (or, before, octant)
     uint32_t j[S::HITS];
     uint32_t wsum[S::THREADS / 32];
-    uint32_t hits, last_bin;
-    uint32_t hist[QL_BINS];           // hits by d2 / R2
+    uint32_t hits;
+    uint32_t last_bin[OCT ? 8 : 1];   // hits beyond (of an octant) are not kept
+    uint32_t n_oct[8], rank;          // OCT: hits of each octant; the largest rank that may be kept
+    alignas(16) uint32_t hist[OCT ? 8 * QL_OCT_BINS : QL_BINS];   // hits by (octant and) d2 / R2
 };
 
-template <int DIM, class S>
-__device__ void query_left(const QueryArgs& a, LeftBuf<S>& b, int64_t i)
+// OCT: the octant-balanced selection (query_one_octant states its rule) by the
+// same passes.  The largest rank R that can be kept is found from the octants'
+// counts so far, each octant's hits beyond the bin of its (R + 1)-th are dropped
+// (R only falls as hits are added, so none of them could be kept later), and what
+// is left loses those with more than R nearer members in their octant, ties
+// excepted, before it is sorted.  By a warp (query_one_octant) the outliers of the
+// jet (1M particles, 3,300 left over, up to 11,900 hits among 45,000 candidates,
+// two million cycles each) set the kernel's time, 1,500 us.  Here 550 us, much of
+// it on candidates that only had to be counted: with the nearest cells first and
+// those left out that nothing waits for 298, with four resident blocks instead of
+// three 283, and with blocks to spare for the uneven particles 244.
+template <int DIM, class S, bool OCT>
+__device__ void query_left(const QueryArgs& a, LeftBuf<S, OCT>& b, int64_t i)
 {
+    constexpr int NO = 1 << DIM, BINS = OCT ? QL_OCT_BINS : QL_BINS;
     constexpr int QL_THREADS = S::THREADS, QL_LOADS = S::LOADS, QL_HITS = S::HITS;
     constexpr int QL_CELLS = FCAP / QL_THREADS;      // start cells a thread looks up
-    static_assert(QL_BINS % QL_THREADS == 0 && FCAP % QL_THREADS == 0 && QL_HITS % QL_THREADS == 0, "whole shares");
+    static_assert(OCT ? QL_THREADS == 256 && KMAX < 256 : QL_BINS % QL_THREADS == 0, "whole shares");
+    static_assert(FCAP % QL_THREADS == 0 && QL_HITS % QL_THREADS == 0, "whole shares");
     const unsigned lane = lane_id();
     const int tid = (int)threadIdx.x, wid = tid >> 5;
     const DevCfg& c = a.c;
@@ -906,12 +936,25 @@ __device__ void query_left(const QueryArgs& a, LeftBuf<S>& b, int64_t i)
     uint32_t* const cstart = reinterpret_cast<uint32_t*>(b.w.front[1]);
     uint32_t* const cexcl = cstart + FCAP;
     if (tid == 0) b.hits = 0;
-    for (int e = tid; e < QL_BINS; e += QL_THREADS) b.hist[e] = 0;
+    for (int e = tid; e < (OCT ? 8 * BINS : BINS); e += QL_THREADS) b.hist[e] = 0;
+    if (tid < (OCT ? 8 : 1)) b.last_bin[tid] = BINS;
     __syncthreads();
-    const float bin_scale = st.R2f > 0.0f ? (float)QL_BINS / st.R2f : 0.0f;
-    auto bin_of = [&](float d2f) { return min(QL_BINS - 1, (int)(d2f * bin_scale)); };   // (monotonic in d2f)
+    const float bin_scale = st.R2f > 0.0f ? (float)BINS / st.R2f : 0.0f;
+    auto bin_of = [&](float d2f) { return min(BINS - 1, (int)(d2f * bin_scale)); };   // (monotonic in d2f)
+    // the bin must not exceed last_bin; an octant keeps what may tie with its last
+    auto keeps = [&](float d2f, unsigned o) {
+        return bin_of(OCT ? d2f * (1.0f - 2.0f * TOL_T) : d2f) <= (int)b.last_bin[OCT ? o : 0u];
+    };
     // the particles of the start cells within reach, QL_CELLS cells a thread
     uint32_t cs[QL_CELLS] = {}, cn[QL_CELLS] = {};
+    // OCT (a cell a thread): its least distance, the octants it meets, and whether
+    // it lies half a cell off: those come second, when the nearest have set the
+    // bins, and the ones that no octant needs and no count waits for are left out
+    float dmin = 0.0f;
+    unsigned touched = 0;
+    bool far = false;
+    // octants with bit k set (offset along k >= 0), per axis
+    constexpr unsigned AXIS_SET[3] = {DIM == 3 ? 0xAAu : 0xAu, 0xCCu, 0xF0u};
 #pragma unroll
     for (int h = 0; h < QL_CELLS; ++h) {
         const int e = QL_CELLS * tid + h;
@@ -921,52 +964,38 @@ __device__ void query_left(const QueryArgs& a, LeftBuf<S>& b, int64_t i)
         uint32_t q[3] = {0, 0, 0};
         const float size = ldexpf(1.0f, mb - l), period = ldexpf(1.0f, mb);
         float dmin2 = 0.0f;
+        unsigned tc = (1u << NO) - 1u;
 #pragma unroll
         for (int k = 0; k < DIM; ++k) {
             q[k] = (uint32_t)wv[k];
-            const float lo = (float)wv[k] * size + (float)shv[k] * period;
-            const float dn = fmaxf(0.0f, fmaxf(lo - st.tq[k], st.tq[k] - (lo + size)));
+            const float lo = (float)wv[k] * size + (float)shv[k] * period, hi = lo + size;
+            const float dn = fmaxf(0.0f, fmaxf(lo - st.tq[k], st.tq[k] - hi));
             dmin2 += dn * dn;
+            if (lo > st.tq[k] + 2.0f) tc &= AXIS_SET[k];               // every offset > 0
+            else if (hi < st.tq[k] - 2.0f) tc &= ~AXIS_SET[k];         // every offset < 0
         }
-        if (sqrtf(dmin2) >= st.Rout) continue;
+        const float dc = sqrtf(dmin2);
+        if (dc >= st.Rout) continue;
+        if (OCT) {
+            dmin = dc;
+            touched = tc;
+            far = 2.0f * dc >= size;
+        }
         const uint64_t code = (st.sim << (DIM * l)) | morton<DIM>(q);
         const unsigned long long ent = a.cells[a.level_off[l] + (int64_t)code];
         cs[h] = (uint32_t)ent;
         const uint32_t ce = (uint32_t)(ent >> 32);
         cn[h] = ce > cs[h] ? ce - cs[h] : 0;
     }
-    uint32_t own = 0;
-#pragma unroll
-    for (int h = 0; h < QL_CELLS; ++h) own += cn[h];
-    uint32_t upto = own;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t v = __shfl_up_sync(0xffffffffu, upto, o);
-        if ((int)lane >= o) upto += v;
-    }
-    if (lane == 31) b.wsum[wid] = upto;
-    __syncthreads();
-    uint32_t before = upto - own, T = 0;
-#pragma unroll
-    for (int w = 0; w < QL_THREADS / 32; ++w) {
-        if (w < wid) before += b.wsum[w];
-        T += b.wsum[w];
-    }
-#pragma unroll
-    for (int h = 0; h < QL_CELLS; ++h) {
-        cstart[QL_CELLS * tid + h] = cs[h];
-        cexcl[QL_CELLS * tid + h] = before;
-        before += cn[h];
-    }
-    __syncthreads();
     // The hits are counted by their bin of d2 and kept while there is room; when
     // the buffer is full, and at the end, those beyond the bin that holds the
     // NB_CAP-th so far are dropped, and later ones beyond it are only counted.
-    // (T, last and the number of hits kept are uniform over the block.)
-    bool small = T <= QL_CAND;
+    // (T, b.last_bin and the number of hits kept are uniform over the block.)
+    bool small = true;
     uint32_t total = 0;
-    int last = QL_BINS;
+    bool pruned = false;
     auto prune = [&] {
+        pruned = true;
         const uint32_t kept = min(b.hits, (uint32_t)QL_HITS);
         unsigned long long k[QL_HITS / QL_THREADS];
         uint32_t jk[QL_HITS / QL_THREADS];
@@ -976,39 +1005,74 @@ __device__ void query_left(const QueryArgs& a, LeftBuf<S>& b, int64_t i)
             k[u] = e < kept ? b.key[e] : ~0ull;
             jk[u] = e < kept ? b.j[e] : 0u;
         }
-        uint32_t h[QL_BINS / QL_THREADS], sum = 0;
+        if constexpr (OCT) {
+            // a warp per octant, four bins a lane
+            static_assert(QL_OCT_BINS == 128, "four bins a lane");
+            const uint4 h4 = *reinterpret_cast<const uint4*>(&b.hist[(wid & 7) * BINS + 4 * lane]);
+            const uint32_t h[4] = {h4.x, h4.y, h4.z, h4.w}, sum = h4.x + h4.y + h4.z + h4.w;
+            uint32_t inc = sum;
 #pragma unroll
-        for (int u = 0; u < QL_BINS / QL_THREADS; ++u) {
-            h[u] = b.hist[tid * (QL_BINS / QL_THREADS) + u];
-            sum += h[u];
-        }
-        uint32_t inc = sum;
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t v = __shfl_up_sync(0xffffffffu, inc, o);
+                if ((int)lane >= o) inc += v;
+            }
+            if (lane == 31) b.n_oct[wid] = inc;
+            __syncthreads();                    // (all have read the buffer too)
+            total = 0;
+            uint32_t upto = 0, below = 0;       // members of a rank up to tid, and below it
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t v = __shfl_up_sync(0xffffffffu, inc, o);
-            if ((int)lane >= o) inc += v;
-        }
-        if (lane == 31) b.wsum[wid] = inc;
-        __syncthreads();                    // (all have read the buffer too)
-        total = 0;
+            for (int q = 0; q < NO; ++q) {
+                total += b.n_oct[q];
+                upto += min(b.n_oct[q], (uint32_t)tid + 1u);
+                below += min(b.n_oct[q], (uint32_t)tid);
+            }
+            const uint32_t kmax = (uint32_t)c.k_max;
+            if (total <= kmax) { if (tid == 0) b.rank = kmax; }
+            else if (below < kmax && kmax <= upto) b.rank = (uint32_t)tid;
+            if (tid == 0) b.hits = 0;
+            __syncthreads();
+            const uint32_t want = b.rank + 1u;
+            uint32_t exc = inc - sum;
 #pragma unroll
-        for (int w = 0; w < QL_THREADS / 32; ++w) {
-            if (w < wid) inc += b.wsum[w];
-            total += b.wsum[w];
-        }
-        uint32_t exc = inc - sum;
+            for (int u = 0; u < 4; ++u) {
+                if (exc < want && want <= exc + h[u]) b.last_bin[wid] = 4 * lane + u;
+                exc += h[u];
+            }
+            __syncthreads();
+        } else {
+            uint32_t h[QL_BINS / QL_THREADS], sum = 0;
 #pragma unroll
-        for (int u = 0; u < QL_BINS / QL_THREADS; ++u) {
-            if (exc < (uint32_t)NB_CAP && (uint32_t)NB_CAP <= exc + h[u])
-                b.last_bin = tid * (QL_BINS / QL_THREADS) + u;
-            exc += h[u];
+            for (int u = 0; u < QL_BINS / QL_THREADS; ++u) {
+                h[u] = b.hist[tid * (QL_BINS / QL_THREADS) + u];
+                sum += h[u];
+            }
+            uint32_t inc = sum;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t v = __shfl_up_sync(0xffffffffu, inc, o);
+                if ((int)lane >= o) inc += v;
+            }
+            if (lane == 31) b.wsum[wid] = inc;
+            __syncthreads();                    // (all have read the buffer too)
+            total = 0;
+#pragma unroll
+            for (int w = 0; w < QL_THREADS / 32; ++w) {
+                if (w < wid) inc += b.wsum[w];
+                total += b.wsum[w];
+            }
+            uint32_t exc = inc - sum;
+#pragma unroll
+            for (int u = 0; u < QL_BINS / QL_THREADS; ++u) {
+                if (exc < (uint32_t)NB_CAP && (uint32_t)NB_CAP <= exc + h[u])
+                    b.last_bin[0] = tid * (QL_BINS / QL_THREADS) + u;
+                exc += h[u];
+            }
+            if (tid == 0) b.hits = 0;
+            __syncthreads();
         }
-        if (tid == 0) b.hits = 0;
-        __syncthreads();
-        last = (int)b.last_bin;
 #pragma unroll
         for (int u = 0; u < QL_HITS / QL_THREADS; ++u) {
-            const bool in = k[u] != ~0ull && bin_of(key_d2(k[u])) <= last;
+            const bool in = k[u] != ~0ull && keeps(key_d2(k[u]), (unsigned)k[u] & 7u);
             const unsigned im = __ballot_sync(0xffffffffu, in);
             if (!im) continue;
             uint32_t pos = 0;
@@ -1018,82 +1082,168 @@ __device__ void query_left(const QueryArgs& a, LeftBuf<S>& b, int64_t i)
         }
         __syncthreads();
     };
-    for (uint32_t base = 0; small && base < T; base += QL_THREADS * QL_LOADS) {
-        uint32_t j[QL_LOADS];
-        float4 ph[QL_LOADS], pl[QL_LOADS];
-        float d2[QL_LOADS];
+    for (int phase = 0; phase < (OCT ? 2 : 1) && small; ++phase) {
+        uint32_t own = 0, cnt[QL_CELLS];
 #pragma unroll
-        for (int u = 0; u < QL_LOADS; ++u) {
-            const uint32_t t = base + (uint32_t)(u * QL_THREADS + tid);
-            j[u] = 0xffffffffu;
-            ph[u] = pl[u] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-            if (t >= T) continue;
-            int lo = 0;                                 // the last cell with cexcl <= t
+        for (int h = 0; h < QL_CELLS; ++h) {
+            if (OCT) {
+                cnt[h] = far == (phase == 1) ? cn[h] : 0;
+                if (phase == 1 && total >= 4u * (uint32_t)c.k_max) {
+                    bool need = false;
 #pragma unroll
-            for (int s = FCAP / 2; s > 0; s >>= 1)
-                if (cexcl[lo + s] <= t) lo += s;
-            j[u] = cstart[lo] + (t - cexcl[lo]);
-            ldg256(a.pos4 + 2 * (int64_t)j[u], ph[u], pl[u]);
-        }
-        unsigned keep = 0;                              // bit u: hit u is to be stored
-#pragma unroll
-        for (int u = 0; u < QL_LOADS; ++u) {
-            const bool test = j[u] != 0xffffffffu && (int64_t)j[u] != i;
-            const float hj[3] = {ph[u].x, ph[u].y, ph[u].z}, lj[3] = {pl[u].x, pl[u].y, pl[u].z};
-            float d2f = 0.0f;
-#pragma unroll
-            for (int k = 0; k < DIM; ++k) {
-                float dh = hj[k] - st.hxi[k];
-                float dl = lj[k] - st.lxi[k];
-                if (c.periodic[k]) {
-                    if (dh > 0.5f * c.Lper_h[k]) { dh -= c.Lper_h[k]; dl -= c.Lper_l[k]; }
-                    else if (dh < -0.5f * c.Lper_h[k]) { dh += c.Lper_h[k]; dl += c.Lper_l[k]; }
+                    for (int q = 0; q < NO; ++q) {
+                        const float cut = sqrtf((float)(b.last_bin[q] + 1u) * (st.R2f / (float)BINS)) * st.inv * (1.0f + 4e-5f) + 1.0f;
+                        need |= ((touched >> q) & 1u) && (b.last_bin[q] >= (uint32_t)BINS - 1u || dmin <= cut);
+                    }
+                    if (!need) cnt[h] = 0;
                 }
-                const float d = dh + dl;
-                d2f = fmaf(d, d, d2f);
+            } else {
+                cnt[h] = cn[h];
             }
-            d2[u] = d2f;
-            bool in = test && d2f <= st.R2f * (1.0f - TOL_R);
-            if (test && !in && d2f <= st.R2f * (1.0f + TOL_R))
-                in = inside64(c, DIM, exact_d2<DIM>(a, i, j[u]), __dmul_rn(a.sm[i], a.sV[i]));
-            if (!in) continue;
-            const int bin = bin_of(d2f);
-            atomicAdd(&b.hist[bin], 1u);
-            if (bin <= last) keep |= 1u << u;
+            own += cnt[h];
         }
-        for (int tries = 0; ; ++tries) {
-            // (one atomic a warp)
-            uint32_t mine = (uint32_t)__popc(keep), incl = mine;
+        uint32_t upto = own;
 #pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const uint32_t v = __shfl_up_sync(0xffffffffu, incl, o);
-                if ((int)lane >= o) incl += v;
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t v = __shfl_up_sync(0xffffffffu, upto, o);
+            if ((int)lane >= o) upto += v;
+        }
+        if (lane == 31) b.wsum[wid] = upto;
+        __syncthreads();
+        uint32_t before = upto - own, T = 0;
+#pragma unroll
+        for (int w = 0; w < QL_THREADS / 32; ++w) {
+            if (w < wid) before += b.wsum[w];
+            T += b.wsum[w];
+        }
+#pragma unroll
+        for (int h = 0; h < QL_CELLS; ++h) {
+            cstart[QL_CELLS * tid + h] = cs[h];
+            cexcl[QL_CELLS * tid + h] = before;
+            before += cnt[h];
+        }
+        __syncthreads();
+        if (T > (OCT ? QL_OCT_CAND : QL_CAND)) { small = false; break; }
+        for (uint32_t base = 0; small && base < T; base += QL_THREADS * QL_LOADS) {
+            uint32_t j[QL_LOADS];
+            float4 ph[QL_LOADS], pl[QL_LOADS];
+            float d2[QL_LOADS];
+            unsigned oct[QL_LOADS];
+#pragma unroll
+            for (int u = 0; u < QL_LOADS; ++u) {
+                const uint32_t t = base + (uint32_t)(u * QL_THREADS + tid);
+                j[u] = 0xffffffffu;
+                ph[u] = pl[u] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                if (t >= T) continue;
+                int lo = 0;                                 // the last cell with cexcl <= t
+#pragma unroll
+                for (int s = FCAP / 2; s > 0; s >>= 1)
+                    if (cexcl[lo + s] <= t) lo += s;
+                j[u] = cstart[lo] + (t - cexcl[lo]);
+                ldg256(a.pos4 + 2 * (int64_t)j[u], ph[u], pl[u]);
             }
-            uint32_t pos = 0;
-            if (lane == 31 && incl) pos = atomicAdd(&b.hits, incl);
-            pos = __shfl_sync(0xffffffffu, pos, 31) + incl - mine;
+            unsigned keep = 0;                              // bit u: hit u is to be stored
 #pragma unroll
-            for (int u = 0; u < QL_LOADS; ++u)
-                if (((keep >> u) & 1u) && pos < (uint32_t)QL_HITS) {
-                    b.key[pos] = (unsigned long long)__float_as_uint(d2[u]) << 32;
-                    b.j[pos++] = j[u];
-                    keep &= ~(1u << u);
+            for (int u = 0; u < QL_LOADS; ++u) {
+                const bool test = j[u] != 0xffffffffu && (int64_t)j[u] != i;
+                const float hj[3] = {ph[u].x, ph[u].y, ph[u].z}, lj[3] = {pl[u].x, pl[u].y, pl[u].z};
+                float d2f = 0.0f;
+#pragma unroll
+                for (int k = 0; k < DIM; ++k) {
+                    float dh = hj[k] - st.hxi[k];
+                    float dl = lj[k] - st.lxi[k];
+                    if (c.periodic[k]) {
+                        if (dh > 0.5f * c.Lper_h[k]) { dh -= c.Lper_h[k]; dl -= c.Lper_l[k]; }
+                        else if (dh < -0.5f * c.Lper_h[k]) { dh += c.Lper_h[k]; dl += c.Lper_l[k]; }
+                    }
+                    const float d = dh + dl;
+                    d2f = fmaf(d, d, d2f);
                 }
-            if (!__syncthreads_or(keep != 0)) break;
-            if (tries == 1) { small = false; break; }   // one bin holds more than the buffer
+                d2[u] = d2f;
+                bool in = test && d2f <= st.R2f * (1.0f - TOL_R);
+                if (test && !in && d2f <= st.R2f * (1.0f + TOL_R))
+                    in = inside64(c, DIM, exact_d2<DIM>(a, i, j[u]), __dmul_rn(a.sm[i], a.sV[i]));
+                oct[u] = 0;
+                if (!in) continue;
+                if (OCT) oct[u] = (unsigned)octant_split<DIM>(a, i, j[u], st.hxi, st.lxi, hj, lj);
+                atomicAdd(&b.hist[oct[u] * BINS + bin_of(d2f)], 1u);
+                if (keeps(d2f, oct[u])) keep |= 1u << u;
+            }
+            for (int tries = 0; ; ++tries) {
+                // (one atomic a warp)
+                uint32_t mine = (uint32_t)__popc(keep), incl = mine;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const uint32_t v = __shfl_up_sync(0xffffffffu, incl, o);
+                    if ((int)lane >= o) incl += v;
+                }
+                uint32_t pos = 0;
+                if (lane == 31 && incl) pos = atomicAdd(&b.hits, incl);
+                pos = __shfl_sync(0xffffffffu, pos, 31) + incl - mine;
+#pragma unroll
+                for (int u = 0; u < QL_LOADS; ++u)
+                    if (((keep >> u) & 1u) && pos < (uint32_t)QL_HITS) {
+                        b.key[pos] = (unsigned long long)__float_as_uint(d2[u]) << 32 | oct[u];
+                        b.j[pos++] = j[u];
+                        keep &= ~(1u << u);
+                    }
+                if (!__syncthreads_or(keep != 0)) break;
+                if (tries == 1) { small = false; break; }   // one bin holds more than the buffer
+                prune();
+#pragma unroll
+                for (int u = 0; u < QL_LOADS; ++u)
+                    if (((keep >> u) & 1u) && !keeps(d2[u], oct[u])) keep &= ~(1u << u);
+            }
+        }
+        if (OCT && small) {
+            __syncthreads();
             prune();
-#pragma unroll
-            for (int u = 0; u < QL_LOADS; ++u)
-                if (((keep >> u) & 1u) && bin_of(d2[u]) > last) keep &= ~(1u << u);
         }
     }
     __syncthreads();
-    if (small && (last < QL_BINS || b.hits > (uint32_t)NB_CAP)) prune();
-    else total = b.hits;
-    const uint32_t near = b.hits;                                   // hits in b.key
-    const int m = (int)min(total, (uint32_t)NB_CAP), kmax = c.k_max;
+    if (!OCT && small) {
+        if (pruned || b.hits > (uint32_t)NB_CAP) prune();
+        else total = b.hits;
+    }
+    uint32_t near = b.hits;                                         // hits in b.key
+    if constexpr (OCT) {
+        unsigned long long k[QL_HITS / QL_THREADS];
+        uint32_t jk[QL_HITS / QL_THREADS];
+        unsigned mine = 0;
+        if (near > (uint32_t)NB_CAP && small) {
+#pragma unroll
+            for (int u = 0; u < QL_HITS / QL_THREADS; ++u) {
+                const uint32_t e = (uint32_t)(u * QL_THREADS + tid);
+                if (e >= near) continue;
+                k[u] = b.key[e];
+                jk[u] = b.j[e];
+                uint32_t r = 0;                                     // members of the octant surely before
+#pragma unroll 4
+                for (uint32_t q = 0; q < near; ++q) {
+                    const unsigned long long v = b.key[q];
+                    r += ((unsigned)v == (unsigned)k[u] && key_d2(v) * (1.0f + 2.0f * TOL_T) < key_d2(k[u])) ? 1u : 0u;
+                }
+                if (r <= b.rank) mine |= 1u << u;
+            }
+            __syncthreads();
+            if (tid == 0) b.hits = 0;
+            __syncthreads();
+#pragma unroll
+            for (int u = 0; u < QL_HITS / QL_THREADS; ++u)
+                if ((mine >> u) & 1u) {
+                    const uint32_t pos = atomicAdd(&b.hits, 1u);
+                    b.key[pos] = k[u];
+                    b.j[pos] = jk[u];
+                }
+            __syncthreads();
+            near = b.hits;
+        }
+        small = small && near <= (uint32_t)NB_CAP;
+    }
+    const int m = OCT ? (int)near : (int)min(total, (uint32_t)NB_CAP), kmax = c.k_max;
     if (small)
-        for (uint32_t e = tid; e < near; e += QL_THREADS) b.key[e] |= a.sid[b.j[e]];
+        for (uint32_t e = tid; e < near; e += QL_THREADS)
+            b.key[e] = (b.key[e] & ~0xffffffffull) | a.sid[b.j[e]];
     if (small) {
         if (tid < 2) b.key[near + tid] = ~0ull;             // pads the last pair
         __syncthreads();
@@ -1113,6 +1263,18 @@ __device__ void query_left(const QueryArgs& a, LeftBuf<S>& b, int64_t i)
     }
     __syncthreads();
     if (wid != 0) return;
+    if constexpr (OCT) {
+        if (!small) {
+            query_one_octant<DIM>(a, b.w, i);
+            return;
+        }
+        order_ties<DIM>(a, b.w, m, i);
+        uint32_t below = 0;                                         // members of a rank below R
+#pragma unroll
+        for (int q = 0; q < NO; ++q) below += min(b.n_oct[q], b.rank);
+        octant_store<DIM>(a, b.w, m, i, st.hxi, st.lxi, b.rank, (uint32_t)kmax - min(below, (uint32_t)kmax), total);
+        return;
+    }
     if (small && total > (uint32_t)NB_CAP) {
         // hits past the buffer may only be missed by a run of ties that spans
         // from the last entry kept to the buffer's end
@@ -1137,13 +1299,13 @@ __device__ void query_left(const QueryArgs& a, LeftBuf<S>& b, int64_t i)
     }
 }
 
-template <int DIM, class S>
-__global__ void __launch_bounds__(S::THREADS) k_query_left(QueryArgs a)
+template <int DIM, class S, bool OCT>
+__global__ void __launch_bounds__(S::THREADS, S::RESIDENT) k_query_left(QueryArgs a)
 {
-    __shared__ LeftBuf<S> b;
+    __shared__ LeftBuf<S, OCT> b;
     const unsigned long long len = *a.list_len;
     for (unsigned long long t = blockIdx.x; t < len; t += gridDim.x) {
-        query_left<DIM, S>(a, b, (int64_t)a.list[t]);
+        query_left<DIM, S, OCT>(a, b, (int64_t)a.list[t]);
         __syncthreads();                    // the buffers are reused by the next particle
     }
 }
@@ -1151,28 +1313,21 @@ __global__ void __launch_bounds__(S::THREADS) k_query_left(QueryArgs a)
 template <int DIM>
 void launch_left(const QueryArgs& a, cudaStream_t s)
 {
-    if (a.n < QL_SMALL_N) k_query_left<DIM, LeftChain><<<152u * LeftChain::BLOCKS, LeftChain::THREADS, 0, s>>>(a);
-    else k_query_left<DIM, LeftMany><<<152u * LeftMany::BLOCKS, LeftMany::THREADS, 0, s>>>(a);
+    const bool octant = a.c.select == LP_SELECT_OCTANT;
+    if (octant) k_query_left<DIM, LeftOct, true><<<152u * LeftOct::BLOCKS, LeftOct::THREADS, 0, s>>>(a);
+    else if (a.n < QL_SMALL_N) k_query_left<DIM, LeftChain, false><<<152u * LeftChain::BLOCKS, LeftChain::THREADS, 0, s>>>(a);
+    else k_query_left<DIM, LeftMany, false><<<152u * LeftMany::BLOCKS, LeftMany::THREADS, 0, s>>>(a);
 }
 
-// the octant-balanced selection (LP_SELECT_OCTANT), warp per particle: every
-// particle, or the particles of a list.  A kernel of its own so that the
-// nearest-first kernel keeps its register budget.
+// the octant-balanced selection of every particle, a warp each.  A kernel of its
+// own so that the nearest-first kernel keeps its register budget.
 template <int DIM>
 __global__ void __launch_bounds__(NB_WARPS * 32) k_query_octant(QueryArgs a)
 {
     __shared__ WarpBuf bufs[NB_WARPS];
     const int w = threadIdx.x >> 5;
-    WarpBuf& b = bufs[w];
-    if (a.list) {
-        const unsigned long long len = *a.list_len;
-        for (unsigned long long t = (unsigned long long)blockIdx.x * NB_WARPS + w; t < len;
-             t += (unsigned long long)gridDim.x * NB_WARPS)
-            query_one_octant<DIM>(a, b, (int64_t)a.list[t]);
-    } else {
-        const int64_t i = (int64_t)blockIdx.x * NB_WARPS + w;
-        if (i < a.n) query_one_octant<DIM>(a, b, i);
-    }
+    const int64_t i = (int64_t)blockIdx.x * NB_WARPS + w;
+    if (i < a.n) query_one_octant<DIM>(a, bufs[w], i);
 }
 
 // ---------------------------------------------------------------------------
@@ -2165,14 +2320,8 @@ cudaError_t query_neighbors(lp_ctx* c, int64_t n, cudaStream_t s)
     if (e != cudaSuccess) return e;
     a.list = c->redo_list;
     a.list_len = c->counters + C_QFB_LEN;
-    if (octant) {
-        const unsigned fblocks = 152u * 4u;
-        if (dim == 3) k_query_octant<3><<<fblocks, NB_WARPS * 32, 0, s>>>(a);
-        else k_query_octant<2><<<fblocks, NB_WARPS * 32, 0, s>>>(a);
-    } else {
-        if (dim == 3) launch_left<3>(a, s);
-        else launch_left<2>(a, s);
-    }
+    if (dim == 3) launch_left<3>(a, s);
+    else launch_left<2>(a, s);
     return cudaGetLastError();
 }
 

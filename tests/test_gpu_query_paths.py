@@ -74,7 +74,11 @@ def _cases():
     yield "scattered-2d", _points(r.normal(size=(2, 3000)) ** 5, r.uniform(0.01, 3.0, 3000)), dict(dim=2, kappa=1.0, k_max=33)
 
 
+OCTANT = ("cloud-20k", "few-kept", "dense-core", "lattice-2.3-64", "lattice-3.3-20", "lattice-3.3-80", "lattice-4.2-50",
+          "lattice-7.1-64", "shell", "n1", "n33", "n129", "periodic-0.2", "periodic-0.49", "periodic-3d", "kh", "scattered-2d")
+
 ALL = list(_cases())
+ALL += [(name + "-octant", st, dict(cfg, select=lp.SELECT_OCTANT)) for name, st, cfg in ALL if name in OCTANT]
 
 
 @pytest.mark.parametrize("name,st,cfg", ALL, ids=[c[0] for c in ALL])
