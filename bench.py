@@ -83,11 +83,11 @@ def fit_flops_per_particle(m: float, refined_frac: float = 0.0, plain_frac: floa
 FIT_TRAFFIC_BPP_2M = 1058.8
 
 # warp instructions per particle of one neighbour query (k_query_tile and the
-# per-particle kernel over the particles it leaves; smsp__inst_executed.sum from
+# kernels over the groups and particles it leaves; smsp__inst_executed.sum from
 # the same capture): the query is bound by instruction issue (integer, shuffle
 # and shared-memory work), so it is reported against the SM issue peak of
 # 4 warp instructions per clock per SM.
-QUERY_INST_PP_2M = 886.0
+QUERY_INST_PP_2M = 914.0
 
 # nominal FP64 rate of a GB300 (TFLOP/s): the roofline of the FP64 fit
 FP64_PEAK_TFLOPS = 1.25
@@ -549,8 +549,8 @@ def run_ours(args):
         q_ms = phases["neighbor-query"][0] / args.steps
         issue_peak = n_sm * 4 * sm_max * 1e6
         q_ach = QUERY_INST_PP_2M * n / (q_ms * 1e-3)
-        tile_kernel = "k_query_tile_q (warp work queue)" if sched & lp.SCHED_QUEUE_QUERY else "k_query_tile"
-        query_roofline = {"kernel": tile_kernel + " + k_query (neighbour query)", "bound": "issue",
+        tile_kernel = "k_query_tile_q (work queue)" if sched & lp.SCHED_QUEUE_QUERY else "k_query_tile"
+        query_roofline = {"kernel": tile_kernel + " + k_query_groups + k_query_left (neighbour query)", "bound": "issue",
                           "achieved": q_ach, "peak": issue_peak, "unit": "warp instructions/s",
                           "frac": q_ach / issue_peak, "inst_per_particle": QUERY_INST_PP_2M,
                           "peak_source": "%d SM x 4 schedulers x 1 warp instruction per clock x %.0f MHz" % (n_sm, sm_max),

@@ -206,8 +206,8 @@ typedef struct {
     int64_t kernel_launches;   /* kernels this context launched (host-side count) */
     int64_t n_mlp_skip;        /* particle-steps the learned estimator declared unflagged */
     int64_t n_mlp_miss;        /* ... of which the plain estimator flags (audit mode) */
-    int64_t n_query_fallback;  /* particles of the last neighbour build listed by the warp-per-particle
-                                  query (more than 64 neighbours, or a tile spread over too many cells) */
+    int64_t n_query_fallback;  /* particles of the last neighbour build listed by the per-particle
+                                  query (more than 64 neighbours, or part of a tile spread over too many cells) */
     int64_t n_refined;         /* FP32 central fits of lp_step that ran the correction pass */
 } lp_stats;
 
@@ -559,15 +559,15 @@ lp_status lp_graph_launch(lp_ctx *ctx, lp_stream stream);
  *                     and LW rates) to a compacted list; a second kernel runs
  *                     the one-sided fits, estimator and blend over that list.
  *   neighbour query:
- *     (default)            one warp per 32 key-ordered particles (tiles), with
- *                          the per-particle kernel for the particles a tile
- *                          leaves (more than 64 neighbours, scattered groups).
+ *     (default)            one block per 32 key-ordered particles (tiles), with
+ *                          a block per particle for those a tile leaves (more
+ *                          than 64 neighbours, scattered groups).
  *     LP_SCHED_QUERY_WARP  one warp per particle for every particle.
  *   work distribution (same results):
  *     LP_SCHED_QUEUE_QUERY the tile kernel runs as a grid of resident blocks
- *                          whose warps take their next tile of 32 particles
- *                          from a device work counter (a warp work queue)
- *                          instead of one tile per warp of the launch.
+ *                          that take their next tile of 32 particles from a
+ *                          device work counter (a work queue) instead of one
+ *                          tile per block of the launch.
  *     LP_SCHED_QUEUE_FIT   likewise for the SPLIT schedule's two kernels
  *                          (32 particles, then 32 list entries, per take);
  *                          FP32 path.

@@ -2,7 +2,8 @@
 // templates instantiated for FP32 (lp_fit_f32.cu, lp_fit_f32_refine.cu) and
 // FP64 (lp_fit_f64.cu).
 //
-// Schedule: one thread per particle; no stencil is staged and no lane idles.
+// Schedule: one thread per particle (the FP64 redo of a few particles takes a
+// block each, lp_fit_redo.cuh); no stencil is staged and no lane idles.
 // The overdetermined GFD system of Sec. 2.1 (and its 1D/3D analogues) is
 // solved in one of two forms, both with the factor, the right-hand sides of
 // all fields and the running row in registers:

@@ -1,4 +1,5 @@
-// lp_fit_f64.cu -- FP64 instantiations of the fit and step kernels.
+// lp_fit_f64.cu -- FP64 instantiations of the fit and step kernels (32-thread
+// blocks), and the order of particles by cost that they run in.
 #include "lp_fit_kern.cuh"
 
 namespace lp {
