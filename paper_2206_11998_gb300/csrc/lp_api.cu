@@ -612,7 +612,7 @@ static lp_status build(lp_ctx* c, lp_particles* p, cudaStream_t s)
         LP_CUDA(build_front(c, p, n_old, s));
     }
     if (!small) {
-        Phase ph(c, LP_PH_SORT, 3 * radix_passes(c), s);
+        Phase ph(c, LP_PH_SORT, radix_pass_launches(n) * radix_passes(c), s);
         LP_CUDA(radix_sort(c, n, s));
     }
     if (c->gather_wait) {

@@ -356,6 +356,7 @@ bool front_is_small(const lp_ctx* c, int64_t n);          // build_front sorts a
 int front_launches(const lp_ctx* c, int64_t n);
 cudaError_t build_front(lp_ctx* c, const lp_particles* p, int64_t n_old, cudaStream_t s);
 int radix_passes(const lp_ctx* c);
+int radix_pass_launches(int64_t n);
 cudaError_t radix_sort(lp_ctx* c, int64_t n, cudaStream_t s);
 cudaError_t gather(lp_ctx* c, const lp_particles* p, cudaStream_t s);
 cudaError_t gather_geometry(lp_ctx* c, const lp_particles* p, cudaStream_t s);

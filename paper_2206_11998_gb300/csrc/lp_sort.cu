@@ -456,6 +456,14 @@ __global__ void k_keys(int64_t n, const double* __restrict__ x0, const double* _
 
 // ---- LSD radix sort, RS_BITS-bit digits ----------------------------------
 
+// Up to RS_FEW tiles, the downsweep's blocks sum the tiles' counts themselves
+// (FEW: counts by tile, read coalesced, independent loads) instead of a scan kernel
+// between: three passes 42 -> 33 us at 20k particles and 43 -> 39 at 131k (65 tiles),
+// and a launch less each, 14 and 15 us of the step.  A tile more costs a pass 0.04 us:
+// at 96 both take the same without the launch, at 245 the kernel takes 57 -> 73.
+constexpr int64_t RS_FEW = 96;
+
+template <bool FEW>
 __global__ void k_rs_upsweep(int64_t n, const uint64_t* __restrict__ keys, int shift,
                              uint32_t* __restrict__ counts, int64_t nblocks)
 {
@@ -469,8 +477,8 @@ __global__ void k_rs_upsweep(int64_t n, const uint64_t* __restrict__ keys, int s
         if (i < n) atomicAdd(&h[(keys[i] >> shift) & RS_MASK], 1u);
     }
     __syncthreads();
-    counts[(int64_t)threadIdx.x * nblocks + blockIdx.x] = h[threadIdx.x];
-    counts[(int64_t)(threadIdx.x + RS_THREADS) * nblocks + blockIdx.x] = h[threadIdx.x + RS_THREADS];
+    for (int d = (int)threadIdx.x; d < RS_BINS; d += RS_THREADS)
+        counts[FEW ? (int64_t)blockIdx.x * RS_BINS + d : (int64_t)d * nblocks + blockIdx.x] = h[d];
 }
 
 // Per digit d (one block each): exclusive scan of the block counts
@@ -513,6 +521,7 @@ __global__ void __launch_bounds__(1024) k_rs_scan(uint32_t* counts, int64_t nblo
 // Scatter of one tile of RS_TILE keys: each warp ranks its 512 consecutive keys
 // round by round (match on the digit), the warps' digit counts are scanned
 // once per tile, and every key goes to digit base + block offset + rank.
+template <bool FEW>
 __global__ void __launch_bounds__(RS_THREADS)
 k_rs_downsweep(int64_t n, const uint64_t* __restrict__ kin, const uint32_t* __restrict__ vin,
                uint64_t* __restrict__ kout, uint32_t* __restrict__ vout, int shift,
@@ -525,7 +534,21 @@ k_rs_downsweep(int64_t n, const uint64_t* __restrict__ kin, const uint32_t* __re
     // digit bases: exclusive scan of the digit totals, thread t owning digits
     // 2t and 2t + 1, plus this tile's offset within each digit
     {
-        const uint32_t v0 = totals[2 * t], v1 = totals[2 * t + 1];
+        uint32_t v0 = 0, v1 = 0, c0 = 0, c1 = 0;
+        if (FEW) {
+#pragma unroll 8
+            for (int b = 0; b < (int)nblocks; ++b) {
+                const uint2 h = reinterpret_cast<const uint2*>(counts)[(int64_t)b * (RS_BINS / 2) + t];
+                if (b == (int)blockIdx.x) { c0 = v0; c1 = v1; }
+                v0 += h.x;
+                v1 += h.y;
+            }
+        } else {
+            v0 = totals[2 * t];
+            v1 = totals[2 * t + 1];
+            c0 = counts[(int64_t)(2 * t) * nblocks + blockIdx.x];
+            c1 = counts[(int64_t)(2 * t + 1) * nblocks + blockIdx.x];
+        }
         const uint32_t v = v0 + v1;
         uint32_t x = v;
 #pragma unroll
@@ -538,8 +561,8 @@ k_rs_downsweep(int64_t n, const uint64_t* __restrict__ kin, const uint32_t* __re
         uint32_t add = 0;
         for (int ww = 0; ww < w; ++ww) add += wc[0][ww];
         const uint32_t b0 = add + x - v;
-        dbase[2 * t] = b0 + counts[(int64_t)(2 * t) * nblocks + blockIdx.x];
-        dbase[2 * t + 1] = b0 + v0 + counts[(int64_t)(2 * t + 1) * nblocks + blockIdx.x];
+        dbase[2 * t] = b0 + c0;
+        dbase[2 * t + 1] = b0 + v0 + c1;
     }
     __syncthreads();
     for (int d = lane; d < RS_BINS; d += 32) wc[w][d] = 0;
@@ -993,18 +1016,32 @@ cudaError_t build_front(lp_ctx* c, const lp_particles* p, int64_t n_old, cudaStr
     return cudaGetLastError();
 }
 
+// one pass of the sort; hist: RS_BINS x (tiles + 1) words
+static void radix_pass(int64_t n, int shift, uint32_t* hist, const uint64_t* kin, const uint32_t* vin, uint64_t* kout,
+                       uint32_t* vout, cudaStream_t s)
+{
+    const int64_t nblocks = (n + RS_TILE - 1) / RS_TILE;
+    const unsigned nb = (unsigned)nblocks;
+    uint32_t* const totals = hist + RS_BINS * nblocks;
+    if (nblocks <= RS_FEW) {
+        k_rs_upsweep<true><<<nb, RS_THREADS, 0, s>>>(n, kin, shift, hist, nblocks);
+        k_rs_downsweep<true><<<nb, RS_THREADS, 0, s>>>(n, kin, vin, kout, vout, shift, hist, totals, nblocks);
+        return;
+    }
+    k_rs_upsweep<false><<<nb, RS_THREADS, 0, s>>>(n, kin, shift, hist, nblocks);
+    k_rs_scan<<<RS_BINS, 1024, 0, s>>>(hist, nblocks, totals);
+    k_rs_downsweep<false><<<nb, RS_THREADS, 0, s>>>(n, kin, vin, kout, vout, shift, hist, totals, nblocks);
+}
+
+int radix_pass_launches(int64_t n) { return (n + RS_TILE - 1) / RS_TILE <= RS_FEW ? 2 : 3; }
+
 int radix_passes(const lp_ctx* c) { return (c->sort_hi_bit - c->sort_lo_bit + RS_BITS - 1) / RS_BITS; }
 
 cudaError_t radix_sort(lp_ctx* c, int64_t n, cudaStream_t s)
 {
-    int64_t nblocks = (n + RS_TILE - 1) / RS_TILE;
     int cur = 0;
     for (int sh = c->sort_lo_bit; sh < c->sort_hi_bit; sh += RS_BITS) {
-        uint32_t* totals = c->hist + RS_BINS * nblocks;
-        k_rs_upsweep<<<(unsigned)nblocks, RS_THREADS, 0, s>>>(n, c->keys[cur], sh, c->hist, nblocks);
-        k_rs_scan<<<RS_BINS, 1024, 0, s>>>(c->hist, nblocks, totals);
-        k_rs_downsweep<<<(unsigned)nblocks, RS_THREADS, 0, s>>>(n, c->keys[cur], c->vals[cur], c->keys[cur ^ 1],
-                                                                c->vals[cur ^ 1], sh, c->hist, totals, nblocks);
+        radix_pass(n, sh, c->hist, c->keys[cur], c->vals[cur], c->keys[cur ^ 1], c->vals[cur ^ 1], s);
         cur ^= 1;
     }
     c->keys_sorted = c->keys[cur];
@@ -1212,13 +1249,9 @@ extern "C" lp_status lp_sort_keys_noalloc(int32_t dim, int64_t n, const double* 
     if (dim == 3) k_keys<3><<<gb, 256, 0, s>>>(n, x0, p1, p2, grid, nullptr, MORTON_BITS, keys[0], vals[0]);
     else if (dim == 2) k_keys<2><<<gb, 256, 0, s>>>(n, x0, p1, p2, grid, nullptr, MORTON_BITS, keys[0], vals[0]);
     else k_keys<1><<<gb, 256, 0, s>>>(n, x0, p1, p2, grid, nullptr, MORTON_BITS, keys[0], vals[0]);
-    int64_t nblocks = (n + RS_TILE - 1) / RS_TILE;
     int cur = 0;
     for (int sh = lo_bit; sh < hi_bit; sh += RS_BITS) {
-        k_rs_upsweep<<<(unsigned)nblocks, RS_THREADS, 0, s>>>(n, keys[cur], sh, hist, nblocks);
-        k_rs_scan<<<RS_BINS, 1024, 0, s>>>(hist, nblocks, hist + RS_BINS * nblocks);
-        k_rs_downsweep<<<(unsigned)nblocks, RS_THREADS, 0, s>>>(n, keys[cur], vals[cur], keys[cur ^ 1],
-                                                                vals[cur ^ 1], sh, hist, hist + RS_BINS * nblocks, nblocks);
+        radix_pass(n, sh, hist, keys[cur], vals[cur], keys[cur ^ 1], vals[cur ^ 1], s);
         cur ^= 1;
     }
     k_copy_sorted<<<gb, 256, 0, s>>>(n, keys[cur], vals[cur], keys_out, perm_out);

@@ -1,6 +1,7 @@
 """The one-block front of a build (extent, cube, keys, sort; up to 8192 particles)
 and the general one above it: the order of the particles against numpy's stable
-sort of the same keys, at sizes around the block's rounds and the rule's limit,
+sort of the same keys, at sizes around the block's rounds, the rule's limit and
+the general sort's (up to 96 tiles of 2048 without a scan kernel),
 with shuffled, ordered, reversed and equal positions; builds of changing size on
 one context (the table entries of the build before are cleared); and a captured
 step replayed against eager ones."""
@@ -21,7 +22,7 @@ def _built():
     ensure_built()
 
 
-SIZES = [1, 2, 33, 1023, 1024, 1025, 2049, 8191, 8192, 8193, 20000]
+SIZES = [1, 2, 33, 1023, 1024, 1025, 2049, 8191, 8192, 8193, 20000, 131071, 96 * 2048, 96 * 2048 + 1]
 
 
 def _points(kind, d, n):
