@@ -64,6 +64,9 @@ def _cases():
     yield "periodic-3d", _points(r.uniform(0, 1, (3, 4000)), r.uniform(0.05, 0.3, 4000)), dict(
         dim=3, kappa=1.0, k_max=64, periodic=(1, 1, 1), box_hi=(1, 1, 1))
     yield "kh", inputs.kh_2d(30000, 0.03, seed=9), dict(dim=2, kappa=2.2, k_max=40, periodic=(1, 1, 0), box_hi=(1, 1, 1))
+    # more particles at one point than the left-over particles' buffers hold: all in one bin
+    p = np.concatenate([np.full((3, 1500), 0.5), r.uniform(0, 1, (3, 1500))], 1)
+    yield "clump", _points(p, 0.2), dict(dim=3, kappa=1.0, k_max=40)
     # as above past the size where the left-over particles change to the smaller blocks
     p = np.concatenate([r.normal(0, 0.02, (3, 12000)), r.uniform(-1, 1, (3, 89000))], 1)
     yield "dense-core-many", _points(p, r.uniform(0.01, 0.2, 101000)), dict(dim=3, kappa=1.0, k_max=64)
@@ -74,7 +77,7 @@ def _cases():
     yield "scattered-2d", _points(r.normal(size=(2, 3000)) ** 5, r.uniform(0.01, 3.0, 3000)), dict(dim=2, kappa=1.0, k_max=33)
 
 
-OCTANT = ("cloud-20k", "few-kept", "dense-core", "lattice-2.3-64", "lattice-3.3-20", "lattice-3.3-80", "lattice-4.2-50",
+OCTANT = ("cloud-20k", "few-kept", "dense-core", "clump", "lattice-2.3-64", "lattice-3.3-20", "lattice-3.3-80", "lattice-4.2-50",
           "lattice-7.1-64", "shell", "n1", "n33", "n129", "periodic-0.2", "periodic-0.49", "periodic-3d", "kh", "scattered-2d")
 
 ALL = list(_cases())
