@@ -1368,7 +1368,10 @@ constexpr float TQ_GAP = 2.0f;        // in radii
 // few and a tile's own time counts: 50 us at 20k against 78 with two and 194 with
 // a warp per tile; 158 and 162 us at 131k.
 constexpr int TQ_SMALL_N = 200000;
-constexpr int tile_blocks(int W) { return 32 / W; }      // resident blocks per SM
+// Resident blocks per SM.  14 of two warps in 2D, whose periodic arithmetic spills at
+// 64 registers: 1.38 ms against 1.41 for 24 shear layers of 2.5M particles in all; in
+// 3D 1.956 against 1.940 at 2M, and 18 or 20 blocks 2.30 and 2.41.
+constexpr int tile_blocks(int W, int dim) { return dim == 2 && W == 2 ? 14 : 32 / W; }
 // Groups and parts with a region too large and no more particles than this go to the
 // per-particle kernel, whose blocks all run at once, where halving down to single
 // particles is a chain in one block: groups and left-over particles together
@@ -2094,7 +2097,7 @@ __device__ __forceinline__ void tile_init(TileBuf<W>& b)
 }
 
 template <int DIM, bool PER, int W>
-__global__ void __launch_bounds__(W * 32, tile_blocks(W)) k_query_tile(QueryArgs a)
+__global__ void __launch_bounds__(W * 32, tile_blocks(W, DIM)) k_query_tile(QueryArgs a)
 {
     __shared__ TileBuf<W> b;
     tile_init(b);
@@ -2104,7 +2107,7 @@ __global__ void __launch_bounds__(W * 32, tile_blocks(W)) k_query_tile(QueryArgs
 
 // the parts of the groups that were too large
 template <int DIM, bool PER, int W>
-__global__ void __launch_bounds__(W * 32, tile_blocks(W)) k_query_groups(QueryArgs a)
+__global__ void __launch_bounds__(W * 32, tile_blocks(W, DIM)) k_query_groups(QueryArgs a)
 {
     __shared__ TileBuf<W> b;
     tile_init(b);
@@ -2120,7 +2123,7 @@ __global__ void __launch_bounds__(W * 32, tile_blocks(W)) k_query_groups(QueryAr
 // Persistent form (LP_SCHED_QUEUE_QUERY): a grid of resident blocks that take
 // their next tile from a.queue until none is left.
 template <int DIM, bool PER, int W>
-__global__ void __launch_bounds__(W * 32, tile_blocks(W)) k_query_tile_q(QueryArgs a)
+__global__ void __launch_bounds__(W * 32, tile_blocks(W, DIM)) k_query_tile_q(QueryArgs a)
 {
     __shared__ TileBuf<W> b;
     tile_init(b);
@@ -2231,7 +2234,7 @@ namespace {
 template <int DIM, bool PER, int W>
 cudaError_t launch_tiles_w(const QueryArgs& a, bool queue, cudaStream_t s)
 {
-    const unsigned tiles = (unsigned)((a.n + 31) / 32), resident = 152u * tile_blocks(W);
+    const unsigned tiles = (unsigned)((a.n + 31) / 32), resident = 152u * tile_blocks(W, DIM);
     if (queue) {
         // as many blocks as are resident at once, never more than the tiles need
         int dev = 0, sms = 0, per_sm = 0;
