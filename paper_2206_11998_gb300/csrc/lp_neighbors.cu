@@ -201,7 +201,24 @@ struct QueryStart {
     float inv;                     // quantised units per length
     float R2f, Rq, Rout, Rin;      // squared radius; radius and box margins, quantised units
     int ncells;                    // start cells in b.front[0]
+    // Bit k: the cells within reach span more than a period of axis k (a radius
+    // above 3/8 of the box), and each was taken once, at one of its images.  The
+    // image says nothing about the cell's distance then (another may be nearer):
+    // cell_axis leaves the axis out of it.
+    unsigned full;
     uint64_t sim;
+
+    // the least and the largest distance along axis k from the particle to the
+    // cell [lo, hi]; false where the cell's image does not bound them
+    __device__ __forceinline__ bool cell_axis(int k, float lo, float hi, float& dn, float& df) const
+    {
+        dn = fmaxf(0.0f, fmaxf(lo - tq[k], tq[k] - hi));
+        df = fmaxf(tq[k] - lo, hi - tq[k]);
+        if (!((full >> k) & 1u)) return true;
+        dn = 0.0f;
+        df = INFINITY;
+        return false;
+    }
 };
 
 template <int DIM, int THREADS = 32>
@@ -248,6 +265,7 @@ __device__ __forceinline__ void query_start(const QueryArgs& a, WarpBuf& b, int6
     const float cell_scale = ldexpf(1.0f, -(mb - l0));
     long long clo[3] = {0, 0, 0};
     int nc[3] = {1, 1, 1};
+    st.full = 0u;
 #pragma unroll
     for (int k = 0; k < DIM; ++k) {
         long long a0 = (long long)floorf((st.tq[k] - Rq - 2.0f) * cell_scale);
@@ -257,6 +275,7 @@ __device__ __forceinline__ void query_start(const QueryArgs& a, WarpBuf& b, int6
             a1 = max(0ll, min(a1, ncell_axis - 1));
         } else if (a1 - a0 + 1 > ncell_axis) {
             a1 = a0 + ncell_axis - 1;
+            st.full |= 1u << k;
         }
         clo[k] = a0;
         nc[k] = (int)(a1 - a0 + 1);
@@ -297,7 +316,6 @@ __device__ void query_one(const QueryArgs& a, WarpBuf& b, int64_t i)
     query_start<DIM>(a, b, i, st);
     const float* hxi = st.hxi;
     const float* lxi = st.lxi;
-    const float* tq = st.tq;
     const float inv = st.inv;
     const float R2f = st.R2f, Rout = st.Rout, Rin = st.Rin;
     const int ncells = st.ncells;
@@ -335,9 +353,8 @@ __device__ void query_one(const QueryArgs& a, WarpBuf& b, int64_t i)
 #pragma unroll
                 for (int k = 0; k < DIM; ++k) {
                     q[k] = (uint32_t)wv[k];
-                    float lo = (float)wv[k] * size + (float)shv[k] * period, hi = lo + size;
-                    float dn = fmaxf(0.0f, fmaxf(lo - tq[k], tq[k] - hi));
-                    float df = fmaxf(tq[k] - lo, hi - tq[k]);
+                    float lo = (float)wv[k] * size + (float)shv[k] * period, hi = lo + size, dn, df;
+                    st.cell_axis(k, lo, hi, dn, df);
                     dmin2 += dn * dn;
                     dmax2 += df * df;
                 }
@@ -637,10 +654,11 @@ __device__ void query_one_octant(const QueryArgs& a, WarpBuf& b, int64_t i)
                     for (int k = 0; k < DIM; ++k) {
                         q[k] = (uint32_t)wv[k];
                         const float lo = (float)wv[k] * size + (float)shv[k] * period, hi = lo + size;
-                        const float dn = fmaxf(0.0f, fmaxf(lo - st.tq[k], st.tq[k] - hi));
-                        const float df = fmaxf(st.tq[k] - lo, hi - st.tq[k]);
+                        float dn, df;
+                        const bool near = st.cell_axis(k, lo, hi, dn, df);
                         dmin2 += dn * dn;
                         dmax2 += df * df;
+                        if (!near) continue;
                         if (lo > st.tq[k] + 2.0f) touched &= AXIS_SET[k];          // every offset > 0
                         else if (hi < st.tq[k] - 2.0f) touched &= ~AXIS_SET[k];    // every offset < 0
                     }
@@ -970,8 +988,10 @@ __device__ void query_left(const QueryArgs& a, LeftBuf<S, OCT>& b, int64_t i)
         for (int k = 0; k < DIM; ++k) {
             q[k] = (uint32_t)wv[k];
             const float lo = (float)wv[k] * size + (float)shv[k] * period, hi = lo + size;
-            const float dn = fmaxf(0.0f, fmaxf(lo - st.tq[k], st.tq[k] - hi));
+            float dn, df;
+            const bool near = st.cell_axis(k, lo, hi, dn, df);
             dmin2 += dn * dn;
+            if (!near) continue;
             if (lo > st.tq[k] + 2.0f) tc &= AXIS_SET[k];               // every offset > 0
             else if (hi < st.tq[k] - 2.0f) tc &= ~AXIS_SET[k];         // every offset < 0
         }
