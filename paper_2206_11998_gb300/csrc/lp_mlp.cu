@@ -143,10 +143,13 @@ __device__ void mlp_block_grad(MlpShared& sm, MlpSample first, const float* __re
             for (int k = 0; k < MLP_IN; ++k) a = fmaf(wu[k], q[k], a);
             const bool live = a > 0.0f;
             gw2 = fmaf(d, live ? a : 0.0f, gw2);
-            const float dh = live ? d * w2u : 0.0f;
-            gb += dh;
+            // (not dh = 0 for a dead unit: 0 times a feature that is not finite is NaN)
+            if (live) {
+                const float dh = d * w2u;
+                gb += dh;
 #pragma unroll
-            for (int k = 0; k < MLP_IN; ++k) gu[k] = fmaf(dh, q[k], gu[k]);
+                for (int k = 0; k < MLP_IN; ++k) gu[k] = fmaf(dh, q[k], gu[k]);
+            }
         }
         __syncwarp();
     }
