@@ -350,10 +350,6 @@ struct Phase {
 
 }  // namespace
 
-namespace {
-lp_status order_fp64(lp_ctx* c, FitArgs& a, cudaStream_t s);
-}
-
 namespace lp {
 
 cudaError_t run_cfl(lp_ctx* c, int64_t n, double cfl, double dt_fixed, double* t, cudaStream_t s)
@@ -378,9 +374,12 @@ namespace {
 
 // FP64 passes over all particles take them by cost, where a warp's worth of
 // lists is long enough to pay for the ordering's launches
+bool fp64_ordered(const lp_ctx* c, int64_t n) { return c->dc.dim > 1 && n >= 2048; }
+int order_launches(const lp_ctx* c, int64_t n) { return fp64_ordered(c, n) ? 2 : 0; }
+
 lp_status order_fp64(lp_ctx* c, FitArgs& a, cudaStream_t s)
 {
-    if (c->dc.dim == 1 || a.n < 2048) return LP_OK;
+    if (!fp64_ordered(c, a.n)) return LP_OK;
     // (the sort's histogram and the FP32 path's lists are free here; the records
     // hold the positions of the last build)
     LP_CUDA(order_by_cost(c->dc.dim, a, c->hist, c->redo_list, c->refine_list, s));
@@ -418,7 +417,7 @@ lp_status run_fit(lp_ctx* c, FitArgs a, const StepOut& o, int sched, cudaStream_
         Phase ph(c, LP_PH_FIT64, 1, s);
         LP_CUDA(launch_step_redo(dim, a, o, s));
     } else {
-        Phase ph(c, LP_PH_FIT64, split ? 4 : 3, s);
+        Phase ph(c, LP_PH_FIT64, (split ? 2 : 1) + order_launches(c, a.n), s);
         const lp_status st = order_fp64(c, a, s);
         if (st != LP_OK) return st;
         LP_CUDA(split ? launch_step_split_f64(dim, a, o, s) : launch_step_f64(dim, a, o, s));
@@ -717,7 +716,7 @@ lp_status lp_gfd_derivs(lp_ctx* c, const lp_particles* p, const double* const* f
             Phase ph(c, LP_PH_FIT64, 1, s);
             LP_CUDA(launch_derivs_redo(dim, F, a, o, s));
         } else {
-            Phase ph(c, LP_PH_FIT64, 3, s);
+            Phase ph(c, LP_PH_FIT64, 1 + order_launches(c, n), s);
             const lp_status st = order_fp64(c, a, s);
             if (st != LP_OK) return st;
             LP_CUDA(launch_derivs_f64(dim, F, a, o, s));
@@ -758,7 +757,7 @@ lp_status lp_onesided_derivs(lp_ctx* c, const lp_particles* p, const double* con
         Phase ph(c, LP_PH_FIT64, 1, s);
         LP_CUDA(launch_onesided_redo(dim, a, derivs, nfields, s));
     } else {
-        Phase ph(c, LP_PH_FIT64, 3, s);
+        Phase ph(c, LP_PH_FIT64, 1 + order_launches(c, n), s);
         const lp_status st = order_fp64(c, a, s);
         if (st != LP_OK) return st;
         LP_CUDA(launch_onesided_f64(dim, a, derivs, nfields, s));
