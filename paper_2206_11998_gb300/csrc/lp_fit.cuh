@@ -54,22 +54,7 @@ template <> struct RN<double> {
     static __device__ __forceinline__ double sub(double a, double b) { return __dsub_rn(a, b); }
     static __device__ __forceinline__ double fma(double a, double b, double c) { return __fma_rn(a, b, c); }
     static __device__ __forceinline__ double div(double a, double b) { return __ddiv_rn(a, b); }
-    // 1 / a to within an ulp.  An FP64 instruction holds a scheduler's FP64 unit
-    // for 64 cycles (19 cycles an SM when all four issue them), so the fits in
-    // FP64 are bound by their count, and a rotation takes a reciprocal per column:
-    // the hardware's approximation y (relative error e below 2^-18, from another
-    // unit) and one step of the third-order iteration y (1 + e + e^2), whose error
-    // is e^3, take three FMAs, the rounded reciprocal six.  Where y could be
-    // denormal or infinite, the rounded reciprocal.
-    static __device__ __forceinline__ double rcp(double a)
-    {
-        const unsigned ex = (unsigned)(__double_as_longlong(a) >> 52) & 0x7ffu;
-        if (ex - 4u >= 0x7f0u) return __drcp_rn(a);
-        double y;
-        asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
-        const double e = __fma_rn(-a, y, 1.0);
-        return __fma_rn(y, __fma_rn(e, e, e), y);
-    }
+    static __device__ __forceinline__ double rcp(double a) { return __drcp_rn(a); }
     // a != 0 and a > 0 from the bits, off the FP64 unit (NaN: as the comparisons)
     static __device__ __forceinline__ bool nonzero(double a) { return (__double_as_longlong(a) << 1) != 0; }
     static __device__ __forceinline__ bool positive(double a)
