@@ -180,7 +180,6 @@ __device__ inline void dt_finalize(int s, double cfl, double dt_fixed, double t_
 // their initial value.
 constexpr int CFL_THREADS = 256;
 constexpr int CFL_ITEMS = 8;
-constexpr unsigned long long DTMIN_INIT = 0x7f7f7f7f7f7f7f7full;      // large positive
 __global__ void __launch_bounds__(CFL_THREADS) k_cfl(int64_t n, DevCfg c, const double* d2min, const double* P,
                                                      const double* V, const uint32_t* id, const uint64_t* keys,
                                                      int key_shift, unsigned long long* dtmin, int nsim, double cfl,
@@ -534,7 +533,7 @@ lp_status lp_create(const lp_config* cfg, lp_ctx** out)
         A(cudaMemset(c->cells, 0, (size_t)c->table_entries * 8));
         A(cudaMemset(c->counters, 0, C_COUNT * 8));
         A(cudaMemset(c->dt_dev, 0, 8 * ns));
-        A(cudaMemset(c->dt_min, 0x7f, 8 * (size_t)ns));      // (every k_cfl and k_begin puts its words back)
+        A(cudaMemset(c->dt_min, 0x7f, 8 * (size_t)ns));      // (k_cfl, k_begin and k_finalize_levels put their words back)
         A(cudaMemset(c->tickets, 0, 2 * sizeof(unsigned int)));
         A(sort_init());
         A(init_extent(c, nullptr));

@@ -38,6 +38,8 @@ constexpr uint32_t ST_TIMEOUT = 1u << LP_ERR_TIMEOUT;
 // per-particle fit flags (lp_gfd_derivs status output)
 constexpr uint32_t FIT_LINEAR = 1u, FIT_NONE = 2u, FIT_FP64 = 8u;
 
+constexpr unsigned long long DTMIN_INIT = 0x7f7f7f7f7f7f7f7full;   // dt_min between steps: a large double
+
 // device counters (unsigned long long each)
 enum Counter {
     C_FLAGGED = 0, C_FP64, C_LINEAR, C_NOFIT, C_OVERFLOW, C_NONFINITE, C_MLP_UNCERTAIN,

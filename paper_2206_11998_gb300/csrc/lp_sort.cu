@@ -156,9 +156,10 @@ __device__ __forceinline__ void block_w_extent(bool valid, double w, uint32_t si
     }
 }
 
-__global__ void k_init_extent(unsigned long long* ext, int nsim)
+__global__ void k_init_extent(unsigned long long* ext, int nsim, unsigned int* ticket)
 {
     int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t == 0) *ticket = 0u;
     if (t < 8 * nsim) {
         int w = t & 7;
         ext[t] = (w < 3 || w == 6) ? ~0ull : 0ull;
@@ -370,11 +371,15 @@ __device__ inline int level_of(int dim, double A, double k, double w)
 // largest radius present; lmax the finest whose edge is at least half the
 // smallest radius (the queries use cells down to half a radius).  Also zeroes
 // the lengths and work counters of the query and the fit pass that follow
-// (fresh_query, fresh_fit: they need no memsets of their own).
+// (fresh_query, fresh_fit: they need no memsets of their own), and puts the
+// words that k_begin and k_cfl leave for the next step to their initial values,
+// whatever they hold: overlapping calls on one context may leave anything there,
+// and a count of finished blocks that is off would never come right by itself.
 constexpr int LEVEL_THREADS = 256;
 __global__ void __launch_bounds__(LEVEL_THREADS) k_finalize_levels(DevCfg c, int lmax_cap, int nsim,
-                                                                   const unsigned long long* ext_all, Grid* grids,
-                                                                   int* grange, unsigned long long* counters)
+                                                                   unsigned long long* ext_all, Grid* grids,
+                                                                   int* grange, unsigned long long* counters,
+                                                                   unsigned int* tickets, unsigned long long* dtmin)
 {
     __shared__ int slo[LEVEL_THREADS], shi[LEVEL_THREADS];
     if (threadIdx.x < 8) {
@@ -382,11 +387,15 @@ __global__ void __launch_bounds__(LEVEL_THREADS) k_finalize_levels(DevCfg c, int
                              C_QUEUE_CENTRAL, C_QUEUE_PLAIN};
         counters[zero[threadIdx.x]] = 0ull;
     }
+    if (threadIdx.x < 2) tickets[threadIdx.x] = 0u;
     int lo_all = 1 << 20, hi_all = 0;
     for (int sim = threadIdx.x; sim < nsim; sim += LEVEL_THREADS) {
-        const unsigned long long* ext = ext_all + 8 * sim;
+        unsigned long long* ext = ext_all + 8 * sim;
         Grid* g = grids + sim;
         const double L = g->L;
+        dtmin[sim] = DTMIN_INIT;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) { ext[k] = ~0ull; ext[3 + k] = 0ull; }
         const bool fixed = c.radius_mode == LP_RADIUS_FIXED;
         // the radius is k w^(1/dim), the fixed one with w = 1.  Margins wider than
         // the per-particle float radius margin (1e-5) keep every particle's level
@@ -966,7 +975,7 @@ static TableArgs table_args(const lp_ctx* c, int64_t n)
 cudaError_t init_extent(lp_ctx* c, cudaStream_t s)
 {
     const int ns = c->dc.nsim_max;
-    k_init_extent<<<(unsigned)((8 * (int64_t)ns + 255) / 256), 256, 0, s>>>(c->ext, ns);
+    k_init_extent<<<(unsigned)((8 * (int64_t)ns + 255) / 256), 256, 0, s>>>(c->ext, ns, c->tickets);
     return cudaGetLastError();
 }
 
@@ -1065,7 +1074,8 @@ cudaError_t gather(lp_ctx* c, const lp_particles* p, cudaStream_t s)
     else k_gather<1><<<gb, 256, 0, s>>>(LP_GATHER_ARGS);
 #undef LP_GATHER_ARGS
     // the cell levels need the m V extent the gather took
-    k_finalize_levels<<<1, LEVEL_THREADS, 0, s>>>(c->dc, c->lmax_cap, c->nsim, c->ext, c->grid, c->grange, c->counters);
+    k_finalize_levels<<<1, LEVEL_THREADS, 0, s>>>(c->dc, c->lmax_cap, c->nsim, c->ext, c->grid, c->grange, c->counters,
+                                               c->tickets, c->dt_min);
     c->fresh_query = c->fresh_fit = 1;
     return cudaGetLastError();
 }
@@ -1084,7 +1094,8 @@ cudaError_t gather_geometry(lp_ctx* c, const lp_particles* p, cudaStream_t s)
     else if (dim == 2) k_gather_geom<2><<<gb, 256, 0, s>>>(LP_GATHER_ARGS);
     else k_gather_geom<1><<<gb, 256, 0, s>>>(LP_GATHER_ARGS);
 #undef LP_GATHER_ARGS
-    k_finalize_levels<<<1, LEVEL_THREADS, 0, s>>>(c->dc, c->lmax_cap, c->nsim, c->ext, c->grid, c->grange, c->counters);
+    k_finalize_levels<<<1, LEVEL_THREADS, 0, s>>>(c->dc, c->lmax_cap, c->nsim, c->ext, c->grid, c->grange, c->counters,
+                                               c->tickets, c->dt_min);
     c->fresh_query = c->fresh_fit = 1;
     return cudaGetLastError();
 }
@@ -1241,8 +1252,8 @@ extern "C" lp_status lp_sort_keys_noalloc(int32_t dim, int64_t n, const double* 
     unsigned gb = grid_for(n, 256);
     int64_t nb_ = gb;
     unsigned rblocks = (unsigned)(nb_ < 152 * 8 ? nb_ : 152 * 8);
-    unsigned int* ticket = reinterpret_cast<unsigned int*>(ext + 8);     // (zero at load, put back by k_begin)
-    k_init_extent<<<1, 32, 0, s>>>(ext, 1);
+    unsigned int* ticket = reinterpret_cast<unsigned int*>(ext + 8);
+    k_init_extent<<<1, 32, 0, s>>>(ext, 1, ticket);
     if (dim == 3) k_begin<3><<<rblocks, 256, 0, s>>>(n, x0, p1, p2, nullptr, ext, dc, 1, grid, ticket, none);
     else if (dim == 2) k_begin<2><<<rblocks, 256, 0, s>>>(n, x0, p1, p2, nullptr, ext, dc, 1, grid, ticket, none);
     else k_begin<1><<<rblocks, 256, 0, s>>>(n, x0, p1, p2, nullptr, ext, dc, 1, grid, ticket, none);
