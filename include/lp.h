@@ -344,6 +344,15 @@ lp_status lp_grid_info(lp_ctx *ctx, double *out, lp_stream stream);
  *   lp_mlp_adam_step    one Adam step (beta 0.9/0.999, eps 1e-8) with grad (device).
  *   lp_mlp_train        minibatch Adam over the samples in order, `epochs` passes;
  *                       epoch_loss (host, may be NULL) gets the mean batch loss.
+ *                       The blocks of a launch meet once a minibatch.  Where one
+ *                       gives up waiting (lp_mlp_wait_limit) the status word gets
+ *                       LP_ERR_TIMEOUT, the rest of the call is left out, and the
+ *                       parameters, moments and step count hold all of that
+ *                       launch's steps (up to 1024 epochs) or none; the call returns
+ *                       LP_ERR_TIMEOUT itself when epoch_loss is given (it then
+ *                       waits for the losses).
+ *   lp_mlp_wait_limit   how often a block looks for the others before it gives up
+ *                       (2^22 after lp_create: seconds; 0: it gives up at once).
  *   lp_mlp_infer        probabilities p [n] (device) for features X.
  */
 #define LP_MLP_NPARAM 321
@@ -354,6 +363,7 @@ lp_status lp_mlp_grad(lp_ctx *ctx, const float *X, const float *y, int64_t n, do
 lp_status lp_mlp_adam_step(lp_ctx *ctx, const float *grad, double lr, lp_stream stream);
 lp_status lp_mlp_train(lp_ctx *ctx, const float *X, const float *y, int64_t n, int32_t epochs,
                        int32_t batch, double lr, double pos_weight, float *epoch_loss, lp_stream stream);
+lp_status lp_mlp_wait_limit(lp_ctx *ctx, uint32_t polls);
 lp_status lp_mlp_infer(lp_ctx *ctx, const float *X, int64_t n, float *p, lp_stream stream);
 
 /*

@@ -72,7 +72,7 @@ void free_all(lp_ctx* c)
                     c->sV, c->su[0], c->su[1], c->su[2], c->sP, c->sm, c->sid, c->rec, c->pos4, c->cells, c->nb_count, c->nb_total,
                     c->nb_idx, c->nb_d2min, c->grid, c->dt_dev, c->dt_min, c->counters, c->redo_list,
                     c->plain_list, c->refine_list, c->mid, c->ext, c->grange, c->level_off_dev, c->sim_of,
-                    c->mlp_master, c->mlp_bf16, c->mlp_m1, c->mlp_m2, c->mlp_grad, c->mlp_work, c->stage_buf,
+                    c->mlp_master, c->mlp_bf16, c->mlp_m1, c->mlp_m2, c->mlp_grad, c->mlp_work, c->mlp_step, c->stage_buf,
                     c->in_pattern, c->in_state, c->in_part, c->tickets};
     for (void* p : ptrs)
         if (p) cudaFree(p);
@@ -529,12 +529,15 @@ lp_status lp_create(const lp_config* cfg, lp_ctx** out)
     A(dalloc(&c->mlp_master, MLP_NPARAM * 4)); A(dalloc(&c->mlp_bf16, MLP_NPARAM * 2));
     A(dalloc(&c->mlp_m1, MLP_NPARAM * 4)); A(dalloc(&c->mlp_m2, MLP_NPARAM * 4));
     A(dalloc(&c->mlp_grad, MLP_NPARAM * 4)); A(dalloc(&c->mlp_work, MLP_WORK * sizeof(float)));
+    A(dalloc(&c->mlp_step, sizeof(long long)));
+    c->mlp_polls = MLP_POLLS;
     if (ok) {
         A(cudaMemset(c->cells, 0, (size_t)c->table_entries * 8));
         A(cudaMemset(c->counters, 0, C_COUNT * 8));
         A(cudaMemset(c->dt_dev, 0, 8 * ns));
         A(cudaMemset(c->dt_min, 0x7f, 8 * (size_t)ns));      // (k_cfl, k_begin and k_finalize_levels put their words back)
         A(cudaMemset(c->tickets, 0, 2 * sizeof(unsigned int)));
+        A(cudaMemset(c->mlp_step, 0, sizeof(long long)));
         A(sort_init());
         A(init_extent(c, nullptr));
         A(cudaMemcpy(c->level_off_dev, c->level_off, sizeof(int64_t) * (MAX_LEVELS + 1), cudaMemcpyHostToDevice));

@@ -325,7 +325,8 @@ struct lp_ctx {
     float* mlp_m2;
     float* mlp_grad;
     float* mlp_work;              // training: epoch losses, gradient buffers, barrier (MLP_WORK)
-    int64_t mlp_step;
+    long long* mlp_step;          // Adam steps taken (on the device: it advances with the weights)
+    unsigned int mlp_polls;       // lp_mlp_wait_limit
     int mlp_ready;
     // reservoir inflow (lp_inflow): the in-plane lattice of a layer [in_npat][2],
     // the device state (committed and next), the sampling partial sums, and

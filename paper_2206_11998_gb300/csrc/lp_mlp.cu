@@ -213,11 +213,11 @@ struct MlpTrainArgs {
     float* gbuf;                  // [3][MLP_NPARAM + 1], zero: gradient, batch loss
     float* loss;                  // [epochs]: sums of the batch losses
     unsigned int* arrived;        // zero
-    int64_t step;                 // Adam steps taken before
+    long long* step;              // Adam steps taken; written with the weights
     unsigned int* lost;           // set (and ST_TIMEOUT in the status word) where the barrier gave up
     unsigned int* status;
+    unsigned int polls;           // reads of the barrier's count before a block gives up
 };
-constexpr unsigned MLP_SPINS = 1u << 22;      // seconds: the blocks of a cooperative launch all run
 
 __global__ void __launch_bounds__(MT_THREADS) k_mlp_train(MlpTrainArgs a)
 {
@@ -237,8 +237,12 @@ __global__ void __launch_bounds__(MT_THREADS) k_mlp_train(MlpTrainArgs a)
             mlp_put(sm, q, bf(a.wb, q));
         }
     }
-    if (tid == 0) lost = 0;
+    const long long step0 = *a.step;            // (block 0 writes it after the last barrier)
+    // (an earlier launch of the call gave up: the shared copy, since a block of this
+    // one may set the flag while others start)
+    if (tid == 0) lost = *reinterpret_cast<volatile unsigned int*>(a.lost) != 0u;
     __syncthreads();
+    if (lost) return;
     const int64_t t0 = (int64_t)blockIdx.x * MT_WARPS + (tid >> 5);
     auto size = [&](int64_t b0) { return a.n - b0 < a.batch ? a.n - b0 : a.batch; };
     MlpSample v = mlp_load(a.X, a.y, size(0), t0);
@@ -259,14 +263,13 @@ __global__ void __launch_bounds__(MT_THREADS) k_mlp_train(MlpTrainArgs a)
             // by the barrier)
             __syncthreads();
             if (tid == 0) asm volatile("red.release.gpu.global.add.u32 [%0], 1;" : : "l"(a.arrived) : "memory");
-            const float step = (float)(a.step + (int64_t)it + 1);
+            const float step = (float)(step0 + (long long)it + 1);
             const float c1 = 1.0f - powf(a.beta1, step), c2 = 1.0f - powf(a.beta2, step);
             if (tid == 0) {
                 const unsigned want = (it + 1u) * gridDim.x;
-                unsigned spins = 0, seen;
-                do {
+                unsigned polls = 0, seen = want - 1u;
+                while ((int)(seen - want) < 0 && polls++ < a.polls)
                     asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(a.arrived) : "memory");
-                } while ((int)(seen - want) < 0 && ++spins < MLP_SPINS);
                 if ((int)(seen - want) < 0) {
                     lost = 1;
                     atomicOr(a.lost, 1u);
@@ -300,16 +303,23 @@ __global__ void __launch_bounds__(MT_THREADS) k_mlp_train(MlpTrainArgs a)
         a.m2[q] = m2[u];
         a.wb[q] = __float2bfloat16_rn(w[u]);
     }
+    if (tid == 0) *a.step = step0 + (long long)it;
 }
 
 // Adam on the FP32 master weights; refreshes the BF16 copy and clears the gradient
-__global__ void k_mlp_adam(float* master, float* grad, float* m1, float* m2, int64_t step, float lr, float beta1,
-                           float beta2, float eps, __nv_bfloat16* wb)
+constexpr int ADAM_THREADS = 352;
+static_assert(ADAM_THREADS >= MLP_NPARAM, "one block, a thread per parameter");
+__global__ void __launch_bounds__(ADAM_THREADS) k_mlp_adam(float* master, float* grad, float* m1, float* m2,
+                                                           long long* taken, float lr, float beta1, float beta2,
+                                                           float eps, __nv_bfloat16* wb)
 {
-    int q = blockIdx.x * blockDim.x + threadIdx.x;
+    const int q = (int)threadIdx.x;
+    const float step = (float)(*taken + 1);
+    __syncthreads();
+    if (q == 0) *taken += 1;
     if (q >= MLP_NPARAM) return;
     float w = master[q];
-    const float c1 = 1.0f - powf(beta1, (float)step), c2 = 1.0f - powf(beta2, (float)step);
+    const float c1 = 1.0f - powf(beta1, step), c2 = 1.0f - powf(beta2, step);
     adam_update(grad[q], m1[q], m2[q], w, c1, c2, lr, beta1, beta2, eps);
     master[q] = w;
     wb[q] = __float2bfloat16_rn(w);
@@ -362,10 +372,10 @@ lp_status lp_mlp_set_params(lp_ctx* c, const float* params)
     LP_CUDA_MLP(cudaMemset(c->mlp_m1, 0, MLP_NPARAM * sizeof(float)));
     LP_CUDA_MLP(cudaMemset(c->mlp_m2, 0, MLP_NPARAM * sizeof(float)));
     LP_CUDA_MLP(cudaMemset(c->mlp_grad, 0, MLP_NPARAM * sizeof(float)));
+    LP_CUDA_MLP(cudaMemset(c->mlp_step, 0, sizeof(long long)));
     k_set_bf16<<<2, 256>>>(c->mlp_master, wbf(c));
     LP_CUDA_MLP(cudaGetLastError());
     LP_CUDA_MLP(cudaDeviceSynchronize());
-    c->mlp_step = 0;
     c->mlp_ready = 1;
     c->launches += 1;
     return LP_OK;
@@ -412,27 +422,38 @@ lp_status lp_mlp_train(lp_ctx* c, const float* X, const float* y, int64_t n, int
     a.gbuf = a.loss + MLP_EPOCHS;
     a.arrived = reinterpret_cast<unsigned int*>(a.gbuf + 3 * (MLP_NPARAM + 1));
     a.status = reinterpret_cast<unsigned int*>(c->counters + C_STATUS);
+    a.step = c->mlp_step;
+    a.polls = c->mlp_polls;
     const int64_t nbatches = (n + batch - 1) / batch, most = n < batch ? n : batch;
     // launches of at most MLP_EPOCHS epochs, whose losses the work area holds
     for (int32_t e0 = 0; e0 < epochs; e0 += MLP_EPOCHS) {
         a.epochs = epochs - e0 < MLP_EPOCHS ? epochs - e0 : MLP_EPOCHS;
-        // (the barrier counts in 32 bits, compared modulo 2^32)
-        a.step = c->mlp_step;
-        LP_CUDA_MLP(cudaMemsetAsync(c->mlp_work, 0, MLP_WORK * sizeof(float), s));
+        // (the barrier counts in 32 bits, compared modulo 2^32; the flag stays set
+        // over the launches of one call, so that none trains on after one gave up)
+        const int kept = e0 > 0 ? 1 : 0;
+        LP_CUDA_MLP(cudaMemsetAsync(c->mlp_work + kept, 0, (MLP_WORK - kept) * sizeof(float), s));
         void* args[] = {&a};
         LP_CUDA_MLP(cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(k_mlp_train), dim3(mlp_blocks(most)),
                                                 dim3(MT_THREADS), args, 0, s));
         c->launches += 1;
-        c->mlp_step += nbatches * a.epochs;
         if (epoch_loss) {
             float h[1 + MLP_EPOCHS];                 // the flag, the losses
             LP_CUDA_MLP(cudaMemcpyAsync(h, c->mlp_work, (size_t)(1 + a.epochs) * sizeof(float), cudaMemcpyDeviceToHost,
                                         s));
             LP_CUDA_MLP(cudaStreamSynchronize(s));
+            unsigned int lost;                       // (its bits: as a float 1 is denormal, and may compare equal to 0)
+            memcpy(&lost, h, sizeof(lost));
+            if (lost != 0u) return LP_ERR_TIMEOUT;
             for (int32_t e = 0; e < a.epochs; ++e) epoch_loss[e0 + e] = h[1 + e] / (float)nbatches;
-            if (h[0] != 0.0f) return LP_ERR_TIMEOUT;
         }
     }
+    return LP_OK;
+}
+
+lp_status lp_mlp_wait_limit(lp_ctx* c, uint32_t polls)
+{
+    if (!c) return LP_ERR_ARG;
+    c->mlp_polls = polls;
     return LP_OK;
 }
 
@@ -442,8 +463,7 @@ lp_status lp_mlp_adam_step(lp_ctx* c, const float* grad, double lr, lp_stream st
     if (!c->mlp_ready) return LP_ERR_STATE;
     cudaStream_t s = (cudaStream_t)stream;
     LP_CUDA_MLP(cudaMemcpyAsync(c->mlp_grad, grad, MLP_NPARAM * sizeof(float), cudaMemcpyDeviceToDevice, s));
-    c->mlp_step += 1;
-    k_mlp_adam<<<2, 256, 0, s>>>(c->mlp_master, c->mlp_grad, c->mlp_m1, c->mlp_m2, c->mlp_step, (float)lr, 0.9f,
+    k_mlp_adam<<<1, ADAM_THREADS, 0, s>>>(c->mlp_master, c->mlp_grad, c->mlp_m1, c->mlp_m2, c->mlp_step, (float)lr, 0.9f,
                                  0.999f, 1e-8f, wbf(c));
     c->launches += 1;
     return cudaGetLastError() == cudaSuccess ? LP_OK : LP_ERR_CUDA;

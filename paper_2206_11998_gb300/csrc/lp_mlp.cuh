@@ -15,6 +15,7 @@ constexpr int OFF_B1 = MLP_H * MLP_IN;
 constexpr int OFF_W2 = OFF_B1 + MLP_H;
 constexpr int OFF_B2 = OFF_W2 + MLP_H;
 constexpr int MLP_NPARAM = OFF_B2 + 1;
+constexpr unsigned MLP_POLLS = 1u << 22;                         // seconds: the blocks of a cooperative launch all run
 constexpr int MLP_EPOCHS = 1024;                                 // epochs of one training launch
 constexpr int MLP_WORK = 2 + MLP_EPOCHS + 3 * (MLP_NPARAM + 1);        // floats: a flag, epoch losses, gradients, barrier
 

@@ -32,7 +32,7 @@ EXPORTED = [
     "lp_export_neighbors", "lp_grid_info", "lp_dt_device", "lp_get_stats", "lp_reset_stats",
     "lp_status_string", "lp_version", "lp_set_profiling", "lp_phase_times", "lp_phase_name",
     "lp_sort_keys_noalloc", "lp_mlp_set_params", "lp_mlp_get_params", "lp_mlp_grad", "lp_mlp_adam_step",
-    "lp_mlp_train", "lp_mlp_infer", "lp_step_batched", "lp_graph_capture", "lp_graph_launch",
+    "lp_mlp_train", "lp_mlp_wait_limit", "lp_mlp_infer", "lp_step_batched", "lp_graph_capture", "lp_graph_launch",
     "lp_set_schedule", "lp_get_schedule", "lp_autotune", "lp_step_host", "lp_inflow", "lp_reserve",
     "lp_remove_outside", "lp_free_surface_ghosts", "lp_remove_ghosts", "lp_octant_coverage",
 ]
@@ -183,6 +183,7 @@ def lib():
         L.lp_mlp_grad.argtypes = [P, P, P, C.c_int64, C.c_double, P, P, P]
         L.lp_mlp_adam_step.argtypes = [P, P, C.c_double, P]
         L.lp_mlp_train.argtypes = [P, P, P, C.c_int64, C.c_int32, C.c_int32, C.c_double, C.c_double, P, P]
+        L.lp_mlp_wait_limit.argtypes = [P, C.c_uint32]
         L.lp_mlp_infer.argtypes = [P, P, C.c_int64, P, P]
         L.lp_inflow.argtypes = [P, C.POINTER(Particles), C.c_int64, C.POINTER(Inlet), C.POINTER(C.c_int64),
                                 C.POINTER(InflowInfo), P]
@@ -199,7 +200,7 @@ def lib():
         L.lp_octant_coverage.argtypes = [P, P, C.POINTER(C.c_int64), P]
         L.lp_octant_coverage.restype = C.c_int
         for name in ("lp_mlp_set_params", "lp_mlp_get_params", "lp_mlp_grad", "lp_mlp_adam_step", "lp_mlp_train",
-                     "lp_mlp_infer"):
+                     "lp_mlp_wait_limit", "lp_mlp_infer"):
             getattr(L, name).restype = C.c_int
         for name in ("lp_create", "lp_destroy", "lp_build_neighbors", "lp_gfd_derivs", "lp_onesided_derivs",
                      "lp_step", "lp_export_neighbors", "lp_grid_info", "lp_get_stats", "lp_reset_stats",
@@ -525,6 +526,10 @@ class Context:
                                   float(pos_weight), losses.ctypes.data_as(C.c_void_p), _stream(stream)),
                "lp_mlp_train")
         return losses
+
+    def mlp_wait_limit(self, polls):
+        """How often a block of a training launch looks for the others before it gives up (lp_mlp_wait_limit)."""
+        _check(lib().lp_mlp_wait_limit(self.h, int(polls)), "lp_mlp_wait_limit")
 
     def mlp_infer(self, X, stream=None):
         import torch
