@@ -117,7 +117,8 @@ enum { LP_OUT_F32 = 0, LP_OUT_F64 = 1 };
  *                  nearest by (d^2, id); LP_SELECT_OCTANT (1) round robin over
  *                  the octants (quadrants in 2D) of the offsets, nearest first
  *                  in each, so that the list covers all directions.  Either way
- *                  the list is stored in (d^2, id) order, and with at most k_max
+ *                  the list is stored in (d^2, id) order (particles that share
+ *                  an id: in key order after that), and with at most k_max
  *                  inside the radius the two agree.  LP_SELECT_OCTANT needs dim
  *                  2 or 3 and a radius (not LP_RADIUS_KSIDE).
  *   reserved       0.

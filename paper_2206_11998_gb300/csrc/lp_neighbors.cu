@@ -1,5 +1,7 @@
 // lp_neighbors.cu -- Sec. 2.2 steps 3-4: neighbour lists
 //   N(i) = {j != i : |x_j - x_i| <= R_i}, ordered by (d^2, id), first k_max kept.
+// (Particles that share an id: by their place in key order after that, so that
+// a list does not depend on the order in which its entries were found.)
 //
 // A block per 32 key-ordered particles (tiles), a block per particle for those
 // the tiles leave, and a warp per particle as a schedule of its own.  A particle
@@ -167,7 +169,8 @@ __device__ void order_ties(const QueryArgs& a, WarpBuf& b, int m, int64_t i)
                 int r = q - 1;
                 while (r >= e) {
                     double dr = b.d64[r];
-                    bool gt = dr > dq || (dr == dq && (uint32_t)b.key[r] > (uint32_t)kq);
+                    const uint32_t ir = (uint32_t)b.key[r], iq = (uint32_t)kq;
+                    const bool gt = dr > dq || (dr == dq && (ir > iq || (ir == iq && b.j[r] > jq)));
                     if (!gt) break;
                     b.key[r + 1] = b.key[r]; b.j[r + 1] = b.j[r]; b.d64[r + 1] = b.d64[r];
                     --r;
@@ -1975,7 +1978,8 @@ __device__ int tile_group(const QueryArgs& a, TileBuf<W>& b, int64_t i, bool act
                         while (r >= s0) {
                             const uint32_t jr = b.kj[r][p];
                             const double dr = exact_d2<DIM>(a, ip, jr);
-                            if (dr < dq || (dr == dq && a.sid[jr] < iq)) break;
+                            const uint32_t ir = a.sid[jr];
+                            if (dr < dq || (dr == dq && (ir < iq || (ir == iq && jr < jq)))) break;
                             b.kj[r + 1][p] = jr;
                             --r;
                         }
