@@ -711,7 +711,7 @@ lp_status lp_gfd_derivs(lp_ctx* c, const lp_particles* p, const double* const* f
             static_assert(C_REFINE_LEN == C_REDO_LEN + 1, "one memset for both lengths");
             LP_CUDA(cudaMemsetAsync(c->counters + C_REDO_LEN, 0, 16, s));
             {
-                Phase ph(c, LP_PH_FIT, c->dc.refine == LP_REFINE_AUTO ? 2 : 1, s);
+                Phase ph(c, LP_PH_FIT, derivs_defer(c->dc, n) ? 2 : 1, s);
                 LP_CUDA(launch_derivs_f32(dim, F, a, o, s));
             }
             a.list = c->redo_list;

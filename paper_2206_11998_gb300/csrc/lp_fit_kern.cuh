@@ -693,13 +693,13 @@ __device__ __forceinline__ void derivs_one(const FitArgs& a, const DerivOut& o, 
 
 // The warp's list rows staged as in k_step_central; DEFER (FP32, correction
 // where the ratio asks for it): the fits that need the correction pass go to
-// k_derivs_refine.  One field needs half of each record and under 100 registers,
-// so more blocks fit an SM.
-template <typename T, int F> struct DerivOcc { static constexpr int v = 1; };
-template <> struct DerivOcc<float, 1> { static constexpr int v = 5; };
-template <> struct DerivOcc<float, 5> { static constexpr int v = 3; };
+// k_derivs_refine.  One field needs half of each record and, without the
+// correction's code, under 100 registers, so more blocks fit an SM.
+template <typename T, int F, bool DEFER> struct DerivOcc { static constexpr int v = 1; };
+template <> struct DerivOcc<float, 1, true> { static constexpr int v = 5; };
+template <bool DEFER> struct DerivOcc<float, 5, DEFER> { static constexpr int v = 3; };
 template <typename T, int DIM, int F, bool DEFER>
-__global__ void __launch_bounds__(FIT_THREADS, DerivOcc<T, F>::v) k_derivs(FitArgs a, DerivOut o)
+__global__ void __launch_bounds__(FIT_THREADS, DerivOcc<T, F, DEFER>::v) k_derivs(FitArgs a, DerivOut o)
 {
     constexpr int SD = DEFER ? 64 : 32;
     __shared__ uint32_t stage[SD][NB_PITCH];
@@ -708,6 +708,14 @@ __global__ void __launch_bounds__(FIT_THREADS, DerivOcc<T, F>::v) k_derivs(FitAr
     if (i >= a.n) return;
     derivs_one<T, DIM, F, DEFER>(a, o, i, NbStaged<SD>{a.idx + i * (int64_t)a.c.k_max, &stage[0][threadIdx.x]});
 }
+
+// Below these sizes (2D: the second) and in 1D the corrections stay in k_derivs: a
+// kernel over the deferred fits takes 23 to 29 us however few they are, one
+// fit's chain, and a launch.  The call, with it and without, one field of the gas
+// cloud: 94 and 60 us at 20k particles, 183 and 177 at 300k, 269 and 322 at 600k,
+// 647 and 884 at 2M; five fields 109 and 82, 282 and 275, 449 and 501; of a random
+// 2D set 412 and 401 at 1M, 618 and 667 at 2M; 1D 390 and 297 at 2M.
+constexpr int64_t DERIVS_DEFER_N = 400000, DERIVS_DEFER_N2 = 1500000;
 
 // the fits k_derivs deferred, with the correction pass on (the caller passes
 // refine = LP_REFINE_ALWAYS)
@@ -913,6 +921,12 @@ inline bool split_defers_t(const FitArgs& a)
     return IsF32<T>::v && a.refine_list && a.c.refine == LP_REFINE_AUTO;
 }
 
+inline bool derivs_defer(const DevCfg& c, int64_t n)
+{
+    return c.precision == LP_PREC_FP32 && c.refine == LP_REFINE_AUTO && c.dim > 1 &&
+           n >= (c.dim == 3 ? DERIVS_DEFER_N : DERIVS_DEFER_N2);
+}
+
 template <typename T>
 inline unsigned fit_blocks(const FitArgs& a)
 {
@@ -925,7 +939,7 @@ cudaError_t launch_derivs(const FitArgs& a, const DerivOut& o, cudaStream_t s)
     const unsigned b = fit_blocks<T>(a);
     constexpr int B = FitBlock<T>::v;
     if constexpr (IsF32<T>::v) {
-        if (split_defers_t<T>(a)) {
+        if (derivs_defer(a.c, a.n)) {
             FitArgs r = a;
             r.c.refine = LP_REFINE_ALWAYS;
             k_derivs<T, DIM, F, true><<<b, B, 0, s>>>(a, o);
