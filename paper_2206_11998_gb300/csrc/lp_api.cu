@@ -752,7 +752,7 @@ lp_status lp_onesided_derivs(lp_ctx* c, const lp_particles* p, const double* con
         }
         LP_CUDA(cudaMemsetAsync(c->counters + C_REDO_LEN, 0, 16, s));
         {
-            Phase ph(c, LP_PH_FIT, 3, s);
+            Phase ph(c, LP_PH_FIT, onesided_staged(dim, n) ? 3 : 1, s);
             LP_CUDA(launch_onesided_f32(dim, a, derivs, nfields, s));
         }
         a.list = c->redo_list;

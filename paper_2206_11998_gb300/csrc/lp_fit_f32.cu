@@ -10,6 +10,10 @@ template <int DIM>
 cudaError_t onesided(const FitArgs& a, double* out, int f_real, cudaStream_t s)
 {
     const unsigned b = fit_blocks<float>(a);
+    if (!onesided_staged(DIM, a.n)) {
+        k_onesided<float, DIM, 5><<<b, FIT_THREADS, 0, s>>>(a, out, f_real);
+        return cudaGetLastError();
+    }
     k_onesided_sides<DIM, 5><<<b, FIT_THREADS, 0, s>>>(a, out, f_real);
     k_onesided_check<DIM, 5><<<b, FIT_THREADS, 0, s>>>(a);
     k_onesided_fill<DIM, 5><<<152u * 4u, FIT_THREADS, 0, s>>>(a, out, f_real);

@@ -95,9 +95,9 @@ cudaError_t launch_onesided_f64(int dim, const FitArgs& a, double* out, int f_re
 {
     if (a.n == 0) return cudaSuccess;
     const unsigned b = fit_blocks<double>(a);
-    if (dim == 3) k_onesided<3, 5><<<b, FitBlock<double>::v, 0, s>>>(a, out, f_real);
-    else if (dim == 2) k_onesided<2, 5><<<b, FitBlock<double>::v, 0, s>>>(a, out, f_real);
-    else k_onesided<1, 5><<<b, FitBlock<double>::v, 0, s>>>(a, out, f_real);
+    if (dim == 3) k_onesided<double, 3, 5><<<b, FitBlock<double>::v, 0, s>>>(a, out, f_real);
+    else if (dim == 2) k_onesided<double, 2, 5><<<b, FitBlock<double>::v, 0, s>>>(a, out, f_real);
+    else k_onesided<double, 1, 5><<<b, FitBlock<double>::v, 0, s>>>(a, out, f_real);
     return cudaGetLastError();
 }
 

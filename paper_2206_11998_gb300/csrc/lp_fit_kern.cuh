@@ -733,19 +733,19 @@ __global__ void __launch_bounds__(FIT_THREADS) k_derivs_refine(FitArgs a, DerivO
 // ---------------------------------------------------------------------------
 // one-sided derivatives (lp_onesided_derivs), out[i][k][s][f] float64
 // ---------------------------------------------------------------------------
-template <int DIM, int F>
+template <typename T, int DIM, int F>
 __device__ void onesided_one(const FitArgs& a, double* out, int f_real, int64_t i)
 {
-    using T = double;
     constexpr int N = NU<DIM>::v;
     const DevCfg& c = a.c;
     Src<T, DIM, F> src(a, i);
     const int cnt = (int)a.count[i];
     const NbGlobal nb{a.idx + i * (int64_t)c.k_max};
     const T invS = (T)inv_scale(last_d2(src, nb, cnt));
-    const T tau = c.tau64;
+    const T tau = IsF32<T>::v ? (T)c.tau32 : (T)c.tau64;
     T cd[N][F];
     if (central_fit<T, DIM, F>(src, nb, cnt, invS, tau, c, cd)) {
+        if (IsF32<T>::v) { push_redo(a, i); return; }
 #pragma unroll
         for (int u = 0; u < N; ++u)
 #pragma unroll
@@ -771,6 +771,7 @@ __device__ void onesided_one(const FitArgs& a, double* out, int f_real, int64_t 
 #pragma unroll
                 for (int f = 0; f < F; ++f) os[k][s][f] = ok[k][s] ? o2[k][s][f] : cd[k][f];
     }
+    if (IsF32<T>::v && ill) { push_redo(a, i); return; }
 #pragma unroll
     for (int k = 0; k < DIM; ++k)
 #pragma unroll
@@ -780,14 +781,14 @@ __device__ void onesided_one(const FitArgs& a, double* out, int f_real, int64_t 
                 if (f < f_real) out[((i * DIM + k) * 2 + s) * f_real + f] = (double)os[k][s][f];
 }
 
-template <int DIM, int F>
+template <typename T, int DIM, int F>
 __global__ void __launch_bounds__(FIT_THREADS) k_onesided(FitArgs a, double* out, int f_real)
 {
     const int64_t i = fit_particle(a);
-    if (i < a.n) onesided_one<DIM, F>(a, out, f_real, i);
+    if (i < a.n) onesided_one<T, DIM, F>(a, out, f_real, i);
 }
 
-// The FP32 path in three kernels.  k_onesided_sides runs the one-sided fits (the
+// The FP32 path of large sets (onesided_staged) in three kernels.  k_onesided_sides runs the one-sided fits (the
 // warp's list rows staged, results written coalesced: 30 doubles a particle, one
 // line per lane and store otherwise) and lists the particles that lack a side,
 // which need central derivatives; k_onesided_check tests the others' central
@@ -797,6 +798,12 @@ __global__ void __launch_bounds__(FIT_THREADS) k_onesided(FitArgs a, double* out
 // them on a 59^3 lattice to use it: 334 us at 205k particles, against 190 us.
 // state[i] (plain_list): nothing more to do, or the FP64 redo has it
 // (SIDES_REDO); else SIDES_CHECK or the mask of the fits it has.
+// Smaller sets (2D: the second line) and 1D take one kernel, in which a particle
+// runs all its fits: three kernels are three chains.  The call, five fields, three
+// kernels and one: the gas cloud 166 and 127 us at 20k particles, 183 and 201 at
+// 60k, 415 and 529 at 300k; a random 2D set 132 and 122 at 60k, 164 and 155 at
+// 131k, 261 and 278 at 300k; 1D 55 and 44 at 10k, 519 and 520 at 2M.
+constexpr int64_t ONESIDED_STAGED_N = 65536, ONESIDED_STAGED_N2 = 131072;
 constexpr uint32_t SIDES_REDO = 0xffffffffu, SIDES_CHECK = 0xfffffffeu;
 template <int DIM, int F>
 __global__ void __launch_bounds__(FIT_THREADS, 5) k_onesided_sides(FitArgs a, double* out, int f_real)
@@ -920,6 +927,8 @@ inline bool split_defers_t(const FitArgs& a)
 {
     return IsF32<T>::v && a.refine_list && a.c.refine == LP_REFINE_AUTO;
 }
+
+inline bool onesided_staged(int dim, int64_t n) { return dim > 1 && n >= (dim == 3 ? ONESIDED_STAGED_N : ONESIDED_STAGED_N2); }
 
 inline bool derivs_defer(const DevCfg& c, int64_t n)
 {

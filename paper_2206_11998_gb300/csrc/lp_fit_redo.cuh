@@ -521,7 +521,7 @@ __global__ void __launch_bounds__(FIT_THREADS) k_onesided_redo(FitArgs a, double
     }
     for (unsigned long long t = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; t < len;
          t += (unsigned long long)gridDim.x * blockDim.x)
-        onesided_one<DIM, F>(a, out, f_real, a.list[t]);
+        onesided_one<double, DIM, F>(a, out, f_real, a.list[t]);
 }
 
 }  // namespace lp

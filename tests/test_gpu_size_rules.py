@@ -68,3 +68,12 @@ def test_derivs(d, fields, n, total, refine):
     b = _run(d, _set(d, n, total - n, n), n, fields, _derivs, refine=refine)
     for p, q in zip(a, b):
         assert np.array_equal(p, q)
+
+
+@pytest.mark.parametrize("d,fields,n,total", [(3, 5, 30000, 65536), (3, 2, 1000, 65537), (2, 5, 30000, 131072),
+                                              (2, 1, 131071, 140001)])
+def test_onesided(d, fields, n, total):
+    call = lambda ctx, ps, f: ctx.onesided_derivs(ps, f)
+    a = _run(d, _set(d, n, 0, n), n, fields, call)
+    b = _run(d, _set(d, n, total - n, n), n, fields, call)
+    assert np.array_equal(a[0], b[0])
