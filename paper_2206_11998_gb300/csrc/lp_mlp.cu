@@ -10,6 +10,8 @@
 #include <cuda_bf16.h>
 #include <string.h>
 
+#include <type_traits>
+
 #include "lp_mlp.cuh"
 
 namespace lp {
@@ -123,6 +125,10 @@ __device__ void mlp_block_grad(MlpShared& sm, MlpSample first, const float* __re
                 gb2 += dz;
             }
         }
+        float size = 0.0f;
+#pragma unroll
+        for (int k = 0; k < MLP_IN; ++k) size = fmaf(0.0f, x[k], size);        // NaN, or 0
+        const bool finite = __all_sync(0xffffffffu, size == 0.0f);
         float* row = xs[lane >> 1];
         if (half == 0) {
             *reinterpret_cast<float4*>(row) = v.x0;
@@ -132,25 +138,29 @@ __device__ void mlp_block_grad(MlpShared& sm, MlpSample first, const float* __re
         }
         __syncwarp();
         if (t + warps < tiles) v = mlp_load(X, y, nb, t + warps);
+        // (a dead unit's dh is 0, and 0 times a feature that is not finite would be NaN:
+        // in tiles with such features dead units are left out)
+        auto backward = [&](auto careful) {
 #pragma unroll 4
-        for (int s = 0; s < MT_TILE; ++s) {
-            const float4 x0 = *reinterpret_cast<const float4*>(xs[s]);
-            const float4 x1 = *reinterpret_cast<const float4*>(xs[s] + 4);
-            const float d = xs[s][8];
-            const float q[MLP_IN] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w};
-            float a = bu;
+            for (int s = 0; s < MT_TILE; ++s) {
+                const float4 x0 = *reinterpret_cast<const float4*>(xs[s]);
+                const float4 x1 = *reinterpret_cast<const float4*>(xs[s] + 4);
+                const float d = xs[s][8];
+                const float q[MLP_IN] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w};
+                float a = bu;
 #pragma unroll
-            for (int k = 0; k < MLP_IN; ++k) a = fmaf(wu[k], q[k], a);
-            const bool live = a > 0.0f;
-            gw2 = fmaf(d, live ? a : 0.0f, gw2);
-            // (not dh = 0 for a dead unit: 0 times a feature that is not finite is NaN)
-            if (live) {
-                const float dh = d * w2u;
+                for (int k = 0; k < MLP_IN; ++k) a = fmaf(wu[k], q[k], a);
+                const bool live = a > 0.0f;
+                gw2 = fmaf(d, live ? a : 0.0f, gw2);
+                if (decltype(careful)::value && !live) continue;
+                const float dh = live ? d * w2u : 0.0f;
                 gb += dh;
 #pragma unroll
                 for (int k = 0; k < MLP_IN; ++k) gu[k] = fmaf(dh, q[k], gu[k]);
             }
-        }
+        };
+        if (finite) backward(std::false_type{});
+        else backward(std::true_type{});
         __syncwarp();
     }
 #pragma unroll
@@ -337,9 +347,10 @@ __global__ void k_mlp_infer(const float* __restrict__ X, int64_t n, const __nv_b
     p[s] = mlp_prob(x, wb);
 }
 
-__global__ void k_set_bf16(const float* master, __nv_bfloat16* wb)
+__global__ void k_set_bf16(const float* master, __nv_bfloat16* wb, long long* step)
 {
     int q = blockIdx.x * blockDim.x + threadIdx.x;
+    if (q == 0) *step = 0;
     if (q < MLP_NPARAM) wb[q] = __float2bfloat16_rn(master[q]);
 }
 
@@ -372,8 +383,7 @@ lp_status lp_mlp_set_params(lp_ctx* c, const float* params)
     LP_CUDA_MLP(cudaMemset(c->mlp_m1, 0, MLP_NPARAM * sizeof(float)));
     LP_CUDA_MLP(cudaMemset(c->mlp_m2, 0, MLP_NPARAM * sizeof(float)));
     LP_CUDA_MLP(cudaMemset(c->mlp_grad, 0, MLP_NPARAM * sizeof(float)));
-    LP_CUDA_MLP(cudaMemset(c->mlp_step, 0, sizeof(long long)));
-    k_set_bf16<<<2, 256>>>(c->mlp_master, wbf(c));
+    k_set_bf16<<<2, 256>>>(c->mlp_master, wbf(c), c->mlp_step);
     LP_CUDA_MLP(cudaGetLastError());
     LP_CUDA_MLP(cudaDeviceSynchronize());
     c->mlp_ready = 1;
