@@ -894,8 +894,24 @@ __global__ void __launch_bounds__(NB_WARPS * 32) k_query(QueryArgs a)
 // the bin that holds the NB_CAP-th so far, and later ones beyond it are only
 // counted.  Each remaining hit then gets its place by counting those that sort
 // before it; the NB_CAP nearest are kept.  Particles with more candidates than
-// QL_CAND, and lists whose last entries tie past the buffer, go through
-// query_one (which prunes by the k_max-th distance) on the first warp.
+// QL_CAND or more hits in a bin than the buffer holds, and lists whose last
+// entries tie past the buffer, go through query_one (which prunes by the k_max-th
+// distance), put off for the block's warps, one each, so that they do not follow
+// one another on one warp: 200k particles with a dense core, half of them listed,
+// 28.5 -> 18.3 ms, the 1M jet, nearest first, 2.41 -> 2.12.
+//
+// A list longer than LONG is bound by throughput, and there a warp per particle
+// takes less: no barriers, and the cells it does not need left out.  Two kinds of
+// particles stay with the blocks (LEFT_DENSE): those of groups with too many
+// candidates or cells, and in 3D, with a k_max above 48, those with more than
+// NB_CAP - 32 hits, which a warp sorts its buffer for over and over (192 hits in
+// LeftChain's sets of 20,000 particles and more, whose long lists take longest).
+// A build, blocks alone and so: a uniform 2D set with 150 hits each, 20k particles
+// 494 -> 327 us, 500k 6.5 -> 4.9 ms; 3D lattices with 82 hits, 97k particles 1.42 ->
+// 0.91 ms, 512k 4.79 -> 4.53, and with 147 hits and k_max = 80 (blocks, as before)
+// 8.27 ms against 10.3 by warps.  LONG: shorter lists wait for their outliers, which
+// a block takes in less (the 60k cloud's 1,972 310 us against 334, the 2M cloud's
+// 9,915 2.608 ms against 2.627).
 //
 // What bounds it: in small sets the chain of one outlier (20k: 9,600 candidates,
 // 178,000 cycles with 128 threads), so 256 threads with four loads each: 56 us at
@@ -905,15 +921,19 @@ __global__ void __launch_bounds__(NB_WARPS * 32) k_query(QueryArgs a)
 // threads in 14 KB and 12 blocks an SM, at the price of a few spills: 84 us at 2M
 // and 52 at 131k, against 103 and 55 with 8 blocks of 56 registers, and before
 // that 188 and 62 with 256 threads, 103 and 65 with 64, 132 and 55 with two passes.
-template <int THREADS_, int LOADS_, int HITS_, int BLOCKS_, int RESIDENT_>
+template <int THREADS_, int LOADS_, int HITS_, int BLOCKS_, int RESIDENT_, int WARPS_, int LONG_>
 struct LeftShape {
     static constexpr int THREADS = THREADS_, LOADS = LOADS_, HITS = HITS_;
     static constexpr int BLOCKS = BLOCKS_, RESIDENT = RESIDENT_;   // blocks launched and resident an SM
+    static constexpr uint32_t WARPS = WARPS_;         // warps that take a particle each, in the block's buffers' room
+    static constexpr uint32_t LONG = LONG_;
 };
-using LeftChain = LeftShape<256, 4, 1024, 8, 4>;
-using LeftMany = LeftShape<128, 2, 512, 12, 12>;
-using LeftOct = LeftShape<256, 4, 1024, 24, 4>;   // LP_SELECT_OCTANT
-constexpr int QL_SMALL_N = 100000;    // below: LeftChain
+using LeftChain = LeftShape<256, 4, 1024, 8, 4, 6, 4096>;
+using LeftMany = LeftShape<128, 2, 512, 12, 12, 2, 16384>;
+using LeftOct = LeftShape<256, 4, 1024, 24, 4, 1, 0>;   // LP_SELECT_OCTANT
+// below, and in 2D: LeftChain (in 2D lists are short or of the whole set, and the
+// uniform set of 500k above takes 4.9 ms, by LeftMany's warps 5.6)
+constexpr int QL_SMALL_N = 100000;
 constexpr uint32_t QL_CAND = 32768, QL_OCT_CAND = 131072;   // (octants: where a warp would take as long)
 constexpr int QL_BINS = 256;
 constexpr int QL_OCT_BINS = 128;      // an octant's, with LP_SELECT_OCTANT
@@ -940,8 +960,14 @@ struct LeftBuf {
 // it on candidates that only had to be counted: with the nearest cells first and
 // those left out that nothing waits for 298, with four resident blocks instead of
 // three 283, and with blocks to spare for the uneven particles 244.
+
+// later: the particles that a warp has to take (not OCT).
+struct LeftLater {
+    uint32_t n, i[32];
+    uint32_t now, k[32];              // and those that the block takes next
+};
 template <int DIM, class S, bool OCT>
-__device__ void query_left(const QueryArgs& a, LeftBuf<S, OCT>& b, int64_t i)
+__device__ void query_left(const QueryArgs& a, LeftBuf<S, OCT>& b, LeftLater& later, int64_t i)
 {
     constexpr int NO = 1 << DIM, BINS = OCT ? QL_OCT_BINS : QL_BINS;
     constexpr int QL_THREADS = S::THREADS, QL_LOADS = S::LOADS, QL_HITS = S::HITS;
@@ -1308,7 +1334,7 @@ __device__ void query_left(const QueryArgs& a, LeftBuf<S, OCT>& b, int64_t i)
         small = !__all_sync(0xffffffffu, open);
     }
     if (!small) {
-        query_one<DIM>(a, b.w, i);
+        if (lane == 0) later.i[later.n++] = (uint32_t)i;
         return;
     }
     order_ties<DIM>(a, b.w, m, i);
@@ -1323,14 +1349,73 @@ __device__ void query_left(const QueryArgs& a, LeftBuf<S, OCT>& b, int64_t i)
     }
 }
 
+// entry of the list: the particle, and whether blocks take it from long lists too
+constexpr uint32_t LEFT_DENSE = 0x80000000u;          // (a particle's index is below 2^31)
+// 3D: the hits above which the blocks keep a long list's particles
+__device__ __forceinline__ uint32_t left_hits(int64_t n, uint32_t kmax)
+{
+    if (kmax <= 48u) return ~0u;
+    return n >= 20000 && n < QL_SMALL_N ? 192u : (uint32_t)NB_CAP - 32u;
+}
+template <class S, bool OCT>
+union LeftShared {
+    LeftBuf<S, OCT> b;
+    WarpBuf w[S::WARPS];
+};
+
 template <int DIM, class S, bool OCT>
 __global__ void __launch_bounds__(S::THREADS, S::RESIDENT) k_query_left(QueryArgs a)
 {
-    __shared__ LeftBuf<S, OCT> b;
-    const unsigned long long len = *a.list_len;
-    for (unsigned long long t = blockIdx.x; t < len; t += gridDim.x) {
-        query_left<DIM, S, OCT>(a, b, (int64_t)a.list[t]);
-        __syncthreads();                    // the buffers are reused by the next particle
+    __shared__ LeftShared<S, OCT> sm;
+    __shared__ LeftLater later;
+    const uint32_t len = (uint32_t)*a.list_len;            // (the list's particles and their numbers fit 31 bits)
+    const uint32_t w = threadIdx.x >> 5;
+    const bool warps = !OCT && len > S::LONG;
+    // particles that the warps take, one each, but for the marked ones
+    auto by_warps = [&](const uint32_t* src, uint32_t first, uint32_t stride, uint32_t n) {
+        if (w < S::WARPS)
+            for (uint32_t q = first + w; q < n; q += stride)
+                if (!(src[q] & LEFT_DENSE)) query_one<DIM>(a, sm.w[w], (int64_t)src[q]);
+    };
+    // They take a long list first, and then, in turn with the block, what it puts
+    // off.  (In 2D long lists have a copy of the code of their own, without which
+    // they take 18 % longer; in 3D it would cost the short lists' registers, 57 ->
+    // 64 us at 131k.  Little is kept in registers over query_left for the same
+    // reason.)
+    if constexpr (DIM == 2 && !OCT) by_warps(a.list, blockIdx.x * S::WARPS, gridDim.x * S::WARPS, warps ? len : 0u);
+    uint32_t c = blockIdx.x;
+    if constexpr (!OCT && DIM == 3 && S::THREADS == LeftChain::THREADS)
+        // a list of a particle a block at most, what small sets leave: without the
+        // loop around it a particle takes 44.8 us, with it 47.3 (20k; LeftMany's 63, 58)
+        if (!warps && len <= gridDim.x && c < len) {
+            if (threadIdx.x == 0) later.n = 0;
+            __syncthreads();
+            query_left<DIM, S, OCT>(a, sm.b, later, (int64_t)(a.list[c] & ~LEFT_DENSE));
+            __syncthreads();
+            c += 32u * gridDim.x;
+        }
+    for (; ; c += 32u * gridDim.x) {
+        if constexpr (!OCT) {
+            const bool put_off = c != blockIdx.x;
+            by_warps(put_off ? later.i : a.list, put_off ? 0u : blockIdx.x * S::WARPS,
+                     put_off ? S::WARPS : gridDim.x * S::WARPS, put_off ? later.n : (DIM == 3 && warps ? len : 0u));
+        }
+        __syncthreads();                        // (the buffers share their room)
+        if (c >= len) return;
+        if (w == 0) {                           // the block's next 32 of the list, what it has to take of them
+            const unsigned lane = lane_id();
+            const uint32_t q = c + lane * gridDim.x;
+            const uint32_t e = q < len ? a.list[q] : 0u;
+            const bool take = q < len && (!warps || (e & LEFT_DENSE));
+            const unsigned m = __ballot_sync(0xffffffffu, take);
+            if (take) later.k[__popc(m & ((1u << lane) - 1u))] = e & ~LEFT_DENSE;
+            if (lane == 0) { later.now = (uint32_t)__popc(m); later.n = 0; }
+        }
+        __syncthreads();
+        for (uint32_t k = 0; k < later.now; ++k) {
+            query_left<DIM, S, OCT>(a, sm.b, later, (int64_t)later.k[k]);
+            __syncthreads();                    // the buffers are reused by the next particle
+        }
     }
 }
 
@@ -1338,9 +1423,16 @@ template <int DIM>
 void launch_left(const QueryArgs& a, cudaStream_t s)
 {
     const bool octant = a.c.select == LP_SELECT_OCTANT;
-    if (octant) k_query_left<DIM, LeftOct, true><<<152u * LeftOct::BLOCKS, LeftOct::THREADS, 0, s>>>(a);
-    else if (a.n < QL_SMALL_N) k_query_left<DIM, LeftChain, false><<<152u * LeftChain::BLOCKS, LeftChain::THREADS, 0, s>>>(a);
-    else k_query_left<DIM, LeftMany, false><<<152u * LeftMany::BLOCKS, LeftMany::THREADS, 0, s>>>(a);
+    if (octant) {
+        k_query_left<DIM, LeftOct, true><<<152u * LeftOct::BLOCKS, LeftOct::THREADS, 0, s>>>(a);
+        return;
+    }
+    if constexpr (DIM == 3)
+        if (a.n >= QL_SMALL_N) {
+            k_query_left<DIM, LeftMany, false><<<152u * LeftMany::BLOCKS, LeftMany::THREADS, 0, s>>>(a);
+            return;
+        }
+    k_query_left<DIM, LeftChain, false><<<152u * LeftChain::BLOCKS, LeftChain::THREADS, 0, s>>>(a);
 }
 
 // the octant-balanced selection of every particle, a warp each.  A kernel of its
@@ -1849,8 +1941,9 @@ __device__ int tile_group(const QueryArgs& a, TileBuf<W>& b, int64_t i, bool act
     // ---- 3. per particle: exact membership, order, row
     const uint32_t cnt = b.cnt[lane];
     const bool mine = act && cnt <= (uint32_t)TQ_CAP;
-    if (wid == 0) list_append(a, act && !mine, (uint32_t)i);
     const uint32_t kmax = (uint32_t)c.k_max;
+    if (wid == 0)
+        list_append(a, act && !mine, (uint32_t)i | (DIM == 3 && cnt > left_hits(a.n, kmax) ? LEFT_DENSE : 0u));
     uint32_t mx = 0, novf = 0;
     // this warp's share: every W-th of the particles
     const unsigned all = __ballot_sync(0xffffffffu, mine);
@@ -2088,7 +2181,7 @@ __device__ __forceinline__ void tile_tile(const QueryArgs& a, TileBuf<W>& b, int
             const int pc = __popc(grp);
             if (r == GROUP_DONE || threadIdx.x >= 32) continue;
             if (pc > TQ_FEW) groups_append(a, i0, grp, max(1, pc >> (r + 1)));
-            else list_append(a, ((grp >> lane) & 1u) != 0u, (uint32_t)i);
+            else list_append(a, ((grp >> lane) & 1u) != 0u, (uint32_t)i | LEFT_DENSE);
             continue;
         }
         // the part, halved (by key order: the halves are smaller regions) while
@@ -2107,7 +2200,7 @@ __device__ __forceinline__ void tile_tile(const QueryArgs& a, TileBuf<W>& b, int
                 stk[sp++] = g & ~lo;
                 stk[sp++] = lo;
             } else if (threadIdx.x < 32) {
-                list_append(a, ((g >> lane) & 1u) != 0u, (uint32_t)i);
+                list_append(a, ((g >> lane) & 1u) != 0u, (uint32_t)i | LEFT_DENSE);
             }
         }
     }

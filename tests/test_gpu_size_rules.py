@@ -1,6 +1,8 @@
 """Calls that take another kernel by the size of the set: the same particles alone
 (below the rule's line) and beside others far away (above it) have the same
-neighbours, so their results are the same bit for bit."""
+neighbours, so their results are the same bit for bit.  And neighbour lists of
+many particles that the blocks put off for their warps, against the
+warp-per-particle query."""
 import numpy as np
 import pytest
 
@@ -77,3 +79,23 @@ def test_onesided(d, fields, n, total):
     a = _run(d, _set(d, n, 0, n), n, fields, call)
     b = _run(d, _set(d, n, total - n, n), n, fields, call)
     assert np.array_equal(a[0], b[0])
+
+
+@pytest.mark.parametrize("d,clumps,size", [(3, 18, 2500), (2, 18, 2500), (3, 41, 2500)])
+def test_lists_that_blocks_put_off(d, clumps, size):
+    # (a clump's particles fill one bin of distances past a block's buffer)
+    r = np.random.Generator(np.random.PCG64(size))
+    x = np.repeat(3.0 * np.arange(clumps)[None] + np.arange(d)[:, None], size, 1)
+    x = np.concatenate([x, r.uniform(0, 3 * clumps, (d, 1000))], 1)
+    out = []
+    for sched in (lp.SCHED_QUERY_WARP, 0):
+        ctx = lp.Context(lp.make_config(d, x.shape[1], radius_mode=lp.RADIUS_FIXED, radius=1.0, k_max=24))
+        ctx.set_schedule(sched)
+        ps = lp.ParticleSet.from_state(_state(x))
+        ctx.build_neighbors(ps)
+        cnt, tot, idx, d2, _ = ctx.export_neighbors(ps.n)
+        idx.masked_fill_(torch.arange(24, device="cuda") >= cnt[:, None], -1)
+        out.append([a.cpu().numpy() for a in (cnt, tot, idx, d2, ps.id)])
+        ctx.close()
+    for a, b in zip(*out):
+        assert np.array_equal(a, b)
