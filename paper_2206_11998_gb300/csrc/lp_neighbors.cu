@@ -886,8 +886,8 @@ __global__ void __launch_bounds__(NB_WARPS * 32) k_query(QueryArgs a)
     if (i < a.n) query_one<DIM>(a, bufs[w], i);
 }
 
-// The particles the tiles left, a block each: 4 % of the 2M cloud, whose 65 to 80
-// hits are a few more than a tile's column holds, 8 % of a cloud of 20k, and a
+// The particles the tiles left, a block each: 0.5 % of the 2M cloud, whose 65 to 80
+// hits are a few more than a tile's column holds, 5 % of a cloud of 20k, and a
 // few outliers with up to 18,000 candidates.  The threads of a block test the
 // candidates of all start cells, LOADS each in flight, count the hits by bin of
 // d2 and keep them in shared memory; a full buffer is pruned to the hits up to
@@ -1476,9 +1476,9 @@ constexpr int TQ_CELLS_PER = 64;      // so many a particle (a compact group of 
 constexpr uint32_t TQ_CAND_MAX = 2048;   // candidates a group may test (fastest of 2048, 4096, 8192 on the gas cloud)
 constexpr int TQ_KC = 512;            // non-empty cells a group may keep
 constexpr float TQ_GAP = 2.0f;        // in radii
-// Warps of a tile's block.  Two, 16 blocks of 64 registers a thread to an SM
-// (32 warps, where a warp per tile with its own column buffer allowed 20), for
-// the throughput of large sets: 1.94 ms at 2M particles, against 2.08 with four
+// Warps of a tile's block.  Two, 15 blocks to an SM (of 64 registers a thread for
+// 16, but 13.9 KB each; 30 warps, where a warp per tile with its own column buffer
+// allowed 20), for the throughput of large sets: 1.94 ms at 2M particles, against 2.08 with four
 // warps, 2.65 with eight, 2.34 with a warp per tile.  Four while the tiles are
 // few and a tile's own time counts: 50 us at 20k against 78 with two and 194 with
 // a warp per tile; 158 and 162 us at 131k.
