@@ -571,8 +571,9 @@ lp_status lp_graph_launch(lp_ctx *ctx, lp_stream stream);
  *                     the one-sided fits, estimator and blend over that list.
  *   neighbour query:
  *     (default)            one block per 32 key-ordered particles (tiles), with
- *                          a block per particle for those a tile leaves (more
- *                          than 64 neighbours, scattered groups).
+ *                          a block, or where they are many a warp, per particle
+ *                          for those a tile leaves (more than 64 neighbours,
+ *                          scattered groups).
  *     LP_SCHED_QUERY_WARP  one warp per particle for every particle.
  *   work distribution (same results):
  *     LP_SCHED_QUEUE_QUERY the tile kernel runs as a grid of resident blocks

@@ -4,7 +4,8 @@
 // a list does not depend on the order in which its entries were found.)
 //
 // A block per 32 key-ordered particles (tiles), a block per particle for those
-// the tiles leave, and a warp per particle as a schedule of its own.  A particle
+// the tiles leave (a warp where they are many), and a warp per particle as a
+// schedule of its own.  A particle
 // or group queries the finest cell level whose edge is at least half its radius;
 // the cells' key-sorted ranges come from the dense per-level tables, so candidates
 // of a cell are contiguous and read coalesced.  Distances are first taken in FP32 from
